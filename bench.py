@@ -63,6 +63,7 @@ def algorithmic_bytes(name, nC, nE, nV, L, T, prec):
         "k_mass_col": EL * sM + CL * 8 + 2 * nC * 8 + nC * 8 + CL * sA + CI * 8,
         "k_theta_flux": EL * sM + CL * sA + EL * sA,
         "k_theta_update": EL * sA + CL * sA + CI * 8 + 2 * CL * 8,
+        "k_exner_table": 256 * L * 16,
         "k_hydro_diag": nC * 8 + CL * 8 + 3 * CL * 8,
         "k_vort": EL * sU + nC * 8 + VL * sA,
         "k_ke": EL * sU + CL * 8,

@@ -37,6 +37,7 @@ struct DyPar {
     const double *rdB;    // [L]   1/dB
     const double *hrdBi;  // [L+1] 1/(dB[j-1] + dB[j]) at interior interfaces j (half the reciprocal mean)
     const double *dBi;    // [L+1] (dB[j-1] + dB[j])/2 at interior interfaces j
+    const double *Bm;     // [L]   (B[k] + B[k+1])/2, mid-layer coordinate
     const float *dBf;     // [L]   dB rounded to single precision
     const double *phis;   // [nC]  surface geopotential
     uint32_t emu;         // GRIST_ROW_* rows rounded to binary32 (precision search)
@@ -389,28 +390,74 @@ __global__ void k_theta_update(DevMesh m, DyPar d, LevelDiv Dh, const typename P
     }
 }
 
+// Reference states of the hydrostatic equation of state.  pow() costs about
+// 100 FP64 instructions, which bounded k_hydro_diag (pipe 90 % active); but
+// Rd (p/p0)^kappa / p at level k depends on the column's mass
+// dps = ps - pi_top alone, p = pi_top + Bm_k dps, so a table of reference
+// columns turns it into a short series: with the reference at the middle
+// dps_c of the bin that dps falls in,
+//   Rd (p/p0)^kappa / p = [Rd (p_c/p0)^kappa / p_c] (1 + x)^(kappa - 1),
+//   x = Bm_k (dps - dps_c) / p_c,   |x| <= 2^-8 since Bm_k dps_c <= p_c,
+// summed by the 8-term series of pow1p_near0 (tail below 2^-58).  A bin is one
+// value of the exponent and the first 7 fraction bits of dps; the table
+// covers the two octaves that end at twice the one of p0 - pi_top (32.8 to
+// 131 kPa for p0 = 1e5), other columns call pow().  Entry [bin][k] = {the
+// bracket, Bm_k / p_c}: 256 x L x 16 bytes, of which a run touches the bins
+// its surface pressures span (a few tens of kB).
+constexpr int kExnerBins = 256;
+struct Exner {
+    const double2 *tab;
+    int base;   // (high word of dps) >> 13 of bin 0
+};
+__device__ __forceinline__ double exner_centre(int base, int bin) {
+    return __hiloint2double(((base + bin) << 13) | (1 << 12), 0);
+}
+
+__global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= kExnerBins * d.L) return;
+    const int bin = n / d.L, k = n - bin * d.L;
+    const double bm = d.Bm[k];
+    const double pc = d.pi_top + bm * exner_centre(base, bin);
+    tab[n] = make_double2(d.rd * pow(pc / d.p0, d.kappa) / pc, bm / pc);
+}
+
 // Eq. 8 (hydrostatic diagnostics), one warp per column: mid-layer pressure,
 // alpha = Rd theta (p/p0)^kappa / p, geopotential integrated upward from
 // phi_s by a suffix scan, layer geopotential = mean of its interfaces.
+// Bound by the FP64 pipe: about 27 instructions a cell-level with the table
+// above against about 130 with pow(); level-6 mesh, 30 levels:
+// 323 -> 76 us a launch, plus 10 us a step for the table.
 template <bool EMU, bool DF>
-__global__ void k_hydro_diag(DevMesh m, DyPar d, const double *__restrict__ ps, const double *__restrict__ th,
-                             double *__restrict__ p, double *__restrict__ al, double *__restrict__ phl) {
+__global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const double *__restrict__ ps,
+                             const double *__restrict__ th, double *__restrict__ p, double *__restrict__ al,
+                             double *__restrict__ phl) {
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= m.nC) return;
     const double dps = ps[i] - d.pi_top;
-    const double rdps = rcp(dps);
+    const double rdps = rcp_nr(dps);
     const int nch = (d.L + 31) >> 5;
+    const int bin = (__double2hiint(dps) >> 13) - ex.base;
+    const bool tabled = bin >= 0 && bin < kExnerBins;   // the same for the whole warp
+    const double off = dps - exner_centre(ex.base, bin);
+    const double2 *row = ex.tab + (size_t)(tabled ? bin : 0) * d.L;
     double carry = ldg(d.phis + i);
     for (int ch = nch - 1; ch >= 0; ch--) {
         const int k = ch * 32 + lane;
         double contrib = 0.0, a = 0.0, pk = 0.0;
         if (k < d.L) {
-            const double pt = d.pi_top + ldg(d.B + k) * dps, pb = d.pi_top + ldg(d.B + k + 1) * dps;
-            const double dp = pb - pt;
-            pk = 0.5 * (pt + pb);
-            a = d.rd * (th[(size_t)i * d.ld + k] * ldg(d.rdB + k) * rdps) * pow(pk / d.p0, d.kappa) / pk;
-            contrib = a * dp;
+            const double thk = th[(size_t)i * d.ld + k];
+            pk = fma(ldg(d.Bm + k), dps, d.pi_top);
+            double e;
+            if (tabled) {
+                const double2 r = ldg(row + k);
+                e = r.x * horner<8>(r.y * off, bk);
+            } else {
+                e = d.rd * pow(pk / d.p0, d.kappa) / pk;
+            }
+            contrib = thk * e;                        // alpha dpi
+            a = contrib * (ldg(d.rdB + k) * rdps);
         }
         // inclusive suffix sum within the chunk
         double v = contrib;
@@ -423,7 +470,7 @@ __global__ void k_hydro_diag(DevMesh m, DyPar d, const double *__restrict__ ps, 
             const size_t x = (size_t)i * d.ld + k;
             p[x] = emu<EMU>(pk, d.emu, GRIST_ROW_EOS);
             al[x] = emu<EMU>(a, d.emu, GRIST_ROW_EOS);
-            const double ph = carry + (v - contrib) + 0.5 * contrib;
+            const double ph = carry + fma(-0.5, contrib, v);
             phl[x] = DF ? pack_split(ph) : emu<EMU>(ph, d.emu, GRIST_ROW_EOS);
         }
         carry += __shfl_sync(0xffffffffu, v, 0);
@@ -942,7 +989,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += al(bytes); return o; };
-    const size_t nvg = 5 * (size_t)L + 3 + ((size_t)L + 1) / 2;   // doubles, then L floats
+    const size_t nvg = 6 * (size_t)L + 3 + ((size_t)L + 1) / 2;   // doubles, then L floats
     const size_t o_vg = take(sizeof(double) * nvg);
     const size_t o_uA = take(nEL * sizeof(TU)), o_uB = take(nEL * sizeof(TU));
     const size_t o_psA = take(m.nC * 8), o_psB = take(m.nC * 8), o_psN = take(m.nC * 8);
@@ -954,6 +1001,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const size_t o_p = take(nCL * 8), o_al = take(nCL * 8), o_phl = take(nCL * 8), o_dpp = take(nCL * 8);
     const size_t o_qv = take(nVL * sizeof(TA)), o_K = take(nCL * 8);
     size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0;
+    const size_t o_ex = take(NH ? 0 : (size_t)kExnerBins * L * sizeof(double2));
     if (NH) {
         o_wA = take(nCI * 8); o_wB = take(nCI * 8); o_phA = take(nCI * 8); o_phB = take(nCI * 8);
         o_wst = take(nCI * 8); o_phst = take(nCI * 8); o_pn = take(nCL * 8); o_fw = take(nCI * 8);
@@ -962,7 +1010,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     char *s = (char *)scratch(h, 1, off);
     if (!s) return GRIST_ENOMEM;
 
-    // vertical grid: B (L+1) | dB (L) | 1/dB (L) | 1/(dB[j-1]+dB[j]) (L+1) | (dB[j-1]+dB[j])/2 (L+1)
+    // vertical grid: B (L+1) | dB (L) | 1/dB (L) | 1/(dB[j-1]+dB[j]) (L+1) | (dB[j-1]+dB[j])/2 (L+1) |
+    // (B[k]+B[k+1])/2 (L) | dB in binary32 (L floats)
     std::vector<double> vg(nvg, 0.0);
     double *hB = vg.data(), *hdB = hB + L + 1, *hrdB = hdB + L, *hhrdBi = hrdB + L, *hdBi = hhrdBi + L + 1;
     for (int k = 0; k <= L; k++) hB[k] = prm->b_interface[k];
@@ -974,7 +1023,9 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
         hhrdBi[j] = 1.0 / (hdB[j - 1] + hdB[j]);
         hdBi[j] = 0.5 * (hdB[j - 1] + hdB[j]);
     }
-    float *hdBf = reinterpret_cast<float *>(hdBi + L + 1);
+    double *hBm = hdBi + L + 1;
+    for (int k = 0; k < L; k++) hBm[k] = 0.5 * (hB[k] + hB[k + 1]);
+    float *hdBf = reinterpret_cast<float *>(hBm + L);
     for (int k = 0; k < L; k++) hdBf[k] = (float)hdB[k];
     double *dvg = (double *)(s + o_vg);
     if (vg_ptr(h) != dvg || vg_cache(h) != vg) {
@@ -991,7 +1042,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     d.beta = prm->offcentre_beta; d.kappa = prm->rd / prm->cp; d.gamma = prm->cp / (prm->cp - prm->rd);
     d.B = dvg; d.dB = dvg + L + 1; d.rdB = dvg + 2 * L + 1; d.hrdBi = dvg + 3 * L + 1; d.dBi = dvg + 4 * L + 2;
     d.phis = prm->phi_surface;
-    d.dBf = reinterpret_cast<const float *>(dvg + 5 * L + 3);
+    d.Bm = dvg + 5 * L + 3;
+    d.dBf = reinterpret_cast<const float *>(dvg + 6 * L + 3);
     d.emu = prm->emulate_fp32_rows;
 
     TU *uA = (TU *)(s + o_uA), *uB = (TU *)(s + o_uB);
@@ -1034,7 +1086,20 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             p_n = dst;
         }
     }
-    const Binom bpos = binomial(d.gamma), bneg = binomial(-d.gamma);
+    const Binom bpos = binomial(d.gamma), bneg = binomial(-d.gamma), bkap = binomial(d.kappa - 1.0);
+    Exner ex{(double2 *)(s + o_ex), 0};
+    if (!NH) {
+        // two octaves up to twice the power of two at or below p0 - pi_top;
+        // bins that no column can fall in where the series' exponent would be
+        // out of its range (kappa - 1 outside (-1, 0)).  Made in every step
+        // (about 10 us): a step recorded in a graph then carries its own
+        int e2 = 0;
+        const double span = prm->p0 - prm->pi_top;
+        if (std::isfinite(span)) std::frexp(span, &e2);   // |span| in [2^(e2-1), 2^e2)
+        ex.base = d.kappa > 0.0 && d.kappa < 1.0 && e2 > -1000 ? (1023 + e2 - 2) << 7 : 1 << 20;
+        GRIST_LAUNCH(h, PN("k_exner_table"), st, k_exner_table<<<grid_for((long long)kExnerBins * L, 32), 32, 0, st>>>(
+            d, ex.base, (double2 *)(s + o_ex)));
+    }
 
     double *p_outs[3] = {p, p, (NH && S->p_nh) ? S->p_nh : p};
 
@@ -1067,7 +1132,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                 phi_outs[s3], p_outs[s3], alp, phl, dpp, bpos, bneg));
         } else {
             GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF><<<gW, kBlock, 0, st>>>(
-                m, d, ps_outs[s3], th_outs[s3], p, alp, phl));
+                m, d, ex, bkap, ps_outs[s3], th_outs[s3], p, alp, phl));
         }
         GRIST_LAUNCH(h, PN("k_vertex_mass"), st, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, st>>>(m, d, ps_in, rdpv));
         GRIST_LAUNCH(h, PN("k_vort"), st, k_vort<P><<<gVH, kBlock, 0, st>>>(m, d, DH, u_in, rdpv, qv));
