@@ -79,6 +79,8 @@ def algorithmic_bytes(name, nC, nE, nV, L, T, prec):
         "k_tr_div": EL * 8 + CL * 8 + 2 * CL * sC + (EL * 4 if sC == 4 else 0),
         "k_tr_edge": T * CL * sQ + EL * sC + T * EL * sC,
         "k_tr_update": T * EL * sC + T * CL * sQ + 2 * CL * sC + T * CL * sQ,
+        # with the low-order phase: + {dpi, div F}, local bounds, div F^L
+        "k_tr_edge_low": T * CL * sQ + EL * sC + T * EL * sC + 2 * CL * sC + 3 * T * CL * sC,
         # limiter: q^n, F, {dpi, div F} -> local bounds {max, min}(q^n, q^td), div F^L
         "k_tr_lowres": T * CL * sQ + EL * sC + 2 * CL * sC + 2 * T * CL * sC + T * CL * sC,
         # q^n, bounds, A, {dpi, div F} -> {R+, R-}

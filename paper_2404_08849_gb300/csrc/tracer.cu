@@ -18,6 +18,16 @@
 // Data layout: q [T][nC][ld], dpi [nC][ld], mass flux [nE][ld], edge
 // fluxes [T][nE][ld]; consecutive threads take consecutive levels of one
 // entity (coalesced rows), neighbour rows are gathered through L1/L2.
+//
+// A work item is a vector of 4 or 2 binary32 or 2 binary64 levels where the
+// member's rows allow it (vec_class): with one level per 4-byte access the
+// L1 data pipe (79 % of its wavefronts) and the latency of many small gathers
+// bounded the binary32 phases.  Level-7 mesh, 4 tracers, 60 levels, binary32,
+// us per launch, one level / vectors: div 231 / 145, edge 365 / 231, update
+// 226 / 140 (then at the DRAM rate), ratios 545 / 335 (half of it the
+// division's slow path, see fct_ratio), final 440 / 307, low-order 270 / 128
+// more in the first edge phase; the step 3261 / 2110.  binary64 is bound by
+// the FP64 pipe and gains little from the width.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -44,7 +54,7 @@ struct MemberDev {
     const double *Mv;       // time-mean vertical mass flux [nC][ldi] or null (no vertical step)
     int ldi;
     LevelDiv DL;            // division by Lg
-    int Lg;                 // level groups: a thread takes levels g, g + Lg, ... (levels_per_thread of them)
+    int Lg;                 // level groups of a thread: V consecutive levels from g V, or levels g, g + Lg, ...
     unsigned long long qs, fs;  // nC*ld, nE*ld
 };
 
@@ -132,11 +142,15 @@ constexpr int kVertMaxL = 128;   // levels supported by the vertical transport
 // Largest block of the work-list kernels (their register use, at most 128
 // per thread, lets every block up to this size launch).
 constexpr int kTracerMaxBlock = 512;
+// Widths of a work item's level vector: 1, 2 or 4 consecutive levels.
+constexpr int kVecClasses = 3;
 
 struct Batch {
     const MemberDev *mem;
     int nm;
-    Space D, C, E;  // D: cell x level (no groups); C: cell x level x group; E: edge x level x group
+    // D: cell x level (no groups); C: cell x level x group; E: edge x level x
+    // group; each by the members' vector width (class c: 2^c levels)
+    Space D[kVecClasses], C[kVecClasses], E[kVecClasses];
     Space T;        // blocks of the fused stage kernel: segment start = first block of (member, group)
     int tpt;
     int lpt;        // levels per thread of the work-list phases (1 or 2; the persistent launch takes 1)
@@ -201,9 +215,72 @@ __device__ __forceinline__ void stage_ratios(float2 dv, double, float dtsf, floa
 __device__ __forceinline__ double end_mass(double2 dv, double dt, float) { return dv.x - dt * dv.y; }
 __device__ __forceinline__ float end_mass(float2 dv, double, float dtf) { return fmaf(-dtf, dv.y, dv.x); }
 
-template <bool PERS, typename TC>
-__device__ __forceinline__ typename Vec2<TC>::T dv_at(const MemberDev &mb, size_t x) {
-    return lds<PERS>((const typename Vec2<TC>::T *)mb.DV + x);
+// Vectors of V consecutive levels (V * sizeof(T) up to 32 bytes), moved as 8-
+// or 16-byte accesses; plan_batch gives a member only a V that its rows and
+// pointers are aligned to.  PERS as in lds().
+template <bool PERS, int V, typename T> __device__ __forceinline__ void ldv(const T *p, T (&o)[V]) {
+    if constexpr (V == 1) {
+        o[0] = lds<PERS>(p);
+    } else if constexpr (sizeof(T) * V == 8) {
+        const float2 a = lds<PERS>((const float2 *)p);
+        o[0] = a.x; o[1] = a.y;
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4) {
+            const float4 a = lds<PERS>((const float4 *)(p + j));
+            o[j] = a.x; o[j + 1] = a.y; o[j + 2] = a.z; o[j + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) {
+            const double2 a = lds<PERS>((const double2 *)(p + j));
+            o[j] = a.x; o[j + 1] = a.y;
+        }
+    }
+}
+template <int V, typename T> __device__ __forceinline__ void stv(T *p, const T (&o)[V]) {
+    if constexpr (V == 1) {
+        *p = o[0];
+    } else if constexpr (sizeof(T) * V == 8) {
+        *(float2 *)p = make_float2(o[0], o[1]);
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4) *(float4 *)(p + j) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) *(double2 *)(p + j) = make_double2(o[j], o[j + 1]);
+    }
+}
+// The caller's q^n where the same launch overwrites it in place (each thread
+// its own levels): an ordinary load.
+template <int V, typename T> __device__ __forceinline__ void ldv_own(const T *p, T (&o)[V]) {
+    if constexpr (V == 1) {
+        o[0] = *p;
+    } else if constexpr (sizeof(T) * V == 8) {
+        const float2 a = *(const float2 *)p;
+        o[0] = a.x; o[1] = a.y;
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4) {
+            const float4 a = *(const float4 *)(p + j);
+            o[j] = a.x; o[j + 1] = a.y; o[j + 2] = a.z; o[j + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) {
+            const double2 a = *(const double2 *)(p + j);
+            o[j] = a.x; o[j + 1] = a.y;
+        }
+    }
+}
+
+// The {dpi, div F} pairs of V levels: d[2 v], d[2 v + 1].
+template <bool PERS, typename TC, int V>
+__device__ __forceinline__ void dv_at(const MemberDev &mb, size_t x, typename Vec2<TC>::T (&o)[V]) {
+    TC d[2 * V];
+    ldv<PERS, 2 * V>((const TC *)mb.DV + 2 * x, d);
+#pragma unroll
+    for (int v = 0; v < V; v++) o[v] = typename Vec2<TC>::T{d[2 * v], d[2 * v + 1]};
 }
 
 // A cell's edges, neighbours and divergence weights, read once per work
@@ -226,154 +303,202 @@ __device__ __forceinline__ void load_cell_row(const DevMesh &m, int i, CellRow<T
 // edge's flux is also rounded once to binary32 for the later phases (by the
 // cell it leaves: positive divergence coefficient), so they read 4 bytes
 // per edge-level instead of 8.
-template <typename TC>
+template <typename TC, int V>
 __device__ __forceinline__ void item_div(const MemberDev &mb, const CellRow<double> &r, int i, int k) {
-    double s = 0.0;
+    double s[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) s[v] = 0.0;
 #pragma unroll
     for (int j = 0; j < GRIST_MAXE; j++) {
-        const int e = r.e[j];
+        const size_t y = (size_t)r.e[j] * mb.ld + k;
         const double cw = r.cw[j];
-        const double f = ldg(mb.F + (size_t)e * mb.ld + k);
-        s += cw * f;
-        if (sizeof(TC) == 4 && cw > 0.0) ((float *)mb.Ff)[(size_t)e * mb.ld + k] = cv<float>(f);
+        double f[V];
+        ldv<false, V>(mb.F + y, f);
+#pragma unroll
+        for (int v = 0; v < V; v++) s[v] += cw * f[v];
+        if constexpr (sizeof(TC) == 4) {
+            if (cw > 0.0) {
+                float g[V];
+#pragma unroll
+                for (int v = 0; v < V; v++) g[v] = cv<float>(f[v]);
+                stv<V>((float *)mb.Ff + y, g);
+            }
+        }
     }
     const size_t x = (size_t)i * mb.ld + k;
-    if (sizeof(TC) == 4) ((float2 *)mb.DV)[x] = make_float2(cv<float>(ldg(mb.dpi + x)), cv<float>(s));
-    else ((double2 *)mb.DV)[x] = make_double2(ldg(mb.dpi + x), s);
+    double dp[V];
+    ldv<false, V>(mb.dpi + x, dp);
+    TC d[2 * V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        d[2 * v] = cv<TC>(dp[v]);
+        d[2 * v + 1] = cv<TC>(s[v]);
+    }
+    stv<2 * V>((TC *)mb.DV + 2 * x, d);
 }
 
-// Mass flux of edge-level x in the compute type: the binary32 copy made by
-// the continuity phase (read coherently inside the persistent launch, which
-// wrote it), or the caller's FP64 array.
-template <bool PERS, typename TC>
-__device__ __forceinline__ TC flux_at(const MemberDev &mb, size_t x) {
-    if (sizeof(TC) == 4) return (TC)lds<PERS>((const float *)mb.Ff + x);
-    return (TC)ldg(mb.F + x);
+// Mass flux of V levels from edge-level x in the compute type: the binary32
+// copy made by the continuity phase (read coherently inside the persistent
+// launch, which wrote it), or the caller's FP64 array.
+template <bool PERS, int V, typename TC>
+__device__ __forceinline__ void flux_at(const MemberDev &mb, size_t x, TC (&f)[V]) {
+    if constexpr (sizeof(TC) == 4) ldv<PERS, V>((const float *)mb.Ff + x, f);
+    else ldv<false, V>(mb.F + x, f);
 }
 
 // Products and sums of the limiter written with explicit rounding, so the
 // edge-centric and cell-centric forms (different kernels) give the same
-// bits: F^L = F q^n_upwind, A = F^H - F^L with F^H = F q_e, div F^L summed
-// by fused multiply-adds in edge order, q^td = r1 q^n - r2 div F^L.
+// bits: F^L = F q^n_upwind, A = F^H - F^L = F (q_e - q^n_upwind), div F^L
+// summed by fused multiply-adds in edge order, q^td = r1 q^n - r2 div F^L.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-template <typename TC> __device__ __forceinline__ TC antidiff(TC f, TC qe, TC qup) {
-    return mul_rn(f, qe) - mul_rn(f, qup);
-}
+template <typename TC> __device__ __forceinline__ TC antidiff(TC f, TC qe, TC qup) { return mul_rn(f, sub_rn(qe, qup)); }
 template <typename TC> __device__ __forceinline__ TC lowres_value(TC r1, TC r2, TC qn, TC divl) {
     return fma_rn(r1, qn, -mul_rn(r2, divl));
 }
 
 // Third-order upwind edge flux (Skamarock-Gassmann form):
 //   q_e = (q1 + q2)/2 - (dc^2/12)(q''1 + q''2) + sgn(F) beta (dc^2/12)(q''2 - q''1)
-// F^H = F q_e.  With beta = 1 only the upwind side's second derivative
-// survives: q_e = (q1 + q2)/2 - 2 (dc^2/12) q''_upwind.
+// F^H = F q_e, on V levels of one edge.  With beta = 1 only the upwind side's
+// second derivative survives: q_e = (q1 + q2)/2 - 2 (dc^2/12) q''_upwind
+// (V = 1 here: the levels of a vector may have different upwind sides).
 // In the final stage of a limited step (qn = q^n) the phase stores the
 // antidiffusive flux A = F^H - F^L instead of F^H.
-template <bool PERS, typename TQ, typename TC>
+template <bool PERS, typename TQ, typename TC, int V>
 __device__ __forceinline__ void item_edge(const DevMesh &m, const MemberDev &mb, const TQ *q, const TQ *qn, int t0,
                                           int t1, int e, int k, bool beta1, TC beta) {
     const int ld = mb.ld;
     const int2 c = ldg(m.coe + e);
-    const TC f = flux_at<PERS, TC>(mb, (size_t)e * ld + k);
+    TC f[V];
+    flux_at<PERS, V>(mb, (size_t)e * ld + k, f);
     const TC dc2 = ldg(Coef<TC>::dc2(m) + e);
     const int32_t *st = m.d2i + (size_t)e * 14;
     const TC *cf = Coef<TC>::d2c(m) + (size_t)e * 14;
     TC *FH = (TC *)mb.FH;
-    if (beta1 && m.d2w_ok) {
-        // one weighted sum over the upwind side's stencil (the mean of c1 and
-        // c2 folded into the weights)
-        const int side = f >= (TC)0 ? 0 : 1;
-        int idx[GRIST_D2P];
-        TC w[GRIST_D2P];
-        load_d2w(m, e, side, idx, w);
-        for (int t = t0; t < t1; t++) {
-            const TQ *qt = q + (size_t)t * mb.qs;
-            TC v = 0;
-#pragma unroll
-            for (int j = 0; j < GRIST_D2P; j++) v += w[j] * static_cast<TC>(lds<PERS>(qt + (size_t)idx[j] * ld + k));
-            FH[(size_t)t * mb.fs + (size_t)e * ld + k] =
-                qn ? antidiff(f, v, static_cast<TC>(qn[(size_t)t * mb.qs + (size_t)idx[0] * ld + k])) : f * v;
-        }
-    } else if (beta1) {
-        const int side = f >= (TC)0 ? 0 : 1;
-        int idx[GRIST_D2P];
-        TC w[GRIST_D2P];
-#pragma unroll
-        for (int j = 0; j < GRIST_D2P; j++) {
-            idx[j] = ldg(st + side * GRIST_D2P + j);
-            w[j] = ldg(cf + side * GRIST_D2P + j);
-        }
-        for (int t = t0; t < t1; t++) {
-            const TQ *qt = q + (size_t)t * mb.qs;
+    for (int t = t0; t < t1; t++) {
+        const TQ *qt = q + (size_t)t * mb.qs + k;
+        TC q1[V], q2[V], qe[V], a[V], b[V];
+        ldv<PERS, V>(qt + (size_t)c.x * ld, q1);
+        ldv<PERS, V>(qt + (size_t)c.y * ld, q2);
+        if (V == 1 && beta1) {
+            const int side = f[0] >= (TC)0 ? 0 : 1;
             TC d = 0;
 #pragma unroll
-            for (int j = 0; j < GRIST_D2P; j++) d += w[j] * static_cast<TC>(lds<PERS>(qt + (size_t)idx[j] * ld + k));
-            const TC q1 = static_cast<TC>(lds<PERS>(qt + (size_t)c.x * ld + k)), q2 = static_cast<TC>(lds<PERS>(qt + (size_t)c.y * ld + k));
-            const TC qe = (TC)0.5 * (q1 + q2) - (TC)2 * dc2 * d;
-            FH[(size_t)t * mb.fs + (size_t)e * ld + k] =
-                qn ? antidiff(f, qe, static_cast<TC>(qn[(size_t)t * mb.qs + (size_t)(f >= (TC)0 ? c.x : c.y) * ld + k]))
-                   : f * qe;
-        }
-    } else {
-        const TC sgn = f >= (TC)0 ? (TC)1 : (TC)-1;
-        for (int t = t0; t < t1; t++) {
-            const TQ *qt = q + (size_t)t * mb.qs;
-            TC d1 = 0, d2 = 0;
+            for (int j = 0; j < GRIST_D2P; j++) {
+                ldv<PERS, V>(qt + (size_t)ldg(st + side * GRIST_D2P + j) * ld, a);
+                d += ldg(cf + side * GRIST_D2P + j) * a[0];
+            }
+            qe[0] = (TC)0.5 * (q1[0] + q2[0]) - (TC)2 * dc2 * d;
+        } else {
+            TC d1[V], d2[V];
+#pragma unroll
+            for (int v = 0; v < V; v++) d1[v] = d2[v] = 0;
 #pragma unroll
             for (int j = 0; j < GRIST_D2P; j++) {
-                d1 += ldg(cf + j) * static_cast<TC>(lds<PERS>(qt + (size_t)ldg(st + j) * ld + k));
-                d2 += ldg(cf + GRIST_D2P + j) * static_cast<TC>(lds<PERS>(qt + (size_t)ldg(st + GRIST_D2P + j) * ld + k));
+                ldv<PERS, V>(qt + (size_t)ldg(st + j) * ld, a);
+                ldv<PERS, V>(qt + (size_t)ldg(st + GRIST_D2P + j) * ld, b);
+                const TC w1 = ldg(cf + j), w2 = ldg(cf + GRIST_D2P + j);
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    d1[v] += w1 * a[v];
+                    d2[v] += w2 * b[v];
+                }
             }
-            const TC q1 = static_cast<TC>(lds<PERS>(qt + (size_t)c.x * ld + k)), q2 = static_cast<TC>(lds<PERS>(qt + (size_t)c.y * ld + k));
-            const TC qe = (TC)0.5 * (q1 + q2) - dc2 * (d1 + d2) + sgn * beta * dc2 * (d2 - d1);
-            FH[(size_t)t * mb.fs + (size_t)e * ld + k] =
-                qn ? antidiff(f, qe, static_cast<TC>(qn[(size_t)t * mb.qs + (size_t)(f >= (TC)0 ? c.x : c.y) * ld + k]))
-                   : f * qe;
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                const TC sgn = f[v] >= (TC)0 ? (TC)1 : (TC)-1;
+                qe[v] = (TC)0.5 * (q1[v] + q2[v]) - dc2 * (d1[v] + d2[v]) + sgn * beta * dc2 * (d2[v] - d1[v]);
+            }
         }
+        if (qn) {
+            ldv<PERS, V>(qn + (size_t)t * mb.qs + (size_t)c.x * ld + k, a);
+            ldv<PERS, V>(qn + (size_t)t * mb.qs + (size_t)c.y * ld + k, b);
+        }
+#pragma unroll
+        for (int v = 0; v < V; v++) qe[v] = qn ? antidiff(f[v], qe[v], f[v] >= (TC)0 ? a[v] : b[v]) : f[v] * qe[v];
+        stv<V>(FH + (size_t)t * mb.fs + (size_t)e * ld + k, qe);
     }
 }
 
-// The edge item over a thread's LPT levels kg, kg + Lg, ...  With the
+// The combined-weight edge flux (beta = 1) of one edge on V levels whose
+// fluxes all run to the side whose stencil row (idx, w) is given.
+template <bool PERS, typename TQ, typename TC, int V>
+__device__ __forceinline__ void edge_combined(const MemberDev &mb, const TQ *q, const TQ *qn, int t0, int t1, int e,
+                                              int k, const TC (&f)[V], const int (&idx)[GRIST_D2P],
+                                              const TC (&w)[GRIST_D2P]) {
+    const int ld = mb.ld;
+    TC *FH = (TC *)mb.FH;
+    for (int t = t0; t < t1; t++) {
+        const TQ *qt = q + (size_t)t * mb.qs + k;
+        TC s[V], a[V];
+#pragma unroll
+        for (int v = 0; v < V; v++) s[v] = 0;
+#pragma unroll
+        for (int j = 0; j < GRIST_D2P; j++) {
+            ldv<PERS, V>(qt + (size_t)idx[j] * ld, a);
+#pragma unroll
+            for (int v = 0; v < V; v++) s[v] += w[j] * a[v];
+        }
+        if (qn) ldv<PERS, V>(qn + (size_t)t * mb.qs + (size_t)idx[0] * ld + k, a);
+#pragma unroll
+        for (int v = 0; v < V; v++) s[v] = qn ? antidiff(f[v], s[v], a[v]) : f[v] * s[v];
+        stv<V>(FH + (size_t)t * mb.fs + (size_t)e * ld + k, s);
+    }
+}
+
+// The edge item over a thread's levels (edge-centric form).  With the
 // combined weights, the upwind side's stencil (4 vector loads) is read once
-// and read again only for a level whose flux runs the other way.
-template <bool PERS, typename TQ, typename TC, int LPT>
+// and read again only for a level whose flux runs the other way; a vector
+// whose levels disagree on the side takes them one by one.
+template <bool PERS, typename TQ, typename TC, int LPT, int V>
 __device__ __forceinline__ void item_edge_levels(const DevMesh &m, const MemberDev &mb, const TQ *q, const TQ *qn,
                                                  int t0, int t1, int e, int kg, bool beta1, TC beta) {
     if (!(beta1 && m.d2w_ok)) {
-#pragma unroll
-        for (int u = 0; u < LPT; u++) {
-            const int k = kg + u * mb.Lg;
+        if (V > 1 && !beta1) {
+            item_edge<PERS, TQ, TC, V>(m, mb, q, qn, t0, t1, e, kg * V, beta1, beta);
+            return;
+        }
+#pragma unroll 1
+        for (int u = 0; u < LPT * V; u++) {
+            const int k = V > 1 ? kg * V + u : kg + u * mb.Lg;
             if (LPT > 1 && k >= mb.L) break;
-            item_edge<PERS, TQ, TC>(m, mb, q, qn, t0, t1, e, k, beta1, beta);
+            item_edge<PERS, TQ, TC, 1>(m, mb, q, qn, t0, t1, e, k, beta1, beta);
         }
         return;
     }
-    const int ld = mb.ld;
-    TC *FH = (TC *)mb.FH;
+    const size_t row = (size_t)e * mb.ld;
     int idx[GRIST_D2P];
     TC w[GRIST_D2P];
-    int loaded = -1;
+    if constexpr (V > 1) {
+        TC f[V];
+        flux_at<PERS, V>(mb, row + kg * V, f);
+        const int side = f[0] >= (TC)0 ? 0 : 1;
+        bool same = true;
 #pragma unroll
-    for (int u = 0; u < LPT; u++) {
-        const int k = kg + u * mb.Lg;
+        for (int v = 1; v < V; v++) same &= (f[v] >= (TC)0 ? 0 : 1) == side;
+        if (same) {
+            load_d2w(m, e, side, idx, w);
+            edge_combined<PERS, TQ, TC, V>(mb, q, qn, t0, t1, e, kg * V, f, idx, w);
+            return;
+        }
+    }
+    int loaded = -1;
+#pragma unroll(V > 1 ? 1 : LPT)
+    for (int u = 0; u < LPT * V; u++) {
+        const int k = V > 1 ? kg * V + u : kg + u * mb.Lg;
         if (LPT > 1 && k >= mb.L) break;
-        const TC f = flux_at<PERS, TC>(mb, (size_t)e * ld + k);
-        const int side = f >= (TC)0 ? 0 : 1;
+        TC f[1];
+        flux_at<PERS, 1>(mb, row + k, f);
+        const int side = f[0] >= (TC)0 ? 0 : 1;
         if (side != loaded) {
             load_d2w(m, e, side, idx, w);
             loaded = side;
         }
-        for (int t = t0; t < t1; t++) {
-            const TQ *qt = q + (size_t)t * mb.qs;
-            TC v = 0;
-#pragma unroll
-            for (int j = 0; j < GRIST_D2P; j++) v += w[j] * static_cast<TC>(lds<PERS>(qt + (size_t)idx[j] * ld + k));
-            FH[(size_t)t * mb.fs + (size_t)e * ld + k] =
-                qn ? antidiff(f, v, static_cast<TC>(qn[(size_t)t * mb.qs + (size_t)idx[0] * ld + k])) : f * v;
-        }
+        edge_combined<PERS, TQ, TC, 1>(mb, q, qn, t0, t1, e, k, f, idx, w);
     }
 }
 
@@ -384,55 +509,147 @@ __device__ __forceinline__ void item_edge_levels(const DevMesh &m, const MemberD
 // written once, by its upwind cell, with the weights and the summation
 // order of the edge-centric form (bit-identical), from 7 gathers per
 // cell-level instead of 7 per edge-level.  The ring values of up to
-// kRingT tracers are gathered first, so each drained edge's weights are
-// read once for them; the cell's divergence signs are kept as two masks
-// (real edge; i is c1).  In the final stage of a limited step (qn = q^n)
-// the phase stores A = F^H - F^L, F^L = F q^n_i.
-#ifndef GRIST_TR_RING_T
-#define GRIST_TR_RING_T 2
-#endif
-constexpr int kRingT = GRIST_TR_RING_T;
-template <bool PERS, typename TQ, typename TC, int LPT>
-__device__ __forceinline__ void item_edge_ring(const DevMesh &m, const MemberDev &mb, const int (&e)[GRIST_MAXE],
-                                               const int (&nb)[GRIST_MAXE], unsigned real, unsigned c1,
-                                               const TQ *q, const TQ *qn, int t0, int t1, int i, int kg) {
+// ring_tracers() tracers are gathered first, so each drained edge's weights
+// are read once for them.  The drained edge-levels are kept as a mask (bit
+// 8 v + j: level v, edge j), and each thread walks its own drained edges: a
+// warp's cells drain different edges, so a walk over all six would spend 4.6
+// passes on the three that each thread has.  An edge whose V levels all
+// drain this cell is stored as one vector.  In the final stage of a limited
+// step (qn = q^n) the phase stores A = F^H - F^L, F^L = F q^n_i.
+// The low-order results of V levels at cell-level y of the tracer arrays: the
+// local bounds {max, min}(q^n, q^td) and div F^L.
+template <typename TC, int V>
+__device__ __forceinline__ void store_lowres(const MemberDev &mb, size_t y, const TC (&r1)[V], const TC (&r2)[V],
+                                             const TC (&qi)[V], const TC (&divl)[V]) {
+    TC b[2 * V];
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        const TC qd = lowres_value(r1[v], r2[v], qi[v], divl[v]);
+        b[2 * v] = fmax_(qi[v], qd);
+        b[2 * v + 1] = fmin_(qi[v], qd);
+    }
+    stv<2 * V>((TC *)mb.X2 + 2 * y, b);
+    stv<V>((TC *)mb.DFL + y, divl);
+}
+
+template <typename TC, int V, bool LOW> constexpr int ring_tracers() {
+    return sizeof(TC) * V <= 8 || (LOW && sizeof(TC) == 4) ? 2 : 1;
+}
+// LOW (the first stage of a limited step, q = q^n): the ring and the fluxes
+// are all that the low-order solution needs, so its phase (item_lowres, the
+// same operations) is done here, without gathering them again.
+template <bool PERS, typename TQ, typename TC, int LPT, int V, bool LOW>
+__device__ __forceinline__ void item_edge_ring(const DevMesh &m, const MemberDev &mb, const TQ *q, const TQ *qn, int t0,
+                                               int t1, int i, int kg, double dt, float dtf) {
+    constexpr int RT = ring_tracers<TC, V, LOW>();
     const int ld = mb.ld;
     TC *FH = (TC *)mb.FH;
+    int nb[GRIST_MAXE];
+    load_row6(m.coc8, i, nb);
 #pragma unroll
     for (int u = 0; u < LPT; u++) {
-        const int k = kg + u * mb.Lg;
+        const int k = (kg + u * mb.Lg) * V;
         if (LPT > 1 && k >= mb.L) break;
-        TC f[GRIST_MAXE];
-        unsigned out = 0;
-#pragma unroll
-        for (int j = 0; j < GRIST_MAXE; j++) {
-            f[j] = flux_at<PERS, TC>(mb, (size_t)e[j] * ld + k);
-            if (((real >> j) & 1u) && ((f[j] >= (TC)0) == (((c1 >> j) & 1u) != 0))) out |= 1u << j;
-        }
-        for (int tb = t0; tb < t1; tb += kRingT) {
-            const int nt = min(kRingT, t1 - tb);
-            TC qr[kRingT][GRIST_D2P], qup[kRingT];
-#pragma unroll
-            for (int a = 0; a < kRingT; a++) {
-                if (a >= nt) break;
-                const TQ *qt = q + (size_t)(tb + a) * mb.qs;
-                qr[a][0] = static_cast<TC>(lds<PERS>(qt + (size_t)i * ld + k));
-#pragma unroll
-                for (int j = 0; j < GRIST_MAXE; j++) qr[a][1 + j] = static_cast<TC>(lds<PERS>(qt + (size_t)nb[j] * ld + k));
-                qup[a] = qn ? static_cast<TC>(qn[(size_t)(tb + a) * mb.qs + (size_t)i * ld + k]) : (TC)0;
-            }
+        unsigned out = 0, c1 = 0;
+        {
+            int e[GRIST_MAXE];
+            TC cw[GRIST_MAXE];
+            load_row6(m.eoc8, i, e);
+            load_row6(Coef<TC>::cdiv8(m), i, cw);
 #pragma unroll
             for (int j = 0; j < GRIST_MAXE; j++) {
-                if (!(out & (1u << j))) continue;
-                TC w[GRIST_D2P];
-                load_d2w_weights(m, e[j], ((c1 >> j) & 1u) ? 0 : 1, w);
+                TC f[V];
+                flux_at<PERS, V>(mb, (size_t)e[j] * ld + k, f);
+                if (cw[j] > (TC)0) c1 |= 1u << j;
+                if (cw[j] != (TC)0) {   // a real edge
 #pragma unroll
-                for (int a = 0; a < kRingT; a++) {
+                    for (int v = 0; v < V; v++)
+                        if ((f[v] >= (TC)0) == (cw[j] > (TC)0)) out |= 1u << (8 * v + j);
+                }
+            }
+        }
+        unsigned any = out;
+        if (V > 2) any |= any >> 16;
+        if (V > 1) any |= any >> 8;
+        any &= 0x3fu;
+        const size_t x = (size_t)i * ld + k;
+        TC r1[V], r2[V];
+        if constexpr (LOW) {
+            typename Vec2<TC>::T dv[V];
+            dv_at<PERS, TC, V>(mb, x, dv);
+#pragma unroll
+            for (int v = 0; v < V; v++) stage_ratios(dv[v], dt, dtf, r1[v], r2[v]);
+        }
+        for (int tb = t0; tb < t1; tb += RT) {
+            const int nt = min(RT, t1 - tb);
+            TC qr[RT][GRIST_D2P][V], qup[RT][V];
+#pragma unroll
+            for (int a = 0; a < RT; a++) {
+                if (a >= nt) break;
+                const TQ *qt = q + (size_t)(tb + a) * mb.qs;
+                ldv<PERS, V>(qt + (size_t)i * ld + k, qr[a][0]);
+#pragma unroll
+                for (int j = 0; j < GRIST_MAXE; j++) ldv<PERS, V>(qt + (size_t)nb[j] * ld + k, qr[a][1 + j]);
+                if (qn) ldv_own<V>(qn + (size_t)(tb + a) * mb.qs + x, qup[a]);
+            }
+            if constexpr (LOW) {
+                TC divl[RT][V];
+#pragma unroll
+                for (int a = 0; a < RT; a++)
+#pragma unroll
+                    for (int v = 0; v < V; v++) divl[a][v] = 0;
+                int e[GRIST_MAXE];
+                TC cw[GRIST_MAXE];
+                load_row6(m.eoc8, i, e);
+                load_row6(Coef<TC>::cdiv8(m), i, cw);
+#pragma unroll
+                for (int j = 0; j < GRIST_MAXE; j++) {
+                    TC f[V];
+                    flux_at<PERS, V>(mb, (size_t)e[j] * ld + k, f);
+#pragma unroll
+                    for (int v = 0; v < V; v++) {
+                        const TC cf = mul_rn(cw[j], f[v]);
+#pragma unroll
+                        for (int a = 0; a < RT; a++)
+                            divl[a][v] = fma_rn(cf, (out >> (8 * v + j)) & 1u ? qr[a][0][v] : qr[a][1 + j][v], divl[a][v]);
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < RT; a++) {
                     if (a >= nt) break;
-                    TC v = 0;
+                    store_lowres<TC, V>(mb, (size_t)(tb + a) * mb.qs + x, r1, r2, qr[a][0], divl[a]);
+                }
+            }
+#pragma unroll 1
+            for (unsigned left = any; left; left &= left - 1) {
+                const int j = __ffs((int)left) - 1;
+                const int e = ldg(m.eoc8 + (size_t)i * 8 + j);
+                TC w[GRIST_D2P], f[V];
+                load_d2w_weights(m, e, ((c1 >> j) & 1u) ? 0 : 1, w);
+                flux_at<PERS, V>(mb, (size_t)e * ld + k, f);
+                const unsigned oj = out >> j;
+                bool all = true;
 #pragma unroll
-                    for (int p = 0; p < GRIST_D2P; p++) v += w[p] * qr[a][p];
-                    FH[(size_t)(tb + a) * mb.fs + (size_t)e[j] * ld + k] = qn ? antidiff(f[j], v, qup[a]) : f[j] * v;
+                for (int v = 0; v < V; v++) all &= ((oj >> (8 * v)) & 1u) != 0;
+#pragma unroll
+                for (int a = 0; a < RT; a++) {
+                    if (a >= nt) break;
+                    TC g[V];
+#pragma unroll
+                    for (int v = 0; v < V; v++) {
+                        TC s = 0;
+#pragma unroll
+                        for (int p = 0; p < GRIST_D2P; p++) s += w[p] * qr[a][p][v];
+                        g[v] = qn ? antidiff(f[v], s, qup[a][v]) : f[v] * s;
+                    }
+                    TC *dst = FH + (size_t)(tb + a) * mb.fs + (size_t)e * ld + k;
+                    if (all) {
+                        stv<V>(dst, g);
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < V; v++)
+                            if ((oj >> (8 * v)) & 1u) dst[v] = g[v];
+                    }
                 }
             }
         }
@@ -443,26 +660,38 @@ __device__ __forceinline__ void item_edge_ring(const DevMesh &m, const MemberDev
 // written as r1 q^n - r2 div with r1 = dpi^n/dpi^(s), r2 = dt_s/dpi^(s)
 // taken once per (cell, level) in FP64 and rounded to the tracer type
 // (Sec. 2.2 (ii): no mixed-kind products inside the tracer loop).
-template <bool PERS, typename TQ, typename TC>
+template <bool PERS, typename TQ, typename TC, int V>
 __device__ __forceinline__ bool item_update(const CellRow<TC> &r, const MemberDev &mb, TQ *qout, int t0, int t1, int i,
                                             int k, double dts, float dtsf) {
     const int ld = mb.ld;
     const size_t x = (size_t)i * ld + k;
-    TC r1, r2;
-    stage_ratios(dv_at<PERS, TC>(mb, x), dts, dtsf, r1, r2);
-    const int *eidx = r.e;
-    const TC *cw = r.cw;
+    typename Vec2<TC>::T dv[V];
+    TC r1[V], r2[V];
+    dv_at<PERS, TC, V>(mb, x, dv);
+#pragma unroll
+    for (int v = 0; v < V; v++) stage_ratios(dv[v], dts, dtsf, r1[v], r2[v]);
     const TQ *qn = (const TQ *)mb.q;
     const TC *FH = (const TC *)mb.FH;
     bool bad = false;
     for (int t = t0; t < t1; t++) {
-        const TC *ft = FH + (size_t)t * mb.fs;
-        TC div = 0;
+        const TC *ft = FH + (size_t)t * mb.fs + k;
+        TC div[V], qv[V];
+        ldv_own<V>(qn + (size_t)t * mb.qs + x, qv);
 #pragma unroll
-        for (int j = 0; j < GRIST_MAXE; j++) div += cw[j] * lds<PERS>(ft + (size_t)eidx[j] * ld + k);
-        const TC v = r1 * static_cast<TC>(qn[(size_t)t * mb.qs + x]) - r2 * div;
-        bad |= !isfinite(v);
-        qout[(size_t)t * mb.qs + x] = static_cast<TQ>(v);
+        for (int v = 0; v < V; v++) div[v] = 0;
+#pragma unroll
+        for (int j = 0; j < GRIST_MAXE; j++) {
+            TC a[V];
+            ldv<PERS, V>(ft + (size_t)r.e[j] * ld, a);
+#pragma unroll
+            for (int v = 0; v < V; v++) div[v] += r.cw[j] * a[v];
+        }
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            qv[v] = r1[v] * qv[v] - r2[v] * div[v];
+            bad |= !isfinite(qv[v]);
+        }
+        stv<V>(qout + (size_t)t * mb.qs + x, qv);
     }
     return bad;
 }
@@ -473,73 +702,115 @@ __device__ __forceinline__ bool item_update(const CellRow<TC> &r, const MemberDe
 // divergence coefficient is positive), stored as the cell's local bounds
 // {max, min}(q^n, q^td) (X2: q^td is the member of the pair that is not
 // q^n, or q^n itself), and div F^L (DFL) for the later phases.
-template <bool PERS, typename TQ, typename TC>
+template <bool PERS, typename TQ, typename TC, int V>
 __device__ __forceinline__ void item_lowres(const CellRow<TC> &r, const MemberDev &mb, int t0, int t1, int i, int k,
                                             double dt, float dtf) {
-    using T2 = typename Vec2<TC>::T;
     const int ld = mb.ld;
     const size_t x = (size_t)i * ld + k;
-    TC r1, r2;
-    stage_ratios(dv_at<PERS, TC>(mb, x), dt, dtf, r1, r2);
-    TC fe[GRIST_MAXE];
+    typename Vec2<TC>::T dv[V];
+    TC r1[V], r2[V];
+    dv_at<PERS, TC, V>(mb, x, dv);
 #pragma unroll
-    for (int j = 0; j < GRIST_MAXE; j++) fe[j] = flux_at<PERS, TC>(mb, (size_t)r.e[j] * ld + k);
+    for (int v = 0; v < V; v++) stage_ratios(dv[v], dt, dtf, r1[v], r2[v]);
+    // s dv/A F of the cell's edges; a level drains this cell through edge j
+    // where bit j V + v is set
+    TC cf[GRIST_MAXE][V];
+    unsigned out = 0;
+#pragma unroll
+    for (int j = 0; j < GRIST_MAXE; j++) {
+        flux_at<PERS, V>(mb, (size_t)r.e[j] * ld + k, cf[j]);
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            if ((cf[j][v] >= (TC)0) == (r.cw[j] > (TC)0)) out |= 1u << (j * V + v);
+            cf[j][v] = mul_rn(r.cw[j], cf[j][v]);
+        }
+    }
     const TQ *qn = (const TQ *)mb.q;
-    T2 *X2 = (T2 *)mb.X2;
-    TC *DFL = (TC *)mb.DFL;
     for (int t = t0; t < t1; t++) {
-        const TQ *qt = qn + (size_t)t * mb.qs;
-        TC divl = 0;
+        const TQ *qt = qn + (size_t)t * mb.qs + k;
+        TC divl[V], qi[V];
+        ldv<PERS, V>(qt + (size_t)i * ld, qi);
+#pragma unroll
+        for (int v = 0; v < V; v++) divl[v] = 0;
 #pragma unroll
         for (int j = 0; j < GRIST_MAXE; j++) {
-            const int up = ((fe[j] >= (TC)0) == (r.cw[j] > (TC)0)) ? i : r.nb[j];
-            divl = fma_rn(r.cw[j], mul_rn(fe[j], static_cast<TC>(lds<PERS>(qt + (size_t)up * ld + k))), divl);
+            TC a[V];
+            ldv<PERS, V>(qt + (size_t)r.nb[j] * ld, a);
+#pragma unroll
+            for (int v = 0; v < V; v++) divl[v] = fma_rn(cf[j][v], (out >> (j * V + v)) & 1u ? qi[v] : a[v], divl[v]);
         }
-        const TC qi = static_cast<TC>(qt[x]);
-        const TC qd = static_cast<TC>(static_cast<TQ>(lowres_value(r1, r2, qi, divl)));
-        X2[(size_t)t * mb.qs + x] = T2{fmax_(qi, qd), fmin_(qi, qd)};
-        DFL[(size_t)t * mb.qs + x] = divl;
+        store_lowres<TC, V>(mb, (size_t)t * mb.qs + x, r1, r2, qi, divl);
     }
 }
+
+// min(1, Q / P) for P >= TINY > 0.  binary32: the approximate reciprocal and
+// one correction of the quotient by its remainder, about half an ulp, instead
+// of the division, which takes its slow path (a call) where P is near TINY,
+// that is wherever a tracer is constant.  A quotient that overflows ends as
+// NaN, and fminf then returns 1.
+__device__ __forceinline__ float fct_ratio(float Q, float P) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(P));
+    const float a = Q * r;
+    return fminf(1.f, fmaf(fmaf(-a, P, Q), r, a));
+}
+__device__ __forceinline__ double fct_ratio(double Q, double P) { return fmin(1.0, Q / P); }
 
 // FCT 2: bounds over the cell and its neighbours of {q^n, q^td} (from the
 // cells' local bounds); antidiffusive in/out sums P+- of A = F^H - F^L (as
 // the final edge phase stored it); allowed changes Q+-; ratios
 // R+- = min(1, Q / (P + TINY)) (Sec. 2.2 (iii): TINY of the working type),
 // stored as the pair {R+, R-}.
-template <bool PERS, typename TQ, typename TC>
+template <bool PERS, typename TQ, typename TC, int V>
 __device__ __forceinline__ void item_ratios(const CellRow<TC> &r, const MemberDev &mb, int t0, int t1, int i, int k,
                                             double dt, float dtf) {
-    using T2 = typename Vec2<TC>::T;
     const int ld = mb.ld;
     const size_t x = (size_t)i * ld + k;
-    const TC dp3 = static_cast<TC>(end_mass(dv_at<PERS, TC>(mb, x), dt, dtf));
+    typename Vec2<TC>::T dv[V];
+    TC dp3[V];
+    dv_at<PERS, TC, V>(mb, x, dv);
+#pragma unroll
+    for (int v = 0; v < V; v++) dp3[v] = static_cast<TC>(end_mass(dv[v], dt, dtf));
     const TC dtc = sizeof(TC) == 4 ? (TC)dtf : (TC)dt;
-    const T2 *X2 = (const T2 *)mb.X2;
+    const TC *X2 = (const TC *)mb.X2;
     const TQ *qn = (const TQ *)mb.q;
     const TC *A = (const TC *)mb.FH;
-    T2 *R2 = (T2 *)mb.R2;
+    TC *R2 = (TC *)mb.R2;
     for (int t = t0; t < t1; t++) {
-        const T2 *xt = X2 + (size_t)t * mb.qs;
-        const TC *at = A + (size_t)t * mb.fs;
-        const T2 bi = lds<PERS>(xt + x);
-        TC qmax = bi.x, qmin = bi.y;
-        TC pp = 0, pm = 0;
+        const TC *xt = X2 + 2 * ((size_t)t * mb.qs + k);
+        const TC *at = A + (size_t)t * mb.fs + k;
+        TC bi[2 * V], qmax[V], qmin[V], pp[V], pm[V], qi[V];
+        ldv<PERS, 2 * V>(xt + 2 * (size_t)i * ld, bi);
+        ldv<PERS, V>(qn + (size_t)t * mb.qs + x, qi);
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            qmax[v] = bi[2 * v];
+            qmin[v] = bi[2 * v + 1];
+            pp[v] = pm[v] = 0;
+        }
 #pragma unroll
         for (int j = 0; j < GRIST_MAXE; j++) {
-            const T2 bn = lds<PERS>(xt + (size_t)r.nb[j] * ld + k);
-            qmax = fmax_(qmax, bn.x);
-            qmin = fmin_(qmin, bn.y);
-            const TC out = r.cw[j] * lds<PERS>(at + (size_t)r.e[j] * ld + k);  // outward A / A_i
-            pp += fmax_((TC)0, -out);
-            pm += fmax_((TC)0, out);
+            TC bn[2 * V], a[V];
+            ldv<PERS, 2 * V>(xt + 2 * (size_t)r.nb[j] * ld, bn);
+            ldv<PERS, V>(at + (size_t)r.e[j] * ld, a);
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                qmax[v] = fmax_(qmax[v], bn[2 * v]);
+                qmin[v] = fmin_(qmin[v], bn[2 * v + 1]);
+                const TC out = r.cw[j] * a[v];  // outward A / A_i
+                pp[v] += fmax_((TC)0, -out);
+                pm[v] += fmax_((TC)0, out);
+            }
         }
-        pp *= dtc;
-        pm *= dtc;
-        const TC qn_i = static_cast<TC>(qn[(size_t)t * mb.qs + x]);
-        const TC qtd_i = bi.x == qn_i ? bi.y : bi.x;
-        const TC Qp = (qmax - qtd_i) * dp3, Qm = (qtd_i - qmin) * dp3;
-        R2[(size_t)t * mb.qs + x] = T2{fmin_((TC)1, Qp / (pp + tiny_of<TC>())), fmin_((TC)1, Qm / (pm + tiny_of<TC>()))};
+        TC rr[2 * V];
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            const TC qtd = bi[2 * v] == qi[v] ? bi[2 * v + 1] : bi[2 * v];
+            const TC Qp = (qmax[v] - qtd) * dp3[v], Qm = (qtd - qmin[v]) * dp3[v];
+            rr[2 * v] = fct_ratio(Qp, pp[v] * dtc + tiny_of<TC>());
+            rr[2 * v + 1] = fct_ratio(Qm, pm[v] * dtc + tiny_of<TC>());
+        }
+        stv<2 * V>(R2 + 2 * ((size_t)t * mb.qs + x), rr);
     }
 }
 
@@ -547,37 +818,47 @@ __device__ __forceinline__ void item_ratios(const CellRow<TC> &r, const MemberDe
 // c1 -> c2 (A >= 0), min(R+(c1), R-(c2)) else; q^{n+1} = (dpi^n q^n - dt
 // div(F^L + C A)) / dpi^(3), with div F^L from the low-order phase, written
 // over q^n in place (each thread reads only its own cell's q^n).
-template <bool PERS, typename TQ, typename TC>
+template <bool PERS, typename TQ, typename TC, int V>
 __device__ __forceinline__ bool item_final(const CellRow<TC> &r, const MemberDev &mb, int t0, int t1, int i, int k,
                                            double dt, float dtf) {
-    using T2 = typename Vec2<TC>::T;
     const int ld = mb.ld;
     const size_t x = (size_t)i * ld + k;
-    TC r1, r2;
-    stage_ratios(dv_at<PERS, TC>(mb, x), dt, dtf, r1, r2);
+    typename Vec2<TC>::T dv[V];
+    TC r1[V], r2[V];
+    dv_at<PERS, TC, V>(mb, x, dv);
+#pragma unroll
+    for (int v = 0; v < V; v++) stage_ratios(dv[v], dt, dtf, r1[v], r2[v]);
     TQ *q = (TQ *)mb.q;
     const TC *A = (const TC *)mb.FH, *DFL = (const TC *)mb.DFL;
-    const T2 *R2 = (const T2 *)mb.R2;
+    const TC *R2 = (const TC *)mb.R2;
     bool bad = false;
     for (int t = t0; t < t1; t++) {
-        const TC *at = A + (size_t)t * mb.fs;
-        const T2 *rt = R2 + (size_t)t * mb.qs;
-        const T2 ri = lds<PERS>(rt + x);
-        TC div = lds<PERS>(DFL + (size_t)t * mb.qs + x);
+        const TC *at = A + (size_t)t * mb.fs + k;
+        const TC *rt = R2 + 2 * ((size_t)t * mb.qs + k);
+        TC ri[2 * V], div[V], qv[V];
+        ldv<PERS, 2 * V>(rt + 2 * (size_t)i * ld, ri);
+        ldv<PERS, V>(DFL + (size_t)t * mb.qs + x, div);
+        ldv_own<V>(q + (size_t)t * mb.qs + x, qv);
 #pragma unroll
         for (int j = 0; j < GRIST_MAXE; j++) {
-            const TC ae = lds<PERS>(at + (size_t)r.e[j] * ld + k);
-            const T2 rn = lds<PERS>(rt + (size_t)r.nb[j] * ld + k);
+            TC ae[V], rn[2 * V];
+            ldv<PERS, V>(at + (size_t)r.e[j] * ld, ae);
+            ldv<PERS, 2 * V>(rt + 2 * (size_t)r.nb[j] * ld, rn);
             const bool i_is_c1 = r.cw[j] > (TC)0;
-            const TC rp1 = i_is_c1 ? ri.x : rn.x, rm1 = i_is_c1 ? ri.y : rn.y;
-            const TC rp2 = i_is_c1 ? rn.x : ri.x, rm2 = i_is_c1 ? rn.y : ri.y;
-            const TC c = ae >= (TC)0 ? fmin_(rm1, rp2) : fmin_(rp1, rm2);
-            div += r.cw[j] * (c * ae);
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                // A leaves cell i: its R- and the neighbour's R+; A enters it: the other two
+                const bool leaves = (ae[v] >= (TC)0) == i_is_c1;
+                const TC c = leaves ? fmin_(ri[2 * v + 1], rn[2 * v]) : fmin_(ri[2 * v], rn[2 * v + 1]);
+                div[v] += r.cw[j] * (c * ae[v]);
+            }
         }
-        const size_t y = (size_t)t * mb.qs + x;
-        const TC v = r1 * static_cast<TC>(q[y]) - r2 * div;
-        bad |= !isfinite(v);
-        q[y] = static_cast<TQ>(v);
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            qv[v] = r1[v] * qv[v] - r2[v] * div[v];
+            bad |= !isfinite(qv[v]);
+        }
+        stv<V>(q + (size_t)t * mb.qs + x, qv);
     }
     return bad;
 }
@@ -588,16 +869,18 @@ __device__ __forceinline__ bool item_final(const CellRow<TC> &r, const MemberDev
 enum Phase { P_DIV = 0, P_EDGE0, P_UPD0, P_EDGE1, P_UPD1, P_EDGE2, P_UPD2, P_LOWRES, P_RATIOS, P_FINAL, P_NPHASE };
 
 // One pass over a work space.  A work item is (entity, level group g) of a
-// member and tracer group; the thread takes the LPT levels g, g + Lg, ...
-// (Lg = ceil(L / LPT)), so consecutive threads still touch consecutive
-// levels, and the entity's tables are read once for its LPT levels.
+// member and tracer group.  V > 1: the thread takes the V consecutive levels
+// g V, ..., g V + V - 1 as one vector.  V = 1: it takes the LPT levels g,
+// g + Lg, ... (Lg = ceil(L / LPT)).  Either way consecutive threads touch
+// consecutive memory, and the entity's tables are read once for its levels.
 // RING: the form of an edge phase, -1 = as B.ring says (the persistent
 // launch), 0 / 1 = compiled for one form (the per-phase kernels, so that a
-// kernel's registers serve the form it runs).
-template <bool PERS, typename TQ, typename TC, int PH, int LPT = 1, int RING = -1>
-__device__ void run_phase(const DevMesh &m, const Batch &B, uint32_t *status) {
-    const bool ring = RING < 0 ? (B.ring != 0) : (RING == 1);
-    const Space &S = (PH == P_DIV) ? B.D : ((PH == P_EDGE0 || PH == P_EDGE1 || PH == P_EDGE2) && !ring) ? B.E : B.C;
+// kernel's registers serve the form it runs), 2 = the cell-centric form with
+// the low-order solution.
+template <bool PERS, typename TQ, typename TC, int PH, int LPT = 1, int V = 1, int RING = -1>
+__device__ void run_phase(const DevMesh &m, const Batch &B, const Space &S, uint32_t *status) {
+    static_assert(V == 1 || LPT == 1, "a vector item has one level group");
+    const bool ring = RING < 0 ? (B.ring != 0) : (RING >= 1);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     int seg = -1;
     bool bad = false;
@@ -617,43 +900,32 @@ __device__ void run_phase(const DevMesh &m, const Batch &B, uint32_t *status) {
             // the final stage of a limited step stores A = F^H - F^L
             const TQ *qn = (PH == P_EDGE2 && B.fct) ? (const TQ *)mb.q : nullptr;
             if (ring) {
-                int e[GRIST_MAXE], nb[GRIST_MAXE];
-                TC cw[GRIST_MAXE];
-                load_row6(m.eoc8, ent, e);
-                load_row6(m.coc8, ent, nb);
-                load_row6(Coef<TC>::cdiv8(m), ent, cw);
-                unsigned real = 0, c1 = 0;
-#pragma unroll
-                for (int j = 0; j < GRIST_MAXE; j++) {
-                    if (cw[j] != (TC)0) real |= 1u << j;
-                    if (cw[j] > (TC)0) c1 |= 1u << j;
-                }
-                item_edge_ring<PERS, TQ, TC, LPT>(m, mb, e, nb, real, c1, qs, qn, t0, t1, ent, kg);
+                item_edge_ring<PERS, TQ, TC, LPT, V, RING == 2>(m, mb, qs, qn, t0, t1, ent, kg, B.dt, dtf);
             } else {
-                item_edge_levels<PERS, TQ, TC, LPT>(m, mb, qs, qn, t0, t1, ent, kg, B.beta1, beta);
+                item_edge_levels<PERS, TQ, TC, LPT, V>(m, mb, qs, qn, t0, t1, ent, kg, B.beta1, beta);
             }
             continue;
         }
-        // the cell's row, once for its LPT levels (FP64 weights for the
+        // the cell's row, once for its levels (FP64 weights for the
         // continuity phase); the limited-flux phase, the one with the most
-        // live values per level, reads it again for each level instead
+        // live values per level, reads it again for each strided level
         using TW = typename std::conditional<PH == P_DIV, double, TC>::type;
         constexpr bool kNb = PH == P_LOWRES || PH == P_RATIOS || PH == P_FINAL;
-        constexpr bool kRowPerLevel = PH == P_FINAL;
+        constexpr bool kRowPerLevel = PH == P_FINAL && LPT > 1;
         CellRow<TW> r;
         if (!kRowPerLevel) load_cell_row<kNb>(m, ent, r);
 #pragma unroll
         for (int u = 0; u < LPT; u++) {
-        const int k = kg + u * mb.Lg;
+        const int k = (kg + u * mb.Lg) * V;
         if (LPT > 1 && k >= mb.L) break;
         if (kRowPerLevel) load_cell_row<kNb>(m, ent, r);
-        if constexpr (PH == P_DIV) item_div<TC>(mb, r, ent, k);
-        if constexpr (PH == P_UPD0) bad |= item_update<PERS, TQ, TC>(r, mb, (TQ *)mb.qA, t0, t1, ent, k, dts, dtsf);
-        if constexpr (PH == P_UPD1) bad |= item_update<PERS, TQ, TC>(r, mb, (TQ *)mb.qB, t0, t1, ent, k, dts, dtsf);
-        if constexpr (PH == P_UPD2) bad |= item_update<PERS, TQ, TC>(r, mb, (TQ *)mb.q, t0, t1, ent, k, dts, dtsf);
-        if constexpr (PH == P_LOWRES) item_lowres<PERS, TQ, TC>(r, mb, t0, t1, ent, k, B.dt, dtf);
-        if constexpr (PH == P_RATIOS) item_ratios<PERS, TQ, TC>(r, mb, t0, t1, ent, k, B.dt, dtf);
-        if constexpr (PH == P_FINAL) bad |= item_final<PERS, TQ, TC>(r, mb, t0, t1, ent, k, B.dt, dtf);
+        if constexpr (PH == P_DIV) item_div<TC, V>(mb, r, ent, k);
+        if constexpr (PH == P_UPD0) bad |= item_update<PERS, TQ, TC, V>(r, mb, (TQ *)mb.qA, t0, t1, ent, k, dts, dtsf);
+        if constexpr (PH == P_UPD1) bad |= item_update<PERS, TQ, TC, V>(r, mb, (TQ *)mb.qB, t0, t1, ent, k, dts, dtsf);
+        if constexpr (PH == P_UPD2) bad |= item_update<PERS, TQ, TC, V>(r, mb, (TQ *)mb.q, t0, t1, ent, k, dts, dtsf);
+        if constexpr (PH == P_LOWRES) item_lowres<PERS, TQ, TC, V>(r, mb, t0, t1, ent, k, B.dt, dtf);
+        if constexpr (PH == P_RATIOS) item_ratios<PERS, TQ, TC, V>(r, mb, t0, t1, ent, k, B.dt, dtf);
+        if constexpr (PH == P_FINAL) bad |= item_final<PERS, TQ, TC, V>(r, mb, t0, t1, ent, k, B.dt, dtf);
         }
     }
     if (bad) atomicOr(status, GRIST_FLAG_NONFINITE);
@@ -686,20 +958,35 @@ __device__ void run_phase(const DevMesh &m, const Batch &B, uint32_t *status) {
 #endif
 constexpr int kTracerRegLimit = 65536 / kTracerMaxBlock;
 constexpr int cap_or_none(int r) { return r > 0 && r < kTracerRegLimit ? r : kTracerRegLimit; }
-template <typename TC, int PH, int RING> constexpr int tracer_phase_regs() {
-    return sizeof(TC) != 4                                      ? kTracerRegLimit
-           : (PH == P_EDGE0 || PH == P_EDGE1 || PH == P_EDGE2)
-               ? cap_or_none(RING == 1 ? GRIST_TR_REGS_RING : GRIST_TR_REGS_EDGE)
-           : (PH == P_UPD0 || PH == P_UPD1 || PH == P_UPD2)    ? cap_or_none(GRIST_TR_REGS_UPD)
-           : PH == P_LOWRES                                    ? cap_or_none(GRIST_TR_REGS_LOWRES)
-           : PH == P_RATIOS                                    ? cap_or_none(GRIST_TR_REGS_RATIOS)
-           : PH == P_FINAL                                     ? cap_or_none(GRIST_TR_REGS_FINAL)
-                                                               : kTracerRegLimit;
+template <typename TC, int PH, int V, int RING> constexpr int tracer_phase_regs() {
+    constexpr bool edge = PH == P_EDGE0 || PH == P_EDGE1 || PH == P_EDGE2;
+    constexpr bool upd = PH == P_UPD0 || PH == P_UPD1 || PH == P_UPD2;
+    if (sizeof(TC) != 4) return kTracerRegLimit;
+    // vector items: bytes in flight come from the width of their loads, so more
+    // registers and fewer warps do better than for single levels
+    if (V > 1)
+        return cap_or_none(edge             ? (RING == 2 ? (V == 4 ? 0 : 80) : (RING == 1 ? 72 : 0))
+                           : PH == P_LOWRES ? 72
+                                            : 0);
+    return cap_or_none(edge             ? (RING >= 1 ? GRIST_TR_REGS_RING : GRIST_TR_REGS_EDGE)
+                       : upd            ? GRIST_TR_REGS_UPD
+                       : PH == P_LOWRES ? GRIST_TR_REGS_LOWRES
+                       : PH == P_RATIOS ? GRIST_TR_REGS_RATIOS
+                       : PH == P_FINAL  ? GRIST_TR_REGS_FINAL
+                                        : 0);
 }
 
-template <typename TQ, typename TC, int PH, int LPT, int RING>
-__global__ void __maxnreg__((tracer_phase_regs<TC, PH, RING>())) k_tracer_phase(DevMesh m, Batch B, uint32_t *status) {
-    run_phase<false, TQ, TC, PH, LPT, RING>(m, B, status);
+// The space a phase runs over: cells without groups, edges (edge-centric
+// fluxes) or cells with tracer groups.
+constexpr bool is_edge_phase(int ph) { return ph == P_EDGE0 || ph == P_EDGE1 || ph == P_EDGE2; }
+__host__ __device__ __forceinline__ const Space &phase_space(const Batch &B, int ph, bool ring, int cls) {
+    return ph == P_DIV ? B.D[cls] : (is_edge_phase(ph) && !ring) ? B.E[cls] : B.C[cls];
+}
+
+template <typename TQ, typename TC, int PH, int LPT, int V, int RING>
+__global__ void __maxnreg__((tracer_phase_regs<TC, PH, V, RING>())) k_tracer_phase(DevMesh m, Batch B, uint32_t *status) {
+    constexpr int cls = V == 4 ? 2 : (V == 2 ? 1 : 0);
+    run_phase<false, TQ, TC, PH, LPT, V, RING>(m, B, phase_space(B, PH, RING >= 1, cls), status);
 }
 
 // Fused RK stage (no limiter) on one tile x 32 levels x the tracers of one
@@ -1010,27 +1297,27 @@ __global__ void k_wait_selftest(unsigned *word, unsigned *abort_word, long long 
 // grid barrier between consecutive ones.
 template <typename TQ, typename TC>
 __global__ void k_tracer_persistent(DevMesh m, Batch B, unsigned *bar, uint32_t *status) {
-    run_phase<true, TQ, TC, P_DIV>(m, B, status);
+    run_phase<true, TQ, TC, P_DIV>(m, B, phase_space(B, P_DIV, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_EDGE0>(m, B, status);
+    run_phase<true, TQ, TC, P_EDGE0>(m, B, phase_space(B, P_EDGE0, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_UPD0>(m, B, status);
+    run_phase<true, TQ, TC, P_UPD0>(m, B, phase_space(B, P_UPD0, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_EDGE1>(m, B, status);
+    run_phase<true, TQ, TC, P_EDGE1>(m, B, phase_space(B, P_EDGE1, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_UPD1>(m, B, status);
+    run_phase<true, TQ, TC, P_UPD1>(m, B, phase_space(B, P_UPD1, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_EDGE2>(m, B, status);
+    run_phase<true, TQ, TC, P_EDGE2>(m, B, phase_space(B, P_EDGE2, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
     if (!B.fct) {
-        run_phase<true, TQ, TC, P_UPD2>(m, B, status);
+        run_phase<true, TQ, TC, P_UPD2>(m, B, phase_space(B, P_UPD2, B.ring != 0, 0), status);
         return;
     }
-    run_phase<true, TQ, TC, P_LOWRES>(m, B, status);
+    run_phase<true, TQ, TC, P_LOWRES>(m, B, phase_space(B, P_LOWRES, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_RATIOS>(m, B, status);
+    run_phase<true, TQ, TC, P_RATIOS>(m, B, phase_space(B, P_RATIOS, B.ring != 0, 0), status);
     if (!grid_sync(bar, status)) return;
-    run_phase<true, TQ, TC, P_FINAL>(m, B, status);
+    run_phase<true, TQ, TC, P_FINAL>(m, B, phase_space(B, P_FINAL, B.ring != 0, 0), status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1040,16 +1327,33 @@ size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct HostPlan {
     std::vector<MemberDev> mem;
-    std::vector<unsigned long long> sD, sC, sE, sT;
-    std::vector<int2> mD, mC, mE, mT;
+    struct Seg {
+        std::vector<unsigned long long> start;   // closed by the total
+        std::vector<int2> mg;
+        size_t o_start = 0, o_mg = 0;            // offsets in the device table
+    };
+    Seg D[kVecClasses], C[kVecClasses], E[kVecClasses], T;
     size_t scratch_bytes = 0;
 };
+
+// The widest vector of consecutive levels, as a power of two, that the
+// member's rows and pointers allow: up to 16 bytes of q and of its binary32
+// scratch, whole vectors only (L and ld multiples of it).
+template <typename TQ> int vec_class(const grist_tracer_member &u) {
+    auto at = [](const void *p, size_t a) { return ((uintptr_t)p) % a == 0; };
+    for (int c = sizeof(TQ) == 4 ? 2 : 1; c > 0; c--) {
+        const int V = 1 << c;
+        if (u.n_levels % V == 0 && u.ld % V == 0 && at(u.q, V * sizeof(TQ)) && at(u.dpi, 16) && at(u.mass_flux, 16))
+            return c;
+    }
+    return 0;
+}
 
 template <typename TQ, typename TC>
 int plan_batch(const DevMesh &m, const grist_tracer_batch *b, int tpt, int lpt, HostPlan &P) {
     P = HostPlan();
     size_t off = 0;
-    unsigned long long tD = 0, tC = 0, tE = 0, tT = 0;
+    unsigned long long tD[kVecClasses] = {0}, tC[kVecClasses] = {0}, tE[kVecClasses] = {0}, tT = 0;
     const unsigned long long ntiles = ((unsigned long long)m.nC + kTileCells - 1) / kTileCells;
     for (int i = 0; i < b->n_members; i++) {
         const grist_tracer_member &u = b->members[i];
@@ -1063,7 +1367,10 @@ int plan_batch(const DevMesh &m, const grist_tracer_batch *b, int tpt, int lpt, 
         d.ld = u.ld;
         d.Mv = u.vmass_flux;
         d.ldi = u.ld_int;
-        d.Lg = (u.n_levels + lpt - 1) / lpt;
+        // levels_per_thread 1 is one level; 2 is a vector where the layout
+        // allows one, else two levels Lg apart
+        const int vc = lpt > 1 ? vec_class<TQ>(u) : 0;
+        d.Lg = vc ? u.n_levels >> vc : (u.n_levels + lpt - 1) / lpt;
         d.DL = make_div((uint32_t)d.Lg);
         d.qs = (unsigned long long)m.nC * u.ld;
         d.fs = (unsigned long long)m.nE * u.ld;
@@ -1080,22 +1387,25 @@ int plan_batch(const DevMesh &m, const grist_tracer_batch *b, int tpt, int lpt, 
         d.DV = (void *)(uintptr_t)off; off += al256(d.qs * 2 * sizeof(TC));
         const int idx = (int)P.mem.size();
         const int G = (d.T + tpt - 1) / tpt;
-        P.sD.push_back(tD); P.mD.push_back(make_int2(idx, 0));
-        tD += (unsigned long long)m.nC * d.Lg;
+        auto add = [&](HostPlan::Seg &S, unsigned long long &tot, int g, unsigned long long n) {
+            S.start.push_back(tot);
+            S.mg.push_back(make_int2(idx, g));
+            tot += n;
+        };
+        add(P.D[vc], tD[vc], 0, (unsigned long long)m.nC * d.Lg);
         for (int g = 0; g < G; g++) {
-            P.sC.push_back(tC); P.mC.push_back(make_int2(idx, g));
-            tC += (unsigned long long)m.nC * d.Lg;
-            P.sE.push_back(tE); P.mE.push_back(make_int2(idx, g));
-            tE += (unsigned long long)m.nE * d.Lg;
-            P.sT.push_back(tT); P.mT.push_back(make_int2(idx, g));
-            tT += ntiles * (unsigned long long)((d.L + 31) / 32);
+            add(P.C[vc], tC[vc], g, (unsigned long long)m.nC * d.Lg);
+            add(P.E[vc], tE[vc], g, (unsigned long long)m.nE * d.Lg);
+            add(P.T, tT, g, ntiles * (unsigned long long)((d.L + 31) / 32));
         }
         P.mem.push_back(d);
     }
-    P.sD.push_back(tD);
-    P.sC.push_back(tC);
-    P.sE.push_back(tE);
-    P.sT.push_back(tT);
+    for (int c = 0; c < kVecClasses; c++) {
+        P.D[c].start.push_back(tD[c]);
+        P.C[c].start.push_back(tC[c]);
+        P.E[c].start.push_back(tE[c]);
+    }
+    P.T.start.push_back(tT);
     P.scratch_bytes = off;
     return GRIST_OK;
 }
@@ -1121,24 +1431,24 @@ int upload_plan(grist_mesh_s *h, TracerCtx *c, HostPlan &P, const grist_tracer_b
     const size_t nm = P.mem.size();
     size_t o = 0;
     const size_t o_mem = o; o += al256(nm * sizeof(MemberDev));
-    const size_t o_sD = o; o += al256(P.sD.size() * 8);
-    const size_t o_sC = o; o += al256(P.sC.size() * 8);
-    const size_t o_sE = o; o += al256(P.sE.size() * 8);
-    const size_t o_mD = o; o += al256(P.mD.size() * sizeof(int2));
-    const size_t o_mC = o; o += al256(P.mC.size() * sizeof(int2));
-    const size_t o_mE = o; o += al256(P.mE.size() * sizeof(int2));
-    const size_t o_sT = o; o += al256(P.sT.size() * 8);
-    const size_t o_mT = o; o += al256(P.mT.size() * sizeof(int2));
+    auto each = [&](auto &&fn) {
+        for (int k = 0; k < kVecClasses; k++) {
+            fn(P.D[k], B.D[k]);
+            fn(P.C[k], B.C[k]);
+            fn(P.E[k], B.E[k]);
+        }
+        fn(P.T, B.T);
+    };
+    each([&](HostPlan::Seg &S, Space &) {
+        S.o_start = o; o += al256(S.start.size() * 8);
+        S.o_mg = o; o += al256(S.mg.size() * sizeof(int2));
+    });
     std::vector<char> ht(o, 0);
     std::memcpy(ht.data() + o_mem, P.mem.data(), nm * sizeof(MemberDev));
-    std::memcpy(ht.data() + o_sD, P.sD.data(), P.sD.size() * 8);
-    std::memcpy(ht.data() + o_sC, P.sC.data(), P.sC.size() * 8);
-    std::memcpy(ht.data() + o_sE, P.sE.data(), P.sE.size() * 8);
-    std::memcpy(ht.data() + o_mD, P.mD.data(), P.mD.size() * sizeof(int2));
-    std::memcpy(ht.data() + o_mC, P.mC.data(), P.mC.size() * sizeof(int2));
-    std::memcpy(ht.data() + o_mE, P.mE.data(), P.mE.size() * sizeof(int2));
-    std::memcpy(ht.data() + o_sT, P.sT.data(), P.sT.size() * 8);
-    std::memcpy(ht.data() + o_mT, P.mT.data(), P.mT.size() * sizeof(int2));
+    each([&](HostPlan::Seg &S, Space &) {
+        std::memcpy(ht.data() + S.o_start, S.start.data(), S.start.size() * 8);
+        if (!S.mg.empty()) std::memcpy(ht.data() + S.o_mg, S.mg.data(), S.mg.size() * sizeof(int2));
+    });
     int ti = -1;
     for (size_t x = 0; x < c->tabs.size() && ti < 0; x++)
         if (c->tabs[x].host.size() == o && std::memcmp(c->tabs[x].host.data(), ht.data(), o) == 0) ti = (int)x;
@@ -1173,10 +1483,10 @@ int upload_plan(grist_mesh_s *h, TracerCtx *c, HostPlan &P, const grist_tracer_b
     }
     B.mem = (const MemberDev *)(dtab + o_mem);
     B.nm = (int)nm;
-    B.D = Space{(const unsigned long long *)(dtab + o_sD), (const int2 *)(dtab + o_mD), (int)P.mD.size(), P.sD.back()};
-    B.C = Space{(const unsigned long long *)(dtab + o_sC), (const int2 *)(dtab + o_mC), (int)P.mC.size(), P.sC.back()};
-    B.E = Space{(const unsigned long long *)(dtab + o_sE), (const int2 *)(dtab + o_mE), (int)P.mE.size(), P.sE.back()};
-    B.T = Space{(const unsigned long long *)(dtab + o_sT), (const int2 *)(dtab + o_mT), (int)P.mT.size(), P.sT.back()};
+    each([&](HostPlan::Seg &S, Space &D) {
+        D = Space{(const unsigned long long *)(dtab + S.o_start), (const int2 *)(dtab + S.o_mg), (int)S.mg.size(),
+                  S.start.back()};
+    });
     B.tpt = c->tune.tracers_per_thread;
     B.lpt = c->tune.persistent ? 1 : c->tune.levels_per_thread;
     B.dt = dt;
@@ -1252,45 +1562,64 @@ int enqueue_horizontal(grist_mesh_s *h, TracerCtx *c, const Batch &B, cudaStream
     for (int ph = P_DIV; ph < P_NPHASE; ph++) {
         if (!B.fct && ph > P_UPD2) break;
         if (B.fct && ph == P_UPD2) continue;
+        // the cell-centric first edge phase of a limited step does the
+        // low-order phase too (a fused stage has no such edge phase)
+        const bool with_low = B.fct && B.ring && !fused;
+        if (ph == P_LOWRES && with_low) continue;
         if (fused && (ph == P_EDGE0 || ph == P_EDGE1 || (!B.fct && ph == P_EDGE2))) continue;
         if (fused && (ph == P_UPD0 || ph == P_UPD1 || ph == P_UPD2)) {
             const int rc = launch_tile(ph == P_UPD0 ? 0 : (ph == P_UPD1 ? 1 : 2));
             if (rc != GRIST_OK) return rc;
             continue;
         }
-        const Space &S = (ph == P_DIV) ? B.D : ((ph == P_EDGE0 || ph == P_EDGE1 || ph == P_EDGE2) && !B.ring) ? B.E : B.C;
-        long long want = (long long)((S.total + block - 1) / block);
-        const long long cap = (long long)sms * 2048 * 32 / block;  // enough blocks to fill every SM many times
-        const unsigned grid = (unsigned)(want < 1 ? 1 : (want > cap ? cap : want));
-        const char *nm = sizeof(TC) == 4 ? names_f[ph] : names_d[ph];
-        switch (ph) {
-#define GRIST_PHASE_LAUNCH(P_, R_) \
-        if (B.lpt == 2) GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 2, R_><<<grid, block, 0, st>>>(m, B, status))); \
-        else GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 1, R_><<<grid, block, 0, st>>>(m, B, status)));
-#define GRIST_PHASE_CASE(P_) \
-    case P_:                                                                                                   \
-        if constexpr (P_ == P_EDGE0 || P_ == P_EDGE1 || P_ == P_EDGE2) {                                       \
-            if (B.ring) {                                                                                      \
-                GRIST_PHASE_LAUNCH(P_, 1)                                                                      \
-            } else {                                                                                           \
-                GRIST_PHASE_LAUNCH(P_, 0)                                                                      \
-            }                                                                                                  \
-        } else {                                                                                               \
-            GRIST_PHASE_LAUNCH(P_, 0)                                                                          \
-        }                                                                                                      \
+        const char *nm = ph == P_EDGE0 && with_low ? (sizeof(TC) == 4 ? "k_tr_edge_low/mix" : "k_tr_edge_low/fp64")
+                         : sizeof(TC) == 4         ? names_f[ph]
+                                                   : names_d[ph];
+        for (int cls = 0; cls < kVecClasses; cls++) {
+            const unsigned long long total = phase_space(B, ph, B.ring != 0, cls).total;
+            if (total == 0) continue;
+            const long long want = (long long)((total + block - 1) / block);
+            const long long cap = (long long)sms * 2048 * 32 / block;  // enough blocks to fill every SM many times
+            const unsigned grid = (unsigned)(want > cap ? cap : want);
+            switch (ph) {
+#define GRIST_PHASE_LAUNCH(P_, R_)                                                                              \
+    if constexpr (sizeof(TC) == 4) {                                                                            \
+        if (cls == 2)                                                                                           \
+            GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 1, 4, R_><<<grid, block, 0, st>>>(m, B, status))); \
+    }                                                                                                           \
+    if (cls == 1)                                                                                               \
+        GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 1, 2, R_><<<grid, block, 0, st>>>(m, B, status)));  \
+    else if (cls == 0 && B.lpt == 2)                                                                            \
+        GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 2, 1, R_><<<grid, block, 0, st>>>(m, B, status)));  \
+    else if (cls == 0)                                                                                          \
+        GRIST_LAUNCH(h, nm, st, (k_tracer_phase<TQ, TC, P_, 1, 1, R_><<<grid, block, 0, st>>>(m, B, status)));
+#define GRIST_PHASE_CASE(P_)                     \
+    case P_:                                     \
+        if constexpr (is_edge_phase(P_)) {       \
+            if (P_ == P_EDGE0 && with_low) {     \
+                GRIST_PHASE_LAUNCH(P_, P_ == P_EDGE0 ? 2 : 1) \
+            } else if (B.ring) {                 \
+                GRIST_PHASE_LAUNCH(P_, 1)        \
+            } else {                             \
+                GRIST_PHASE_LAUNCH(P_, 0)        \
+            }                                    \
+        } else {                                 \
+            GRIST_PHASE_LAUNCH(P_, 0)            \
+        }                                        \
         break;
-            GRIST_PHASE_CASE(P_DIV)
-            GRIST_PHASE_CASE(P_EDGE0)
-            GRIST_PHASE_CASE(P_UPD0)
-            GRIST_PHASE_CASE(P_EDGE1)
-            GRIST_PHASE_CASE(P_UPD1)
-            GRIST_PHASE_CASE(P_EDGE2)
-            GRIST_PHASE_CASE(P_UPD2)
-            GRIST_PHASE_CASE(P_LOWRES)
-            GRIST_PHASE_CASE(P_RATIOS)
-            GRIST_PHASE_CASE(P_FINAL)
+                GRIST_PHASE_CASE(P_DIV)
+                GRIST_PHASE_CASE(P_EDGE0)
+                GRIST_PHASE_CASE(P_UPD0)
+                GRIST_PHASE_CASE(P_EDGE1)
+                GRIST_PHASE_CASE(P_UPD1)
+                GRIST_PHASE_CASE(P_EDGE2)
+                GRIST_PHASE_CASE(P_UPD2)
+                GRIST_PHASE_CASE(P_LOWRES)
+                GRIST_PHASE_CASE(P_RATIOS)
+                GRIST_PHASE_CASE(P_FINAL)
 #undef GRIST_PHASE_CASE
 #undef GRIST_PHASE_LAUNCH
+            }
         }
     }
     return cudaGetLastError() == cudaSuccess ? GRIST_OK : GRIST_ECUDA;
