@@ -188,6 +188,86 @@ template <typename TC> __device__ __forceinline__ TC tiny_of();
 template <> __device__ __forceinline__ double tiny_of<double>() { return 2.2250738585072014e-308; }
 template <> __device__ __forceinline__ float tiny_of<float>() { return 1.17549435e-38f; }
 
+// Comparisons, maxima and minima of binary64 in integer arithmetic.  A DSETP
+// occupies the FP64 pipe, which bounds the FP64 policy, like an addition: 64
+// cycles of a scheduler for a warp; the integer form is 8 to 12 instructions of
+// the otherwise idle ALU.  The order key of a double's bits: negative
+// numbers with their magnitude bits inverted, so that keys compare like the
+// numbers (+-NaN beyond the infinities); the map is its own inverse.
+__device__ __forceinline__ long long okey(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double of_okey(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+constexpr long long kKeyInf = 0x7ff0000000000000ll;       // of +infinity
+constexpr long long kKeyNegInf = ~kKeyInf;                 // of -infinity
+
+// x >= 0, with -0 (NaN by its sign)
+__device__ __forceinline__ bool nonneg(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 || b == (long long)0x8000000000000000ull;
+}
+__device__ __forceinline__ bool nonneg(float x) { return x >= 0.f; }
+// x > 0 and x != 0 for the finite mesh weights
+__device__ __forceinline__ bool pos(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool pos(float x) { return x > 0.f; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
+__device__ __forceinline__ bool is_nan(double x) { return (__double_as_longlong(x) & 0x7fffffffffffffffll) > kKeyInf; }
+
+// Running maximum and minimum that ignore NaN as fmax and fmin do.
+template <typename TC> struct Bounds;
+template <> struct Bounds<float> {
+    float hi, lo;
+    __device__ __forceinline__ Bounds() {}
+    __device__ __forceinline__ Bounds(float a, float b) : hi(a), lo(b) {}
+    __device__ __forceinline__ void take(float a, float b) {
+        hi = fmaxf(hi, a);
+        lo = fminf(lo, b);
+    }
+    __device__ __forceinline__ float max() const { return hi; }
+    __device__ __forceinline__ float min() const { return lo; }
+};
+template <> struct Bounds<double> {
+    long long hi, lo;   // keys; NaN starts as the key that every number beats
+    __device__ __forceinline__ Bounds() {}
+    __device__ __forceinline__ Bounds(double a, double b) : hi(okey(a)), lo(okey(b)) {
+        if (hi > kKeyInf) hi = (long long)0x8000000000000000ull;
+        if (lo < kKeyNegInf) lo = 0x7fffffffffffffffll;
+    }
+    __device__ __forceinline__ void take(double a, double b) {
+        const long long ka = okey(a), kb = okey(b);
+        if (ka > hi && ka <= kKeyInf) hi = ka;
+        if (kb < lo && kb >= kKeyNegInf) lo = kb;
+    }
+    __device__ __forceinline__ double max() const { return of_okey(hi); }
+    __device__ __forceinline__ double min() const { return of_okey(lo); }
+};
+// min(a, b) of two numbers (no NaN)
+__device__ __forceinline__ float min_num(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ double min_num(double a, double b) { return okey(b) < okey(a) ? b : a; }
+
+// a == b for a value and a copy of it
+__device__ __forceinline__ bool same_num(float a, float b) { return a == b; }
+__device__ __forceinline__ bool same_num(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+
+// pm += max(0, x), pp += max(0, -x): the other sum would gain a zero, so one
+// addition serves both.  NaN adds nothing.
+__device__ __forceinline__ void add_signed(float x, float &pp, float &pm) {
+    pp += fmaxf(0.f, -x);
+    pm += fmaxf(0.f, x);
+}
+__device__ __forceinline__ void add_signed(double x, double &pp, double &pm) {
+    const bool neg = __double2hiint(x) < 0;
+    const double acc = neg ? pp : pm;
+    double sum = acc + fabs(x);
+    if (is_nan(x)) sum = acc;
+    pp = neg ? sum : pp;
+    pm = neg ? pm : sum;
+}
+
 // ---------------------------------------------------------------------------
 // phase bodies (one work item each)
 
@@ -525,8 +605,10 @@ __device__ __forceinline__ void store_lowres(const MemberDev &mb, size_t y, cons
 #pragma unroll
     for (int v = 0; v < V; v++) {
         const TC qd = lowres_value(r1[v], r2[v], qi[v], divl[v]);
-        b[2 * v] = fmax_(qi[v], qd);
-        b[2 * v + 1] = fmin_(qi[v], qd);
+        Bounds<TC> bd(qi[v], qi[v]);
+        bd.take(qd, qd);
+        b[2 * v] = bd.max();
+        b[2 * v + 1] = bd.min();
     }
     stv<2 * V>((TC *)mb.X2 + 2 * y, b);
     stv<V>((TC *)mb.DFL + y, divl);
@@ -560,11 +642,11 @@ __device__ __forceinline__ void item_edge_ring(const DevMesh &m, const MemberDev
             for (int j = 0; j < GRIST_MAXE; j++) {
                 TC f[V];
                 flux_at<PERS, V>(mb, (size_t)e[j] * ld + k, f);
-                if (cw[j] > (TC)0) c1 |= 1u << j;
-                if (cw[j] != (TC)0) {   // a real edge
+                if (pos(cw[j])) c1 |= 1u << j;
+                if (nonzero(cw[j])) {   // a real edge
 #pragma unroll
                     for (int v = 0; v < V; v++)
-                        if ((f[v] >= (TC)0) == (cw[j] > (TC)0)) out |= 1u << (8 * v + j);
+                        if (nonneg(f[v]) == pos(cw[j])) out |= 1u << (8 * v + j);
                 }
             }
         }
@@ -721,7 +803,7 @@ __device__ __forceinline__ void item_lowres(const CellRow<TC> &r, const MemberDe
         flux_at<PERS, V>(mb, (size_t)r.e[j] * ld + k, cf[j]);
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            if ((cf[j][v] >= (TC)0) == (r.cw[j] > (TC)0)) out |= 1u << (j * V + v);
+            if (nonneg(cf[j][v]) == pos(r.cw[j])) out |= 1u << (j * V + v);
             cf[j][v] = mul_rn(r.cw[j], cf[j][v]);
         }
     }
@@ -754,7 +836,21 @@ __device__ __forceinline__ float fct_ratio(float Q, float P) {
     const float a = Q * r;
     return fminf(1.f, fmaf(fmaf(-a, P, Q), r, a));
 }
-__device__ __forceinline__ double fct_ratio(double Q, double P) { return fmin(1.0, Q / P); }
+// binary64: 1 where Q >= P, decided on the keys, so that a warp none of whose
+// cells is limited issues no division; else Q/P from the FMA reciprocal and
+// the same correction (P above 2^1020: the division).  NaN gives 1.
+__device__ __forceinline__ double fct_ratio(double Q, double P) {
+    if (okey(Q) >= okey(P)) return 1.0;
+    double a;
+    if (__double2hiint(P) < 0x7fb00000) {
+        const double r = rcp_nr(P);
+        a = Q * r;
+        a = fma(fma(-a, P, Q), r, a);
+    } else {
+        a = Q / P;
+    }
+    return is_nan(a) ? 1.0 : a;
+}
 
 // FCT 2: bounds over the cell and its neighbours of {q^n, q^td} (from the
 // cells' local bounds); antidiffusive in/out sums P+- of A = F^H - F^L (as
@@ -779,13 +875,13 @@ __device__ __forceinline__ void item_ratios(const CellRow<TC> &r, const MemberDe
     for (int t = t0; t < t1; t++) {
         const TC *xt = X2 + 2 * ((size_t)t * mb.qs + k);
         const TC *at = A + (size_t)t * mb.fs + k;
-        TC bi[2 * V], qmax[V], qmin[V], pp[V], pm[V], qi[V];
+        TC bi[2 * V], pp[V], pm[V], qi[V];
         ldv<PERS, 2 * V>(xt + 2 * (size_t)i * ld, bi);
         ldv<PERS, V>(qn + (size_t)t * mb.qs + x, qi);
+        Bounds<TC> bd[V];
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            qmax[v] = bi[2 * v];
-            qmin[v] = bi[2 * v + 1];
+            bd[v] = Bounds<TC>(bi[2 * v], bi[2 * v + 1]);
             pp[v] = pm[v] = 0;
         }
 #pragma unroll
@@ -795,18 +891,15 @@ __device__ __forceinline__ void item_ratios(const CellRow<TC> &r, const MemberDe
             ldv<PERS, V>(at + (size_t)r.e[j] * ld, a);
 #pragma unroll
             for (int v = 0; v < V; v++) {
-                qmax[v] = fmax_(qmax[v], bn[2 * v]);
-                qmin[v] = fmin_(qmin[v], bn[2 * v + 1]);
-                const TC out = r.cw[j] * a[v];  // outward A / A_i
-                pp[v] += fmax_((TC)0, -out);
-                pm[v] += fmax_((TC)0, out);
+                bd[v].take(bn[2 * v], bn[2 * v + 1]);
+                add_signed(r.cw[j] * a[v], pp[v], pm[v]);  // outward A / A_i
             }
         }
         TC rr[2 * V];
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            const TC qtd = bi[2 * v] == qi[v] ? bi[2 * v + 1] : bi[2 * v];
-            const TC Qp = (qmax[v] - qtd) * dp3[v], Qm = (qtd - qmin[v]) * dp3[v];
+            const TC qtd = same_num(bi[2 * v], qi[v]) ? bi[2 * v + 1] : bi[2 * v];
+            const TC Qp = (bd[v].max() - qtd) * dp3[v], Qm = (qtd - bd[v].min()) * dp3[v];
             rr[2 * v] = fct_ratio(Qp, pp[v] * dtc + tiny_of<TC>());
             rr[2 * v + 1] = fct_ratio(Qm, pm[v] * dtc + tiny_of<TC>());
         }
@@ -844,12 +937,12 @@ __device__ __forceinline__ bool item_final(const CellRow<TC> &r, const MemberDev
             TC ae[V], rn[2 * V];
             ldv<PERS, V>(at + (size_t)r.e[j] * ld, ae);
             ldv<PERS, 2 * V>(rt + 2 * (size_t)r.nb[j] * ld, rn);
-            const bool i_is_c1 = r.cw[j] > (TC)0;
+            const bool i_is_c1 = pos(r.cw[j]);
 #pragma unroll
             for (int v = 0; v < V; v++) {
                 // A leaves cell i: its R- and the neighbour's R+; A enters it: the other two
-                const bool leaves = (ae[v] >= (TC)0) == i_is_c1;
-                const TC c = leaves ? fmin_(ri[2 * v + 1], rn[2 * v]) : fmin_(ri[2 * v], rn[2 * v + 1]);
+                const bool leaves = nonneg(ae[v]) == i_is_c1;
+                const TC c = leaves ? min_num(ri[2 * v + 1], rn[2 * v]) : min_num(ri[2 * v], rn[2 * v + 1]);
                 div[v] += r.cw[j] * (c * ae[v]);
             }
         }
