@@ -249,6 +249,14 @@ template <> struct Bounds<double> {
 __device__ __forceinline__ float min_num(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double min_num(double a, double b) { return okey(b) < okey(a) ? b : a; }
 
+// a <= b (false for NaN), |a|
+__device__ __forceinline__ bool le_num(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool le_num(double a, double b) {
+    const long long ka = okey(a), kb = okey(b);
+    return ka <= kb && kb <= kKeyInf && ka >= kKeyNegInf;
+}
+__device__ __forceinline__ float abs_num(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_num(double x) { return fabs(x); }
 // a == b for a value and a copy of it
 __device__ __forceinline__ bool same_num(float a, float b) { return a == b; }
 __device__ __forceinline__ bool same_num(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
@@ -1200,136 +1208,168 @@ __global__ void __launch_bounds__(256) k_tr_tile_stage(DevMesh m, TileMesh tm, B
 __device__ __forceinline__ double vinv(double x) { return rcp(x); }   // correctly rounded, as 1.0 / x
 __device__ __forceinline__ float vinv(float x) { return 1.0f / x; }
 
-// One warp per column, lanes over levels (level k = lane + 32 r, r < R;
-// R = 2 up to 64 levels, else 4).  Each lane forms the flux split
-// at the two interfaces of its layers (an interface shared by two layers is
-// split by both from the same operands, so identically).  When no interface
-// of the column has an implicit share (every Courant number <= cmax, the
-// usual case) the tridiagonal system is diagonal: the Thomas sweep then
-// reduces exactly to q+_k = rhs_k * (1 / b_k), which every lane evaluates for
-// its own levels in parallel.  Otherwise the rows go through shared memory
-// and one lane runs the Thomas sweep of the column; the diagonal case is
-// exactly what that sweep computes when the off-diagonals vanish.
+// One warp per column; lane l holds the K consecutive levels from l K (K =
+// ceil(L / 32)) and the interfaces above them, so the neighbours it needs
+// come from the next lanes by shuffles, a tracer's column is read once, and
+// each interface's flux is formed once.  Whether the interface moves explicitly
+// is decided by |M| dt <= cmax dpi*_donor (no division); only an interface
+// beyond that takes the Courant number and its share.  When no interface of
+// the column has an implicit share (the usual case) the tridiagonal system is
+// diagonal: the Thomas sweep then reduces to q+_k = rhs_k * (1 / b_k), which
+// every lane evaluates for its own levels.  Otherwise the rows go through
+// shared memory and one lane runs the sweep.  Up to kVertT tracers' columns
+// are loaded before the first is used.  Level 7, 4 tracers, 60 levels, us a
+// launch against a split by both neighbours with a division each and lanes
+// over every 32nd level: binary64 1946 -> 585 (FP64 pipe, 26.7 -> 8
+// instructions a tracer-level), binary32 246 -> 125 (memory latency).
 constexpr int kVertWarps = 8;
+constexpr int kVertT = 4;
 
-template <typename TQ, typename TC, int kVertR>
+template <typename TQ, typename TC, int K, bool VEC>
 __global__ void __launch_bounds__(kVertWarps * 32) k_tr_vertical(DevMesh m, MemberDev mb, double dt, double cmax,
                                                                 uint32_t *status) {
-    __shared__ TC sA[kVertWarps][kVertMaxL], sB[kVertWarps][kVertMaxL], sC[kVertWarps][kVertMaxL],
-        sD[kVertWarps][kVertMaxL];
+    __shared__ TC sA[kVertWarps][K * 32], sB[kVertWarps][K * 32], sC[kVertWarps][K * 32], sD[kVertWarps][K * 32],
+        sE[kVertWarps][K * 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kVertWarps + warp;
     if (i >= m.nC) return;   // whole warps only: no block barrier below
-    const int L = mb.L, ld = mb.ld, ldi = mb.ldi;
+    const int L = mb.L, k0 = lane * K;
     const TC dtc = cv<TC>(dt), cm = cv<TC>(cmax);
-    const size_t row = (size_t)i * ld, irow = (size_t)i * ldi;
-    // start layer mass of the vertical step: the end of the horizontal one
-    const typename Vec2<TC>::T *DV = (const typename Vec2<TC>::T *)mb.DV;
-    const float dtf = cv<float>(dt);
-    auto dstar = [&](int kk) -> TC { return (TC)end_mass(DV[row + kk], dt, dtf); };
-    // interface j between layers j-1 (above) and j (below), with those
-    // layers' start masses: explicit and implicit shares
-    auto split = [&](int j, TC above, TC below, TC &me, TC &mi) {
-        const TC Mj = (j > 0 && j < L) ? cv<TC>(mb.Mv[irow + j]) : (TC)0;
-        me = mi = (TC)0;
-        if (Mj != (TC)0) {
-            const TC cour = fabs(Mj) * dtc / (Mj > (TC)0 ? above : below);
-            const TC f = cour <= cm ? (TC)1 : cm / cour;
-            me = f * Mj;
-            mi = Mj - me;
-        }
-    };
-    TC dps[kVertR], met[kVertR], mit[kVertR], meb[kVertR], mib[kVertR], a[kVertR], b[kVertR], c[kVertR];
-    bool implicit = false;
+    const size_t row = (size_t)i * mb.ld + k0, irow = (size_t)i * mb.ldi + k0;
+    constexpr unsigned kAllLanes = 0xffffffffu;
+    // a lane's levels as one vector (VEC: whole vectors, aligned), else one by one
+    auto load = [&](const auto *p, auto (&o)[K]) {
 #pragma unroll
-    for (int r = 0; r < kVertR; r++) {
-        const int k = lane + 32 * r;
-        dps[r] = met[r] = mit[r] = meb[r] = mib[r] = a[r] = c[r] = (TC)0;
-        b[r] = (TC)1;
-        if (k < L) {
-            const TC d0 = dstar(k);
-            const TC dm = k > 0 ? dstar(k - 1) : (TC)0, dp = k + 1 < L ? dstar(k + 1) : (TC)0;
-            dps[r] = d0;
-            split(k, dm, d0, met[r], mit[r]);
-            split(k + 1, d0, dp, meb[r], mib[r]);
-            const TC Mt = met[r] + mit[r], Mb = meb[r] + mib[r];
-            const TC dpn = d0 - dtc * (Mb - Mt);
-            a[r] = -dtc * fmax_((TC)0, mit[r]);
-            b[r] = dpn + dtc * (fmax_((TC)0, mib[r]) - fmin_((TC)0, mit[r]));
-            c[r] = dtc * fmin_((TC)0, mib[r]);
-            implicit |= (mit[r] != (TC)0) | (mib[r] != (TC)0);
-        }
-    }
-    implicit = __any_sync(0xffffffffu, implicit);
-    TC rb[kVertR];
-#pragma unroll
-    for (int r = 0; r < kVertR; r++) rb[r] = vinv(b[r]);
-    bool bad = false;
-    for (int t = 0; t < mb.T; t++) {
-        TQ *qt = (TQ *)mb.q + (size_t)t * mb.qs + row;
-        TC rhs[kVertR];
-#pragma unroll
-        for (int r = 0; r < kVertR; r++) {
-            const int k = lane + 32 * r;
-            rhs[r] = (TC)0;
-            if (k < L) {
-                const TC qk = (TC)qt[k];
-                const TC qm = k > 0 ? (TC)qt[k - 1] : (TC)0, qp = k + 1 < L ? (TC)qt[k + 1] : (TC)0;
-                const TC Mt = met[r] + mit[r], Mb = meb[r] + mib[r];
-                const TC q_top = Mt > (TC)0 ? qm : qk;
-                const TC q_bot = Mb > (TC)0 ? qk : qp;
-                rhs[r] = dps[r] * qk - dtc * (meb[r] * q_bot - met[r] * q_top);
-            }
-        }
-        __syncwarp();   // every lane has read the column before any lane writes it
-        if (!implicit) {
-#pragma unroll
-            for (int r = 0; r < kVertR; r++) {
-                const int k = lane + 32 * r;
-                if (k < L) {
-                    const TC x = rhs[r] * rb[r];
-                    bad |= !isfinite(x);
-                    qt[k] = (TQ)x;
-                }
-            }
+        for (int r = 0; r < K; r++) o[r] = 0;
+        if constexpr (VEC) {
+            if (k0 < L) ldv_own<K>(p, o);
         } else {
 #pragma unroll
-            for (int r = 0; r < kVertR; r++) {
-                const int k = lane + 32 * r;
-                if (k < L) {
-                    sA[warp][k] = a[r];
-                    sB[warp][k] = b[r];
-                    sC[warp][k] = c[r];
-                    sD[warp][k] = rhs[r];
-                }
-            }
-            __syncwarp();
-            if (lane == 0) {
-                // Thomas sweep (forward elimination into sC / sD, back
-                // substitution into sD), the arithmetic of k_tr_vertical
-                for (int k = 0; k < L; k++) {
-                    const TC rden = vinv(k == 0 ? sB[warp][k] : sB[warp][k] - sA[warp][k] * sC[warp][k - 1]);
-                    const TC cpk = sC[warp][k] * rden;
-                    sD[warp][k] = (k == 0 ? sD[warp][k] : sD[warp][k] - sA[warp][k] * sD[warp][k - 1]) * rden;
-                    sC[warp][k] = cpk;
-                }
-                TC qb = (TC)0;
-                for (int k = L - 1; k >= 0; k--) {
-                    qb = (k == L - 1) ? sD[warp][k] : sD[warp][k] - sC[warp][k] * qb;
-                    sD[warp][k] = qb;
-                }
-            }
-            __syncwarp();
+            for (int r = 0; r < K; r++)
+                if (k0 + r < L) o[r] = p[r];
+        }
+    };
+    // start layer mass of the vertical step (the end of the horizontal one),
+    // that of the layer above the lane's first, interface fluxes
+    TC dps[K], Mt[K];
+    const float dtf = cv<float>(dt);
+    {
+        const typename Vec2<TC>::T *DV = (const typename Vec2<TC>::T *)mb.DV + row;
 #pragma unroll
-            for (int r = 0; r < kVertR; r++) {
-                const int k = lane + 32 * r;
-                if (k < L) {
-                    const TC x = sD[warp][k];
-                    bad |= !isfinite(x);
-                    qt[k] = (TQ)x;
-                }
+        for (int r = 0; r < K; r++) {
+            const int k = k0 + r;
+            dps[r] = (TC)1;
+            Mt[r] = (TC)0;
+            if (k < L) {
+                dps[r] = (TC)end_mass(DV[r], dt, dtf);
+                if (k > 0) Mt[r] = cv<TC>(mb.Mv[irow + r]);
             }
-            __syncwarp();   // the next tracer reuses the rows
+        }
+    }
+    const TC above0 = __shfl_up_sync(kAllLanes, dps[K - 1], 1);
+    // dt times the explicit and implicit shares of the flux at the lane's
+    // interfaces; bit r of up: its donor is the layer above
+    TC me[K], mi[K];
+    unsigned up = 0;
+    bool implicit = false;
+#pragma unroll
+    for (int r = 0; r < K; r++) {
+        me[r] = dtc * Mt[r];
+        mi[r] = (TC)0;
+        if (pos(Mt[r])) up |= 1u << r;
+        const TC donor = (up >> r) & 1u ? (r ? dps[r - 1] : above0) : dps[r];
+        if (nonzero(Mt[r]) && !le_num(abs_num(me[r]), cm * donor)) {
+            const TC cour = fabs(Mt[r]) * dtc / donor;
+            const TC f = cour <= cm ? (TC)1 : cm / cour;
+            const TC e = f * Mt[r];
+            mi[r] = dtc * (Mt[r] - e);
+            me[r] = dtc * e;
+            implicit |= mi[r] != (TC)0;
+        }
+    }
+    implicit = __any_sync(kAllLanes, implicit);
+    // shares at the interface below the lane's last layer (none at the ground)
+    TC meb = __shfl_down_sync(kAllLanes, me[0], 1), mib = (TC)0;
+    unsigned upb = __shfl_down_sync(kAllLanes, up, 1);
+    if (implicit) mib = __shfl_down_sync(kAllLanes, mi[0], 1);
+    if (lane == 31) {
+        meb = mib = (TC)0;
+        upb = 0;
+    }
+    TC rb[K];
+#pragma unroll
+    for (int r = 0; r < K; r++) {
+        const TC et = me[r], eb = r + 1 < K ? me[(r + 1) % K] : meb;
+        TC b = dps[r] - (eb - et);
+        if (implicit) {
+            const TC it = mi[r], ib = r + 1 < K ? mi[(r + 1) % K] : mib;
+            b = dps[r] - ((eb + ib) - (et + it)) + (fmax_((TC)0, ib) - fmin_((TC)0, it));
+            const int k = k0 + r;
+            sA[warp][k] = -fmax_((TC)0, it);
+            sB[warp][k] = b;
+            sC[warp][k] = fmin_((TC)0, ib);
+        }
+        rb[r] = vinv(b);
+    }
+    bool bad = false;
+    for (int tb = 0; tb < mb.T; tb += kVertT) {
+        TC q[kVertT][K];
+#pragma unroll
+        for (int a = 0; a < kVertT; a++)
+            if (tb + a < mb.T) load((const TQ *)mb.q + (size_t)(tb + a) * mb.qs + row, q[a]);
+#pragma unroll
+        for (int a = 0; a < kVertT; a++) {
+            if (tb + a >= mb.T) break;
+            TQ *qt = (TQ *)mb.q + (size_t)(tb + a) * mb.qs + row;
+            const TC qm = __shfl_up_sync(kAllLanes, q[a][K - 1], 1), qp = __shfl_down_sync(kAllLanes, q[a][0], 1);
+            TC x[K], fl = me[0] * ((up & 1u) ? qm : q[a][0]);
+            // the lane's last interface: the flux of the next lane's first
+            const TC flb = meb * ((upb & 1u) ? q[a][K - 1] : qp);
+#pragma unroll
+            for (int r = 0; r < K; r++) {
+                const TC fb = r + 1 < K ? me[(r + 1) % K] * ((up >> (r + 1)) & 1u ? q[a][r] : q[a][(r + 1) % K]) : flb;
+                x[r] = dps[r] * q[a][r] - (fb - fl);
+                fl = fb;
+            }
+            if (!implicit) {
+#pragma unroll
+                for (int r = 0; r < K; r++) x[r] *= rb[r];
+            } else {
+#pragma unroll
+                for (int r = 0; r < K; r++) sD[warp][k0 + r] = x[r];
+                __syncwarp();
+                if (lane == 0) {
+                    // Thomas sweep: forward elimination into sE and sD, back
+                    // substitution into sD
+                    TC cpk = (TC)0, dk = (TC)0;
+                    for (int k = 0; k < L; k++) {
+                        const TC ak = sA[warp][k];
+                        const TC rden = vinv(k == 0 ? sB[warp][k] : sB[warp][k] - ak * cpk);
+                        cpk = sC[warp][k] * rden;
+                        dk = (k == 0 ? sD[warp][k] : sD[warp][k] - ak * dk) * rden;
+                        sE[warp][k] = cpk;
+                        sD[warp][k] = dk;
+                    }
+                    TC qb = (TC)0;
+                    for (int k = L - 1; k >= 0; k--) {
+                        qb = (k == L - 1) ? sD[warp][k] : sD[warp][k] - sE[warp][k] * qb;
+                        sD[warp][k] = qb;
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < K; r++) x[r] = sD[warp][k0 + r];
+                __syncwarp();   // the next tracer reuses the rows
+            }
+#pragma unroll
+            for (int r = 0; r < K; r++) bad |= k0 + r < L && !isfinite(x[r]);
+            if constexpr (VEC) {
+                if (k0 < L) stv<K>(qt, x);
+            } else {
+#pragma unroll
+                for (int r = 0; r < K; r++)
+                    if (k0 + r < L) qt[r] = (TQ)x[r];
+            }
         }
     }
     if (bad) atomicOr(status, GRIST_FLAG_NONFINITE);
@@ -1730,14 +1770,18 @@ int enqueue_step(grist_mesh_s *h, TracerCtx *c, const Batch &B, cudaStream_t st)
     for (int j = 0; j < B.nm; j++) {
         if (!hm[j].Mv) continue;
         const unsigned gv = grid_for(m.nC, kVertWarps);
-        if (hm[j].L <= 64)
+        const int K = (hm[j].L + 31) / 32;
+        const bool vec = hm[j].L % K == 0 && hm[j].ld % K == 0 && (uintptr_t)hm[j].q % std::min<size_t>(16, K * sizeof(TQ)) == 0;
+        auto go = [&](auto kern) {
             GRIST_LAUNCH(h, sizeof(TC) == 4 ? "k_tr_vertical/mix" : "k_tr_vertical/fp64", st,
-                         (k_tr_vertical<TQ, TC, 2><<<gv, kVertWarps * 32, 0, st>>>(m, hm[j], B.dt, B.cmax,
-                                                                                   status_word(h))));
-        else
-            GRIST_LAUNCH(h, sizeof(TC) == 4 ? "k_tr_vertical/mix" : "k_tr_vertical/fp64", st,
-                         (k_tr_vertical<TQ, TC, kVertMaxL / 32><<<gv, kVertWarps * 32, 0, st>>>(
-                             m, hm[j], B.dt, B.cmax, status_word(h))));
+                         (kern<<<gv, kVertWarps * 32, 0, st>>>(m, hm[j], B.dt, B.cmax, status_word(h))));
+        };
+        if (K == 1) go(k_tr_vertical<TQ, TC, 1, false>);
+        else if (K == 2 && vec) go(k_tr_vertical<TQ, TC, 2, true>);
+        else if (K == 2) go(k_tr_vertical<TQ, TC, 2, false>);
+        else if (K == 3) go(k_tr_vertical<TQ, TC, 3, false>);
+        else if (vec) go(k_tr_vertical<TQ, TC, 4, true>);
+        else go(k_tr_vertical<TQ, TC, 4, false>);
     }
     return cudaGetLastError() == cudaSuccess ? GRIST_OK : GRIST_ECUDA;
 }

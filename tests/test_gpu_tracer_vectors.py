@@ -61,3 +61,33 @@ def test_every_width_equals_single_levels(mesh_cache, prec, limiter, beta, ring,
     for a, b in zip(*got):
         assert float((a - b).abs().max()) <= tol * float(a.abs().max())
     mesh.close()
+
+
+@pytest.mark.parametrize("prec", ["mix", "fp64"])
+@pytest.mark.parametrize("L,ld", [(2, 2), (31, 31), (32, 32), (33, 33), (60, 60), (60, 61), (64, 64), (65, 66), (96, 96),
+                                  (97, 97), (128, 128), (127, 128)])
+@pytest.mark.parametrize("cmax,courant", [(0.0, 6.0), (0.5, 6.0), (float("inf"), 0.4)])
+def test_vertical_layouts_against_the_oracle(mesh_cache, prec, L, ld, cmax, courant):
+    """Lanes hold 1 to 4 consecutive levels, as vectors or one by one; more
+    tracers than one group of loads.  Column fluxes, and so the bounds, of the
+    other vertical tests (no layer loses more than about half its mass)."""
+    import oracle as O
+    import torch
+    import paper_2404_08849_gb300 as G
+    from test_gpu_vertical import _column_flux, _member as vertical_member
+    m = mesh_cache(3)
+    mesh = G.Mesh(m)
+    rng = np.random.default_rng(L)
+    T, dt = 5, 400.0
+    dpi = rng.uniform(600, 1200, (m["n_cells"], L))
+    M = _column_flux(rng, m["n_cells"], L, dt, 600.0, courant)
+    M[::3] = 0.0
+    q = rng.uniform(0.1, 1.0, (T, m["n_cells"], L))
+    mb = vertical_member(mesh, q, dpi, np.zeros((m["n_edges"], L)), M, prec, ld, ld + 1)
+    mesh.tracer_step([mb], dt, prec=prec, vertical_courant_max=cmax)
+    torch.cuda.synchronize()
+    ref = O.tracer_vertical_step(q, dpi, M, dt, cmax)
+    got = mesh.from_internal(mb["q"].double().cpu().numpy()[..., :L], "cell", 1)
+    assert O.max_rel_diff(got, ref) <= (1e-12 if prec == "fp64" else 2e-5)
+    assert mesh.last_status() == 0
+    mesh.close()
