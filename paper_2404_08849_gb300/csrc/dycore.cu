@@ -105,7 +105,7 @@ __device__ __forceinline__ double col_reduce(double part) {
 // executing the call.
 struct Binom {
     double c[10];
-    float f[6];   // the same coefficients in binary32 (GRIST_MIX_DF increments)
+    float f[10];   // the same coefficients in binary32
 };
 
 template <int N> __device__ __forceinline__ double horner(double x, const Binom &B) {
@@ -128,11 +128,43 @@ __device__ __forceinline__ double pow1p_near0(double x, double g, const Binom &B
     return horner<10>(x, B);
 }
 
+// The same with the last terms, from the M-th on, where |x|^M <= 2^-30, summed
+// by Horner's rule in binary32: their rounding, 2^-24 of them, is below 2^-53
+// of the result, and 2, 3, 4 or 6 FP64 instructions do for |x| < 2^-15,
+// 2^-11, 2^-8, 2^-6 where all terms in FP64 take 3, 5, 7 or 9.  For the FP64
+// policy and the hydrostatic core; in the mixed policies the NH column state
+// keeps the bits of the form above (an ulp of phi moves the binary32
+// advection of the next stage by whole roundings).
+__device__ __forceinline__ double f2d_normal(float f) {   // a normal number or zero
+    const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+    const uint32_t hi = a < 0x00800000u ? 0u : (a >> 3) + 0x38000000u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(a << 29));
+}
+template <int M, int N> __device__ __forceinline__ double horner_tail(double x, const Binom &B) {
+    const float xf = d2f_trunc(x);
+    float t = B.f[N - 1];
+#pragma unroll
+    for (int n = N - 2; n >= M; n--) t = fmaf(t, xf, B.f[n]);
+    double s = f2d_normal(t);
+#pragma unroll
+    for (int n = M - 1; n >= 0; n--) s = fma(s, x, B.c[n]);
+    return s;
+}
+__device__ __forceinline__ double pow1p_tail(double x, double g, const Binom &B, unsigned mask) {
+    const unsigned hx = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    const unsigned hm = __reduce_max_sync(mask, hx);
+    if (hm < 0x3f000000u) return horner_tail<2, 4>(x, B);    // |x| < 2^-15
+    if (hm < 0x3f400000u) return horner_tail<3, 6>(x, B);    // 2^-11
+    if (hm < 0x3f700000u) return horner_tail<4, 8>(x, B);    // 2^-8
+    if (hx > 0x3f900000u || (hx == 0x3f900000u && __double2loint(x) != 0)) return pow(1.0 + x, g);
+    return horner_tail<6, 10>(x, B);
+}
+
 Binom binomial(double g) {
     Binom b;
     b.c[0] = 1.0;
     for (int n = 1; n < 10; n++) b.c[n] = b.c[n - 1] * (g - (n - 1)) / n;
-    for (int n = 0; n < 6; n++) b.f[n] = (float)b.c[n];
+    for (int n = 0; n < 10; n++) b.f[n] = (float)b.c[n];
     return b;
 }
 
@@ -163,6 +195,10 @@ __device__ __forceinline__ double scale_near1_df(double p, double x, double g, c
 // mass change cancels to round-off).  In the final stage fscale times the
 // flux is accumulated for the tracer solver (Sec. 2.3: single computed,
 // saved double).
+// Whether the column solve takes the short forms (one product for the t^n
+// reference, series tails in binary32): the FP64 policy; see horner_tail.
+template <class P> constexpr bool solve_short() { return sizeof(typename P::TA) == 8 && !P::EMU; }
+
 template <class P>
 __global__ void k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
                             const typename P::TU *__restrict__ u_s, typename P::TM *__restrict__ F,
@@ -222,7 +258,10 @@ __global__ void k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
 // update, 1/(ps - pi_top)) runs one cell per lane, then the warp walks its
 // cells with the lanes over levels: layer divergence D_k (mass-flux type),
 // vertical mass flux M_{k+1/2} = -B_{k+1/2} dps/dt - sum_{l<=k} D_l by a
-// warp scan, theta = (dpi theta)/dpi of the stage input for Eq. 4.
+// warp scan, theta = (dpi theta)/dpi of the stage input for Eq. 4.  In the
+// first stage of the NH core also the t^n state that the column solve's
+// equation of state is taken relative to: 1/(dpi theta) and dphi, or their
+// product (solve_short).
 template <class P>
 __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict__ F,
                            const double *__restrict__ Fcol, const double *__restrict__ ps_s,
@@ -230,6 +269,7 @@ __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict_
                            const double *__restrict__ th_s, typename P::TA *__restrict__ theta,
                            double *__restrict__ Mv, double dts, double *__restrict__ dpi_out,
                            double *__restrict__ rdps_out, double *__restrict__ rth_out,
+                           double *__restrict__ dphi_out, const double *__restrict__ phi_n,
                            double *__restrict__ Macc, double fscale) {
     using TM = typename P::TM;
     using TA = typename P::TA;
@@ -271,7 +311,16 @@ __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict_
                 const size_t x = (size_t)i * d.ld + k;
                 theta[x] = emu<P::EMU>(cv<TA>(th_s[x] * ldg(d.rdB + k) * rdps), d.emu, GRIST_ROW_THETA);
                 if (dpi_out) dpi_out[x] = ldg(d.dB + k) * dps;
-                if (rth_out) rth_out[x] = rcp(th_s[x]);
+                if (rth_out) {
+                    const size_t y = (size_t)i * d.ldi + k;
+                    const double dphi = phi_n[y] - phi_n[y + 1];
+                    if constexpr (solve_short<P>()) {
+                        rth_out[x] = dphi * rcp(th_s[x]);
+                    } else {
+                        rth_out[x] = rcp(th_s[x]);
+                        dphi_out[x] = dphi;
+                    }
+                }
             }
             // inclusive prefix of D over the chunk, carried across chunks:
             // FP64 terms in FP64, FP32 terms in compensated FP32
@@ -452,7 +501,7 @@ __global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const doubl
             double e;
             if (tabled) {
                 const double2 r = ldg(row + k);
-                e = r.x * horner<8>(r.y * off, bk);
+                e = r.x * horner_tail<4, 8>(r.y * off, bk);
             } else {
                 e = d.rd * pow(pk / d.p0, d.kappa) / pk;
             }
@@ -797,11 +846,14 @@ __device__ __forceinline__ void stage_out(double *X, size_t S, int col0, int nco
     }
 }
 
-// Implicit part of Eqs. 6-7 and Eq. 9, one thread per column (a block is
-// one warp of 32 consecutive columns), FP64.  Column data moves through
-// shared memory in kSolveKC-level chunks (whole-sector global access).
+// Implicit part of Eqs. 6-7 and Eq. 9, FP64; two kernels with the same
+// arithmetic.  k_nh_solve: one thread per column, a block is one warp of 32
+// consecutive columns; column data moves through shared memory in
+// kSolveKC-level chunks (whole-sector global access).  k_nh_solve_block, below:
+// a block of 8 warps takes 32 columns.
 // Equation of state relative to the t^n state (1/th_r, phi_r, p_r):
-//   p** = p_r ((th dphi_r) / (th_r dphi**))^gamma     (pow1p_near0)
+//   p** = p_r ((th dphi_r) / (th_r dphi**))^gamma     (pow1p_near0; dphi_r
+//   of t^n is formed once per step)
 // linearised about phi**: p_k = p**_k - C_k (w_k - w_{k+1}),
 // C_k = gamma p**_k beta dt g / dphi**_k; tridiagonal rows for interior
 // interfaces j = 1..L-1 (w = 0 at top and ground),
@@ -812,13 +864,13 @@ __device__ __forceinline__ void stage_out(double *X, size_t S, int col0, int nco
 // Thomas algorithm; phi = phi** + beta dt g w; the full EOS then gives
 //   p = p** (dphi / dphi**)^(-gamma),  dphi = dphi** + beta dt g (w_k - w_{k+1});
 // finally alpha = dphi/dpi, layer phi and dp/dpi averaged to layers
-// (interface value 1 at top and bottom) for the momentum equation.  phi_out
-// may be phi_r and p may be p_r (the last stage writes the state in place):
-// each block reads all reference values of its columns before writing them.
-template <bool EMU, bool DF>
+// (interface value 1 at top and bottom) for the momentum equation.  p may be
+// p_r (the last stage writes the state in place): each block reads all
+// reference values of its columns before writing them.
+template <bool EMU, bool DF, bool SHORT>
 __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyPar d, const double *__restrict__ wst,
                                                  const double *__restrict__ phst, const double *__restrict__ th,
-                                                 const double *__restrict__ rth_r, const double *phi_r,
+                                                 const double *__restrict__ rth_r, const double *__restrict__ dphi_r,
                                                  const double *p_r, const double *__restrict__ ps, double dts,
                                                  double *w_out, double *phi_out, double *p, double *__restrict__ al,
                                                  double *__restrict__ phl, double *__restrict__ dpp, Binom bg_pos,
@@ -837,7 +889,7 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
     const double psg = dps * rcp(bg);   // 1/a_j = dBi_j psg
     const unsigned amask = __ballot_sync(0xffffffffu, act);
     double cp[kNHMax], dd[kNHMax], pst[kNHMax], rdf[kNHMax];
-    double ftop = act ? phst[(size_t)i * d.ldi] : 0.0, rtop = act ? phi_r[(size_t)i * d.ldi] : 0.0;
+    double ftop = act ? phst[(size_t)i * d.ldi] : 0.0;
     const double phi_top0 = ftop;
     double pst_prev = 0.0, C_prev = 0.0;
     // forward sweep
@@ -845,7 +897,7 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
         const int nk = min(kSolveKC, L - k0);
         __syncwarp();
         stage_in(phst, d.ldi, col0, ncol, k0 + 1, nk, sA + 0 * kStage);
-        stage_in(phi_r, d.ldi, col0, ncol, k0 + 1, nk, sA + 1 * kStage);
+        if (!SHORT) stage_in(dphi_r, d.ld, col0, ncol, k0, nk, sA + 1 * kStage);
         stage_in(th, d.ld, col0, ncol, k0, nk, sA + 2 * kStage);
         stage_in(rth_r, d.ld, col0, ncol, k0, nk, sA + 3 * kStage);
         stage_in(p_r, d.ld, col0, ncol, k0, nk, sA + 4 * kStage);
@@ -855,12 +907,14 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
             for (int kk = 0; kk < nk; kk++) {
                 const int j = k0 + kk;
                 const int o = kk * kRow + lane;
-                const double fbot = sA[0 * kStage + o], rbot = sA[1 * kStage + o];
+                const double fbot = sA[0 * kStage + o];
                 const double rdfj = rcp_nr(ftop - fbot);
                 // x = th dphi_r / (th_r dphi**) - 1, the ratio's offset from 1
-                const double x = fma(sA[2 * kStage + o] * sA[3 * kStage + o], (rtop - rbot) * rdfj, -1.0);
-                const double pstj = DF ? scale_near1_df(sA[4 * kStage + o], x, d.gamma, bg_pos)
-                                       : sA[4 * kStage + o] * pow1p_near0(x, d.gamma, bg_pos, amask);
+                const double tr = sA[2 * kStage + o] * sA[3 * kStage + o];
+                const double x = SHORT ? fma(tr, rdfj, -1.0) : fma(tr, sA[1 * kStage + o] * rdfj, -1.0);
+                const double pstj = DF      ? scale_near1_df(sA[4 * kStage + o], x, d.gamma, bg_pos)
+                                    : SHORT ? sA[4 * kStage + o] * pow1p_tail(x, d.gamma, bg_pos, amask)
+                                            : sA[4 * kStage + o] * pow1p_near0(x, d.gamma, bg_pos, amask);
                 pst[j] = pstj;
                 rdf[j] = rdfj;
                 const double C = gbg * pstj * rdfj;
@@ -886,7 +940,6 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
                 pst_prev = pstj;
                 C_prev = C;
                 ftop = fbot;
-                rtop = rbot;
             }
         }
     }
@@ -928,8 +981,9 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
                 const double w_bot = (kk + 1 < nk) ? sA[1 * kStage + o + kRow] : sA[6 * kStage + lane];
                 const double phi_bot = (k + 1 < L) ? fma(bg, w_bot, sA[o]) : ldg(d.phis + i);
                 const double xk = bg * (w_top - w_bot) * rdf[k];
-                const double pk = DF ? scale_near1_df(pst[k], xk, -d.gamma, bg_neg)
-                                     : pst[k] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
+                const double pk = DF      ? scale_near1_df(pst[k], xk, -d.gamma, bg_neg)
+                                  : SHORT ? pst[k] * pow1p_tail(xk, -d.gamma, bg_neg, amask)
+                                          : pst[k] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
                 double hcur = 0.5;
                 if (k > 0) {
                     hcur = (pk - pprev) * (ldg(d.hrdBi + k) * rdps);
@@ -956,6 +1010,170 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
         stage_out(dpp, d.ld, col0, ncol, k0, nk - 1, sA + 5 * kStage);
     }
     if (act) dpp[(size_t)i * d.ld + L - 1] = emu<EMU>(htop + 0.5, d.emu, GRIST_ROW_EOS);
+}
+
+// The same solve by blocks of 8 warps and 32 columns, the column arrays in
+// shared memory ([level][33]).  Passes:
+//   A   lanes = columns, a warp per level: p**, 1/dphi**, C;
+//   B   Thomas sweep, one lane per column of one warp (on the scheduler
+//       blockIdx mod 8 picks, so that resident blocks' sweeps spread);
+//   C   lanes = columns, a warp per level: the new pressure;
+//   D   the block's threads over the flat (column, level) index, so the
+//       outputs are written as whole rows.
+// The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 40).
+// One warp for 32 columns needs about 24 blocks an SM to keep the pipe busy
+// (78 % then); with fewer columns than that the levels are the parallelism
+// left (solve_by_blocks has the figures).
+// SHORT: rth_r holds dphi_r / th_r and the series' tails are binary32.
+constexpr int kSolveWarps = 8;
+
+template <bool EMU, bool DF, bool SHORT>
+__global__ void __launch_bounds__(kSolveWarps * 32) k_nh_solve_block(
+    DevMesh m, DyPar d, LevelDiv Dv, const double *__restrict__ wst, const double *__restrict__ phst,
+    const double *__restrict__ th, const double *__restrict__ rth_r, const double *__restrict__ dphi_r,
+    const double *p_r, const double *__restrict__ ps, double dts, double *w_out, double *phi_out, double *p,
+    double *__restrict__ al, double *__restrict__ phl, double *__restrict__ dpp, Binom bg_pos, Binom bg_neg) {
+    extern __shared__ __align__(16) double sol[];
+    const int L = d.L;
+    double *sP = sol, *sD = sP + L * kRow, *sC = sD + L * kRow, *sW = sC + L * kRow;
+    __shared__ double s_rdps[kSolveCols], s_psg[kSolveCols];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int col0 = blockIdx.x * kSolveCols;
+    const int ncol = min(kSolveCols, m.nC - col0);
+    const bool act = lane < ncol;
+    const unsigned amask = __ballot_sync(0xffffffffu, act);
+    const double bg = d.beta * dts * d.g;
+    const double gbg = d.gamma * bg;
+    if (warp == 0 && act) {
+        const double dps = ps[col0 + lane] - d.pi_top;
+        s_rdps[lane] = rcp(dps);
+        s_psg[lane] = dps * rcp(bg);   // 1/a_j = dBi_j psg
+    }
+    // A
+    if (act) {
+        const size_t x0 = (size_t)(col0 + lane) * d.ld, y0 = (size_t)(col0 + lane) * d.ldi;
+        for (int k = warp; k < L; k += kSolveWarps) {
+            const double rdf = rcp_nr(phst[y0 + k] - phst[y0 + k + 1]);
+            const double pr = p_r[x0 + k], tr = ldg(th + x0 + k) * ldg(rth_r + x0 + k);
+            // th dphi_r / (th_r dphi**) - 1
+            const double x = SHORT ? fma(tr, rdf, -1.0) : fma(tr, ldg(dphi_r + x0 + k) * rdf, -1.0);
+            const double pst = DF      ? scale_near1_df(pr, x, d.gamma, bg_pos)
+                               : SHORT ? pr * pow1p_tail(x, d.gamma, bg_pos, amask)
+                                       : pr * pow1p_near0(x, d.gamma, bg_pos, amask);
+            const int o = k * kRow + lane;
+            sP[o] = pst;
+            sD[o] = rdf;
+            sC[o] = gbg * pst * rdf;
+            sW[o] = wst[y0 + k] - bg;
+        }
+    }
+    __syncthreads();
+    // B
+    if (warp == (int)(blockIdx.x % kSolveWarps) && act) {
+        const double psg = s_psg[lane];
+        double Cp = sC[lane], pp = sP[lane], cp = 0.0, dd = 0.0;
+        for (int j = 1; j < L; j++) {
+            const int o = j * kRow + lane;
+            const double C = sC[o], pj = sP[o];
+            // row j / a_j, as in k_nh_solve
+            const double sj = ldg(d.dBi + j) * psg;
+            const double b = sj + (Cp + C);
+            const double rhs = fma(sW[o], sj, pj - pp);
+            const double rden = rcp_nr(fma(Cp, cp, b));
+            cp = j == L - 1 ? -0.0 * rden : -C * rden;
+            dd = fma(Cp, dd, rhs) * rden;
+            sC[o] = cp;
+            sW[o] = dd;
+            Cp = C;
+            pp = pj;
+        }
+        double wn = 0.0;
+        for (int j = L - 1; j >= 1; j--) {
+            const int o = j * kRow + lane;
+            wn = fma(-sC[o], wn, sW[o]);
+            sW[o] = wn;
+        }
+        sW[lane] = 0.0;
+    }
+    __syncthreads();
+    // C
+    if (act) {
+        for (int k = warp; k < L; k += kSolveWarps) {
+            const int o = k * kRow + lane;
+            const double w_bot = k + 1 < L ? sW[o + kRow] : 0.0;
+            const double xk = bg * (sW[o] - w_bot) * sD[o];
+            sP[o] = DF      ? scale_near1_df(sP[o], xk, -d.gamma, bg_neg)
+                    : SHORT ? sP[o] * pow1p_tail(xk, -d.gamma, bg_neg, amask)
+                            : sP[o] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
+        }
+    }
+    __syncthreads();
+    // D: a warp takes 31 items and the one after them (the interface below)
+    const int items = ncol * L;
+    for (int base = warp * 31; base < items; base += kSolveWarps * 31) {
+        const int n = min(base + lane, items - 1);
+        int c, k;
+        split_index((uint32_t)n, Dv, c, k);
+        const size_t x = (size_t)(col0 + c) * d.ld + k, y = (size_t)(col0 + c) * d.ldi + k;
+        const int o = k * kRow + c;
+        const double rdps = s_rdps[c], pk = sP[o], w = sW[o];
+        const double phi_top = k > 0 ? fma(bg, w, phst[y]) : phst[y];
+        double phi_bot = __shfl_down_sync(0xffffffffu, phi_top, 1);
+        // halves of dp/dpi at the layer's interfaces (1 at top and ground)
+        const double hc = k > 0 ? (pk - sP[o - kRow]) * (ldg(d.hrdBi + k) * rdps) : 0.5;
+        double hb = __shfl_down_sync(0xffffffffu, hc, 1);
+        if (k == L - 1) {
+            hb = 0.5;
+            phi_bot = ldg(d.phis + col0 + c);
+        }
+        if (lane < 31 && base + lane < items) {
+            const double dphi = phi_top - phi_bot;
+            w_out[y] = w;
+            phi_out[y] = phi_top;
+            if (k == L - 1) {
+                w_out[y + 1] = 0.0;
+                phi_out[y + 1] = phi_bot;
+            }
+            p[x] = emu<EMU>(pk, d.emu, GRIST_ROW_EOS);
+            al[x] = emu<EMU>(dphi * (ldg(d.rdB + k) * rdps), d.emu, GRIST_ROW_EOS);
+            const double phm = fma(0.5, dphi, phi_bot);   // layer mean (phi_top + phi_bot)/2
+            phl[x] = DF ? pack_split(phm) : emu<EMU>(phm, d.emu, GRIST_ROW_EOS);
+            dpp[x] = emu<EMU>(hc + hb, d.emu, GRIST_ROW_EOS);
+        }
+    }
+}
+
+// Which form, by columns and levels.  Measured (us a launch, one warp / block,
+// 10,242, 40,962, 163,842 and 655,362 columns): 30 levels 99 / 52, 155 / 151,
+// 552 / 485, 1845 / 1828; 60 levels 195 / 97, 298 / 275, 1022 / 1026, 3519 /
+// 3811; 100 levels 355 / 303, 496 / 728, 1717 / 2387.  So the block form while
+// the one-warp form has less than a wave (24 resident blocks of 32 columns on
+// 152 SMs) or columns are short, where three blocks' arrays fit an SM (70
+// levels; with fewer blocks an SM waits through every pass); above 70 levels
+// only for a few blocks per SM in all.
+inline bool solve_by_blocks(int nC, int L) {
+    if (L > 70) return nC <= 152 * kSolveCols * 3;
+    return nC < 152 * kSolveCols * kSolveMinBlocks || L <= 40;
+}
+
+template <bool EMU, bool DF, bool SHORT>
+cudaError_t launch_solve(const DevMesh &m, const DyPar &d, LevelDiv Dv, const double *wst, const double *phst,
+                         const double *th, const double *rth, const double *dphi, const double *p_r, const double *ps,
+                         double dts, double *w_out, double *phi_out, double *p, double *al, double *phl, double *dpp,
+                         const Binom &bp, const Binom &bn, cudaStream_t st) {
+    const unsigned grid = grid_for(m.nC, kSolveCols);
+    if (solve_by_blocks(m.nC, d.L)) {
+        const int bytes = 4 * d.L * kRow * 8;
+        const cudaError_t e = cudaFuncSetAttribute(k_nh_solve_block<EMU, DF, SHORT>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        k_nh_solve_block<EMU, DF, SHORT><<<grid, kSolveWarps * 32, bytes, st>>>(
+            m, d, Dv, wst, phst, th, rth, dphi, p_r, ps, dts, w_out, phi_out, p, al, phl, dpp, bp, bn);
+    } else {
+        k_nh_solve<EMU, DF, SHORT><<<grid, kSolveCols, 0, st>>>(m, d, wst, phst, th, rth, dphi, p_r, ps, dts, w_out, phi_out, p,
+                                                         al, phl, dpp, bp, bn);
+    }
+    return cudaSuccess;
 }
 
 // Relative vorticity at the vertices (diagnostic): zeta_v = sum_j ccurl u,
@@ -1000,12 +1218,13 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const size_t o_theta = take(nCL * sizeof(TA)), o_Fth = take(nEL * sizeof(TA));
     const size_t o_p = take(nCL * 8), o_al = take(nCL * 8), o_phl = take(nCL * 8), o_dpp = take(nCL * 8);
     const size_t o_qv = take(nVL * sizeof(TA)), o_K = take(nCL * 8);
-    size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0;
+    size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0, o_dph = 0;
     const size_t o_ex = take(NH ? 0 : (size_t)kExnerBins * L * sizeof(double2));
     if (NH) {
         o_wA = take(nCI * 8); o_wB = take(nCI * 8); o_phA = take(nCI * 8); o_phB = take(nCI * 8);
         o_wst = take(nCI * 8); o_phst = take(nCI * 8); o_pn = take(nCL * 8); o_fw = take(nCI * 8);
         o_rth = take(nCL * 8);
+        o_dph = take(solve_short<P>() ? 0 : nCL * 8);
     }
     char *s = (char *)scratch(h, 1, off);
     if (!s) return GRIST_ENOMEM;
@@ -1060,14 +1279,15 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     double *K = (double *)(s + o_K);
     double *wA = (double *)(s + o_wA), *wB = (double *)(s + o_wB), *phA = (double *)(s + o_phA),
            *phB = (double *)(s + o_phB), *wst = (double *)(s + o_wst), *phst = (double *)(s + o_phst),
-           *pn = (double *)(s + o_pn), *fwn = (double *)(s + o_fw), *rthn = (double *)(s + o_rth);
+           *pn = (double *)(s + o_pn), *fwn = (double *)(s + o_fw), *rthn = (double *)(s + o_rth),
+           *dphn = (double *)(s + o_dph);
 
     TU *u = (TU *)S->u;
     uint32_t *status = status_word(h);
     const LevelDiv DL = make_div((uint32_t)L), DI = make_div((uint32_t)(L + 1)), DH = make_div((uint32_t)(L + 1) / 2);
     const unsigned gC = grid_for((long long)m.nC * L, kBlock), gE = grid_for((long long)m.nE * L, kBlock),
                    gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for((long long)m.nC * 32, kBlock),
-                   gI = grid_for((long long)m.nC * (L + 1), kBlock), gSolve = grid_for(m.nC, kSolveCols),
+                   gI = grid_for((long long)m.nC * (L + 1), kBlock),
                    gVx = grid_for(m.nV, kBlock), gE32 = grid_for((long long)m.nE + 31, kBlock),
                    gC32 = grid_for((long long)m.nC + 31, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
                    gCH = grid_for((long long)m.nC * DH.d, kBlock), gVH = grid_for((long long)m.nV * DH.d, kBlock);
@@ -1116,7 +1336,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             m, d, ps_in, u_in, F, s3 == 2 ? S->mass_flux_accum : nullptr, ascale, rsum, fcol));
         GRIST_LAUNCH(h, PN("k_mass_col"), st, k_mass_col<P><<<gC32, kBlock, 0, st>>>(
             m, d, F, fcol, ps_in, psN, ps_outs[s3], th_in, theta, Mv, h3, s3 == 0 ? S->dpi_start : nullptr, rdps,
-            (NH && s3 == 0) ? rthn : nullptr, s3 == 2 ? S->vmass_flux_accum : nullptr, ascale));
+            (NH && s3 == 0) ? rthn : nullptr, dphn, S->phi, s3 == 2 ? S->vmass_flux_accum : nullptr, ascale));
         GRIST_LAUNCH(h, PN("k_theta_flux"), st, k_theta_flux<P><<<gEH, kBlock, 0, st>>>(m, d, DH, F, theta, Fth));
         GRIST_LAUNCH(h, PN("k_theta_update"), st, k_theta_update<P><<<gCH, kBlock, 0, st>>>(
             m, d, DH, Fth, theta, Mv, S->dpi_theta, th_outs[s3], h3));
@@ -1127,9 +1347,11 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             else
                 GRIST_LAUNCH(h, PN("k_nh_explicit"), st, k_nh_explicit<P, false><<<gI, kBlock, 0, st>>>(
                     m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
-            GRIST_LAUNCH(h, PN("k_nh_solve"), st, k_nh_solve<P::EMU, P::DF><<<gSolve, kSolveCols, 0, st>>>(
-                m, d, wst, phst, th_outs[s3], rthn, S->phi, p_n, ps_outs[s3], h3, w_outs[s3],
-                phi_outs[s3], p_outs[s3], alp, phl, dpp, bpos, bneg));
+            cudaError_t se = cudaSuccess;
+            GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, solve_short<P>()>(
+                m, d, DL, wst, phst, th_outs[s3], rthn, dphn, p_n, ps_outs[s3], h3, w_outs[s3], phi_outs[s3], p_outs[s3],
+                alp, phl, dpp, bpos, bneg, st)));
+            if (se != cudaSuccess) return GRIST_ECUDA;
         } else {
             GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF><<<gW, kBlock, 0, st>>>(
                 m, d, ex, bkap, ps_outs[s3], th_outs[s3], p, alp, phl));
