@@ -17,6 +17,7 @@
 // once per level (1/dB), and the equation of state inside a stage is
 // evaluated relative to the stage-input state (see pow1p_near0).
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -28,6 +29,12 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr int kNHMax = 128;  // levels supported by the column solver
+// Edges or cells that a warp of the mass kernels walks.  The per-entity FP64
+// scalars run one entity per lane, so fewer entities waste more of the FP64
+// pipe; but with 32 a 10,242-cell mesh has two warps an SM.  8 against 32, us a
+// launch: level 5, 30 levels, mass_col 67 / 24, mass_edge 38 / 16; level 8, 60
+// levels, 699 / 696 and 595 / 306.
+constexpr int kMassGroup = 8;
 
 struct DyPar {
     int L, ld, ldi;
@@ -85,12 +92,58 @@ __device__ __forceinline__ F2 f2_shfl_up(F2 v, int o) {
     return F2{__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
 }
 
-// Column sum of a level-indexed value over the warp's lanes: FP64 terms
-// are added in FP64; FP32 terms in compensated FP32, converted once.
-__device__ __forceinline__ double col_reduce(double part) {
+// Sums over a warp's lanes of G values per lane (one column sum per entity),
+// lane l ending with the sum of entity l mod G.  The sums add in the order of
+// a butterfly (xor 16, 8, 4, 2, 1, own value first) that each entity would
+// do for itself, but once a step tells two entities apart a lane keeps the
+// partial sum of one and sends that of the other: 31 additions for 32
+// entities instead of 5 each.  Entities are visited in bit-reversed order, so
+// at most log2(G) partial sums are held.  leaf(j): entity j's value in this
+// lane.  FP64 terms are added in FP64, FP32 terms in compensated FP32.
+__device__ __forceinline__ double lane_add(double a, double b) { return a + b; }
+__device__ __forceinline__ F2 lane_add(F2 a, F2 b) { return f2_add(a, b); }
+__device__ __forceinline__ double lane_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ F2 lane_xor(F2 v, int o) { return f2_shfl_xor(v, o); }
+__device__ __forceinline__ double lane_pick(bool c, double a, double b) { return c ? a : b; }
+__device__ __forceinline__ F2 lane_pick(bool c, F2 a, F2 b) { return F2{c ? a.hi : b.hi, c ? a.lo : b.lo}; }
+
+// Pieces of the column prefix (k_mass_col): lane_carry adds the earlier chunks'
+// total, lane_next is the total for the next chunk.
+template <class S> __device__ __forceinline__ S lane_zero();
+template <> __device__ __forceinline__ double lane_zero<double>() { return 0.0; }
+template <> __device__ __forceinline__ F2 lane_zero<F2>() { return F2{0.f, 0.f}; }
+template <class S> __device__ __forceinline__ S lane_value(double x) {
+    if constexpr (sizeof(S) == 8 && std::is_same<S, double>::value) return x;
+    else return F2{cv<float>(x), 0.f};
+}
+template <class S> __device__ __forceinline__ S lane_value(float x) {
+    if constexpr (std::is_same<S, double>::value) return (double)x;
+    else return F2{x, 0.f};
+}
+__device__ __forceinline__ double lane_up(double v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ F2 lane_up(F2 v, int o) { return f2_shfl_up(v, o); }
+__device__ __forceinline__ double lane_carry(double run, double v) { return run + v; }
+__device__ __forceinline__ F2 lane_carry(F2 run, F2 v) { return f2_add(v, run); }
+__device__ __forceinline__ double lane_total(double v) { return v; }
+__device__ __forceinline__ double lane_total(F2 v) { return f2d(v.hi) + f2d(v.lo); }
+__device__ __forceinline__ double lane_next(double run, double v, double) { return run + __shfl_sync(0xffffffffu, v, 31); }
+__device__ __forceinline__ F2 lane_next(F2, F2, F2 pre) {
+    return F2{__shfl_sync(0xffffffffu, pre.hi, 31), __shfl_sync(0xffffffffu, pre.lo, 31)};
+}
+
+template <int G, int O, class Leaf>   // O: the step that tells this call's two halves apart; 2 G > O >= 1
+__device__ __forceinline__ auto entity_sums(Leaf &leaf, int j, int lane) {
+    if constexpr (O >= G) {
+        auto v = leaf(j);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    return part;
+        for (int o = 16; o >= G; o >>= 1) v = lane_add(v, lane_xor(v, o));
+        return v;
+    } else {
+        const auto a = entity_sums<G, 2 * O>(leaf, j, lane);
+        const auto b = entity_sums<G, 2 * O>(leaf, j | O, lane);
+        const bool up = (lane & O) != 0;
+        return lane_add(lane_pick(up, b, a), lane_xor(lane_pick(up, a, b), O));
+    }
 }
 
 // r^g for a ratio r close to 1 by the binomial series
@@ -184,32 +237,35 @@ __device__ __forceinline__ double scale_near1_df(double p, double x, double g, c
 }
 
 // ---------------------------------------------------------------------------
-// Eq. 3: mass flux at edges F = dpi_e u, dpi_e = mean of the two cells'
-// layer mass = dB_k (ps1 + ps2 - 2 pi_top)/2.  One warp takes 32 edges: the
-// per-edge FP64 work (column factor, the reciprocal 1/(ps1 + ps2 - 2 pi_top)
-// for the momentum equation) runs one edge per lane - an FP64 instruction
-// costs the FP64 pipe a full warp slot however few lanes are active - then
-// the warp walks its edges with the lanes over levels, forming the product
-// in the mass-flux type and the edge's column sum sum_k F_k by a fixed
-// butterfly (both cells of the edge later use the same value, so the global
-// mass change cancels to round-off).  In the final stage fscale times the
-// flux is accumulated for the tracer solver (Sec. 2.3: single computed,
-// saved double).
 // Whether the column solve takes the short forms (one product for the t^n
 // reference, series tails in binary32): the FP64 policy; see horner_tail.
 template <class P> constexpr bool solve_short() { return sizeof(typename P::TA) == 8 && !P::EMU; }
 
+// Eq. 3: mass flux at edges F = dpi_e u, dpi_e = mean of the two cells'
+// layer mass = dB_k (ps1 + ps2 - 2 pi_top)/2.  One warp takes G edges: the
+// per-edge FP64 work (column factor, the reciprocal 1/(ps1 + ps2 - 2 pi_top)
+// for the momentum equation) runs one edge per lane - an FP64 instruction
+// costs the FP64 pipe a full warp slot however few lanes are active - then
+// the warp walks its edges with the lanes over levels, forming the product
+// in the mass-flux type and the edges' column sums sum_k F_k (entity_sums;
+// both cells of the edge later use the same value, so the global mass change
+// cancels to round-off).  In the final stage fscale times the flux is
+// accumulated for the tracer solver (Sec. 2.3: single computed, saved double).
+// Against one edge at a time (its load, product and butterfly of five
+// compensated additions in turn, 32 edges a warp), mixed: level 8, 60 levels
+// 417 -> 306 us a launch (139 at the DRAM rate), level 5, 30 levels 34 -> 16.
 template <class P>
-__global__ void k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
+__global__ void __launch_bounds__(kBlock) k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
                             const typename P::TU *__restrict__ u_s, typename P::TM *__restrict__ F,
                             double *__restrict__ Facc, double fscale, double *__restrict__ rsum_e,
                             double *__restrict__ Fcol) {
     const bool scaled = fscale != 1.0;
     using TM = typename P::TM;
-    const int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
+    constexpr int G = kMassGroup;
+    const int e0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G;
     const int lane = threadIdx.x & 31;
     if (e0 >= m.nE) return;
-    const int ne = min(32, m.nE - e0);
+    const int ne = min(G, m.nE - e0);
     TM hs_l = 0;
     if (lane < ne) {
         const int2 c = ldg(m.coe + e0 + lane);
@@ -217,43 +273,53 @@ __global__ void k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
         hs_l = cv<TM>(0.5 * sum);
         rsum_e[e0 + lane] = 0.5 * rcp(sum);   // 1 / (2 dpi_e / dB)
     }
-    double col64 = 0.0;
-    float col_hi = 0.f, col_lo = 0.f;
-    for (int j = 0; j < ne; j++) {
-        const int e = e0 + j;
-        const TM hs = __shfl_sync(0xffffffffu, hs_l, j);
-        if (sizeof(TM) == 8) {
-            double col = 0.0;
-            for (int k = lane; k < d.L; k += 32) {
-                const size_t x = (size_t)e * d.ld + k;
-                const TM f = emu<P::EMU>((TM)ldg(d.dB + k) * hs * cv<TM>(u_s[x]), d.emu, GRIST_ROW_MASS_FLUX);
-                F[x] = f;
-                col += (double)f;
-                if (Facc) Facc[x] += scaled ? fscale * (double)f : (double)f;
-            }
-            col = col_reduce(col);
-            if (lane == j) col64 = col;
-        } else {
-            F2 col{0.f, 0.f};
-            for (int k = lane; k < d.L; k += 32) {
-                const size_t x = (size_t)e * d.ld + k;
-                const TM f = ldg(d.dBf + k) * hs * cv<TM>(u_s[x]);
-                F[x] = f;
-                col = f2_add(col, F2{cv<float>(f), 0.f});
-                if (Facc) Facc[x] += scaled ? fscale * cv<double>(f) : cv<double>(f);
-            }
+    // two 32-level chunks of all the warp's edges are loaded before the first
+    // is used; past the last edge its loads are repeated and nothing is stored
+    using Sum = typename std::conditional<sizeof(TM) == 8, double, F2>::type;
+    Sum part[G];
+    TM hs[G];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) col = f2_add(col, f2_shfl_xor(col, o));
-            if (lane == j) {
-                col_hi = col.hi;
-                col_lo = col.lo;
+    for (int j = 0; j < G; j++) {
+        part[j] = lane_zero<Sum>();
+        hs[j] = __shfl_sync(0xffffffffu, hs_l, j);
+    }
+    for (int k0 = lane; k0 < d.L; k0 += 64) {
+        const bool two = k0 + 32 < d.L;
+        typename P::TU u[G][2];
+#pragma unroll
+        for (int j = 0; j < G; j++) {
+            const size_t x = (size_t)(e0 + min(j, ne - 1)) * d.ld + k0;
+            u[j][0] = u_s[x];
+            u[j][1] = two ? u_s[x + 32] : (typename P::TU)0;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int k = k0 + 32 * h;
+            if (k >= d.L) break;
+            const TM dB = sizeof(TM) == 8 ? (TM)ldg(d.dB + k) : (TM)ldg(d.dBf + k);
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                if (j >= ne) break;
+                const size_t x = (size_t)(e0 + j) * d.ld + k;
+                const TM f = emu<P::EMU>(dB * hs[j] * cv<TM>(u[j][h]), d.emu, GRIST_ROW_MASS_FLUX);
+                F[x] = f;
+                part[j] = lane_add(part[j], lane_value<Sum>(f));
+                if (Facc) Facc[x] += scaled ? fscale * cv<double>(f) : cv<double>(f);
             }
         }
     }
-    if (lane < ne) Fcol[e0 + lane] = sizeof(TM) == 8 ? col64 : f2d(col_hi) + f2d(col_lo);
+    auto leaf = [&](int j) { return part[j]; };
+    // lane l ends with edge l mod G; the butterfly of edge j (counted from a
+    // multiple of 32) is the one that ends in lane j mod 32
+    const auto col = entity_sums<G, 1>(leaf, 0, lane);
+    const int at = e0 & 31;
+    if (lane >= at && lane < at + ne) {
+        if constexpr (sizeof(TM) == 8) Fcol[e0 + lane - at] = col;
+        else Fcol[e0 + lane - at] = f2d(col.hi) + f2d(col.lo);
+    }
 }
 
-// Eq. 3 column part.  One warp takes 32 cells; the per-cell FP64 work (the
+// Eq. 3 column part.  One warp takes G cells; the per-cell FP64 work (the
 // surface pressure tendency -sum_j s dv/A (column sum of edge j), its stage
 // update, 1/(ps - pi_top)) runs one cell per lane, then the warp walks its
 // cells with the lanes over levels: layer divergence D_k (mass-flux type),
@@ -262,8 +328,16 @@ __global__ void k_mass_edge(DevMesh m, DyPar d, const double *__restrict__ ps_s,
 // first stage of the NH core also the t^n state that the column solve's
 // equation of state is taken relative to: 1/(dpi theta) and dphi, or their
 // product (solve_short).
+//
+// The two 32-level chunks of a pair are loaded and scanned together (the scans
+// are independent until the carry is added), which hides half the shuffles'
+// latency.  The scan keeps the order of one 32-lane scan per chunk: M, and so
+// the mixed policies, keep their bits.  FP64 policy, level 7, 60 levels
+// 528 -> 399 us a launch; mixed, level 8 730 -> 696 (the correctly rounded
+// 1/(dpi theta) of the first stage holds the FP64 pipe 80 % there), level 6,
+// 30 levels 65 -> 40.
 template <class P>
-__global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict__ F,
+__global__ void __launch_bounds__(kBlock) k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict__ F,
                            const double *__restrict__ Fcol, const double *__restrict__ ps_s,
                            const double *__restrict__ ps_n, double *__restrict__ ps_out,
                            const double *__restrict__ th_s, typename P::TA *__restrict__ theta,
@@ -273,10 +347,11 @@ __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict_
                            double *__restrict__ Macc, double fscale) {
     using TM = typename P::TM;
     using TA = typename P::TA;
-    const int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
+    constexpr int G = kMassGroup;
+    const int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G;
     const int lane = threadIdx.x & 31;
     if (i0 >= m.nC) return;
-    const int nci = min(32, m.nC - i0);
+    const int nci = min(G, m.nC - i0);
     double pst_l = 0.0, dps_l = 0.0, rdps_l = 0.0;
     if (lane < nci) {
         const int i = i0 + lane;
@@ -290,6 +365,8 @@ __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict_
         Mv[(size_t)i * d.ldi + d.L] = 0.0;
     }
     const int nch = (d.L + 31) >> 5;
+    using Sum = typename std::conditional<sizeof(TM) == 8, double, F2>::type;
+#pragma unroll 1
     for (int c = 0; c < nci; c++) {
         const int i = i0 + c;
         const double pst = __shfl_sync(0xffffffffu, pst_l, c);
@@ -299,62 +376,61 @@ __global__ void k_mass_col(DevMesh m, DyPar d, const typename P::TM *__restrict_
         TM cw[GRIST_MAXE];
         load_row6(m.eoc8, i, eidx);
         load_row6(Coef<TM>::cdiv8(m), i, cw);
-        double run = 0.0;
-        F2 runf{0.f, 0.f};
-        for (int ch = 0; ch < nch; ch++) {
-            const int k = ch * 32 + lane;
-            TM s = 0;
-            if (k < d.L) {
+        Sum run = lane_zero<Sum>();
+        auto chunks = [&](auto count, int ch) {
+            constexpr int H = decltype(count)::value;
+            Sum v[H];
 #pragma unroll
-                for (int j = 0; j < GRIST_MAXE; j++) s += cw[j] * ldg(F + (size_t)eidx[j] * d.ld + k);
-                s = emu<P::EMU>(s, d.emu, GRIST_ROW_MASS_FLUX);
-                const size_t x = (size_t)i * d.ld + k;
-                theta[x] = emu<P::EMU>(cv<TA>(th_s[x] * ldg(d.rdB + k) * rdps), d.emu, GRIST_ROW_THETA);
-                if (dpi_out) dpi_out[x] = ldg(d.dB + k) * dps;
-                if (rth_out) {
-                    const size_t y = (size_t)i * d.ldi + k;
-                    const double dphi = phi_n[y] - phi_n[y + 1];
-                    if constexpr (solve_short<P>()) {
-                        rth_out[x] = dphi * rcp(th_s[x]);
-                    } else {
-                        rth_out[x] = rcp(th_s[x]);
-                        dphi_out[x] = dphi;
+            for (int h = 0; h < H; h++) {
+                const int k = (ch + h) * 32 + lane;
+                TM s = 0;
+                if (k < d.L) {
+#pragma unroll
+                    for (int j = 0; j < GRIST_MAXE; j++) s += cw[j] * ldg(F + (size_t)eidx[j] * d.ld + k);
+                    s = emu<P::EMU>(s, d.emu, GRIST_ROW_MASS_FLUX);
+                    const size_t x = (size_t)i * d.ld + k;
+                    theta[x] = emu<P::EMU>(cv<TA>(th_s[x] * ldg(d.rdB + k) * rdps), d.emu, GRIST_ROW_THETA);
+                    if (dpi_out) dpi_out[x] = ldg(d.dB + k) * dps;
+                    if (rth_out) {
+                        const size_t y = (size_t)i * d.ldi + k;
+                        const double dphi = phi_n[y] - phi_n[y + 1];
+                        if constexpr (solve_short<P>()) {
+                            rth_out[x] = dphi * rcp(th_s[x]);
+                        } else {
+                            rth_out[x] = rcp(th_s[x]);
+                            dphi_out[x] = dphi;
+                        }
                     }
                 }
+                v[h] = lane_value<Sum>(s);
             }
-            // inclusive prefix of D over the chunk, carried across chunks:
-            // FP64 terms in FP64, FP32 terms in compensated FP32
-            if (sizeof(TM) == 8) {
-                double v = (double)s;
+            // inclusive prefix of D over each chunk, carried across chunks: FP64
+            // terms in FP64, FP32 terms in compensated FP32 (the earlier
+            // chunks' total too, so the prefix reaches FP64 once, at M)
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const double t = __shfl_up_sync(0xffffffffu, v, o);
-                    if (lane >= o) v += t;
+            for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                for (int h = 0; h < H; h++) {
+                    const Sum t = lane_up(v[h], o);
+                    if (lane >= o) v[h] = lane_add(v[h], t);
                 }
+            }
+#pragma unroll
+            for (int h = 0; h < H; h++) {
+                const int k = (ch + h) * 32 + lane;
+                const Sum pre = lane_carry(run, v[h]);
                 if (k < d.L - 1) {
-                    const double mk = -ldg(d.B + k + 1) * pst - (run + v);
+                    const double mk = -ldg(d.B + k + 1) * pst - lane_total(pre);
                     Mv[(size_t)i * d.ldi + k + 1] = mk;
                     if (Macc) Macc[(size_t)i * d.ldi + k + 1] += fscale * mk;
                 }
-                run += __shfl_sync(0xffffffffu, v, 31);
-            } else {
-                // the earlier chunks' total is carried as a compensated pair
-                // too, so the prefix reaches FP64 once, at M
-                F2 v{cv<float>(s), 0.f};
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const F2 t = f2_shfl_up(v, o);
-                    if (lane >= o) v = f2_add(v, t);
-                }
-                v = f2_add(v, runf);
-                if (k < d.L - 1) {
-                    const double mk = -ldg(d.B + k + 1) * pst - (f2d(v.hi) + f2d(v.lo));
-                    Mv[(size_t)i * d.ldi + k + 1] = mk;
-                    if (Macc) Macc[(size_t)i * d.ldi + k + 1] += fscale * mk;
-                }
-                runf = F2{__shfl_sync(0xffffffffu, v.hi, 31), __shfl_sync(0xffffffffu, v.lo, 31)};
+                run = lane_next(run, v[h], pre);
             }
-        }
+        };
+        int ch = 0;
+#pragma unroll 1
+        for (; ch + 1 < nch; ch += 2) chunks(std::integral_constant<int, 2>(), ch);
+        if (ch < nch) chunks(std::integral_constant<int, 1>(), ch);
     }
 }
 
@@ -1288,8 +1364,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const unsigned gC = grid_for((long long)m.nC * L, kBlock), gE = grid_for((long long)m.nE * L, kBlock),
                    gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for((long long)m.nC * 32, kBlock),
                    gI = grid_for((long long)m.nC * (L + 1), kBlock),
-                   gVx = grid_for(m.nV, kBlock), gE32 = grid_for((long long)m.nE + 31, kBlock),
-                   gC32 = grid_for((long long)m.nC + 31, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
+                   gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
+                   gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
                    gCH = grid_for((long long)m.nC * DH.d, kBlock), gVH = grid_for((long long)m.nV * DH.d, kBlock);
     const double dts[3] = {dt / 3.0, dt / 2.0, dt};
     const double ascale = S->accum_scale != 0.0 ? S->accum_scale : 1.0;
@@ -1332,9 +1408,9 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     double *phi_outs[3] = {phA, phB, S->phi};
     for (int s3 = 0; s3 < 3; s3++) {
         const double h3 = dts[s3];
-        GRIST_LAUNCH(h, PN("k_mass_edge"), st, k_mass_edge<P><<<gE32, kBlock, 0, st>>>(
+        GRIST_LAUNCH(h, PN("k_mass_edge"), st, k_mass_edge<P><<<gEG, kBlock, 0, st>>>(
             m, d, ps_in, u_in, F, s3 == 2 ? S->mass_flux_accum : nullptr, ascale, rsum, fcol));
-        GRIST_LAUNCH(h, PN("k_mass_col"), st, k_mass_col<P><<<gC32, kBlock, 0, st>>>(
+        GRIST_LAUNCH(h, PN("k_mass_col"), st, k_mass_col<P><<<gCG, kBlock, 0, st>>>(
             m, d, F, fcol, ps_in, psN, ps_outs[s3], th_in, theta, Mv, h3, s3 == 0 ? S->dpi_start : nullptr, rdps,
             (NH && s3 == 0) ? rthn : nullptr, dphn, S->phi, s3 == 2 ? S->vmass_flux_accum : nullptr, ascale));
         GRIST_LAUNCH(h, PN("k_theta_flux"), st, k_theta_flux<P><<<gEH, kBlock, 0, st>>>(m, d, DH, F, theta, Fth));
