@@ -50,6 +50,14 @@ struct DyPar {
     uint32_t emu;         // GRIST_ROW_* rows rounded to binary32 (precision search)
 };
 
+// Whether the pressure, geopotential and column kernels take forms that round
+// differently from the first ones (short series, tabled reference states):
+// the FP64 policy only.  In the mixed policies these fields feed binary32
+// values (u, the mass flux, the advection of w and phi) by differences, and
+// an ulp of phi moves some of those by a whole binary32 rounding; there the
+// kernels keep every bit.
+template <class P> constexpr bool short_forms() { return sizeof(typename P::TA) == 8 && !P::EMU; }
+
 // Storage-rounding emulation of a single-precision row (precision search,
 // Sec. 2.2 Eqs. 1-2): in the emulating FP64 policy (E) a double value of a
 // row whose bit is set is rounded to binary32 where it is produced; the
@@ -237,10 +245,6 @@ __device__ __forceinline__ double scale_near1_df(double p, double x, double g, c
 }
 
 // ---------------------------------------------------------------------------
-// Whether the column solve takes the short forms (one product for the t^n
-// reference, series tails in binary32): the FP64 policy; see horner_tail.
-template <class P> constexpr bool solve_short() { return sizeof(typename P::TA) == 8 && !P::EMU; }
-
 // Eq. 3: mass flux at edges F = dpi_e u, dpi_e = mean of the two cells'
 // layer mass = dB_k (ps1 + ps2 - 2 pi_top)/2.  One warp takes G edges: the
 // per-edge FP64 work (column factor, the reciprocal 1/(ps1 + ps2 - 2 pi_top)
@@ -394,7 +398,7 @@ __global__ void __launch_bounds__(kBlock) k_mass_col(DevMesh m, DyPar d, const t
                     if (rth_out) {
                         const size_t y = (size_t)i * d.ldi + k;
                         const double dphi = phi_n[y] - phi_n[y + 1];
-                        if constexpr (solve_short<P>()) {
+                        if constexpr (short_forms<P>()) {
                             rth_out[x] = dphi * rcp(th_s[x]);
                         } else {
                             rth_out[x] = rcp(th_s[x]);
@@ -550,10 +554,10 @@ __global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
 // Eq. 8 (hydrostatic diagnostics), one warp per column: mid-layer pressure,
 // alpha = Rd theta (p/p0)^kappa / p, geopotential integrated upward from
 // phi_s by a suffix scan, layer geopotential = mean of its interfaces.
-// Bound by the FP64 pipe: about 27 instructions a cell-level with the table
-// above against about 130 with pow(); level-6 mesh, 30 levels:
-// 323 -> 76 us a launch, plus 10 us a step for the table.
-template <bool EMU, bool DF>
+// Bound by the FP64 pipe: about 24 instructions a cell-level with the table
+// above (SHORT, see short_forms) against about 130 with pow(); level-6 mesh,
+// 30 levels: 323 -> 76 us a launch, plus 10 us a step for the table.
+template <bool EMU, bool DF, bool SHORT>
 __global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const double *__restrict__ ps,
                              const double *__restrict__ th, double *__restrict__ p, double *__restrict__ al,
                              double *__restrict__ phl) {
@@ -561,11 +565,11 @@ __global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const doubl
     const int lane = threadIdx.x & 31;
     if (i >= m.nC) return;
     const double dps = ps[i] - d.pi_top;
-    const double rdps = rcp_nr(dps);
+    const double rdps = SHORT ? rcp_nr(dps) : rcp(dps);
     const int nch = (d.L + 31) >> 5;
-    const int bin = (__double2hiint(dps) >> 13) - ex.base;
+    const int bin = SHORT ? (__double2hiint(dps) >> 13) - ex.base : -1;
     const bool tabled = bin >= 0 && bin < kExnerBins;   // the same for the whole warp
-    const double off = dps - exner_centre(ex.base, bin);
+    const double off = SHORT ? dps - exner_centre(ex.base, bin) : 0.0;
     const double2 *row = ex.tab + (size_t)(tabled ? bin : 0) * d.L;
     double carry = ldg(d.phis + i);
     for (int ch = nch - 1; ch >= 0; ch--) {
@@ -573,16 +577,18 @@ __global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const doubl
         double contrib = 0.0, a = 0.0, pk = 0.0;
         if (k < d.L) {
             const double thk = th[(size_t)i * d.ld + k];
-            pk = fma(ldg(d.Bm + k), dps, d.pi_top);
-            double e;
             if (tabled) {
                 const double2 r = ldg(row + k);
-                e = r.x * horner_tail<4, 8>(r.y * off, bk);
+                pk = fma(ldg(d.Bm + k), dps, d.pi_top);
+                contrib = thk * (r.x * horner_tail<4, 8>(r.y * off, bk));   // alpha dpi
+                a = contrib * (ldg(d.rdB + k) * rdps);
             } else {
-                e = d.rd * pow(pk / d.p0, d.kappa) / pk;
+                const double pt = d.pi_top + ldg(d.B + k) * dps, pb = d.pi_top + ldg(d.B + k + 1) * dps;
+                const double dp = pb - pt;
+                pk = 0.5 * (pt + pb);
+                a = d.rd * (thk * ldg(d.rdB + k) * rdps) * pow(pk / d.p0, d.kappa) / pk;
+                contrib = a * dp;
             }
-            contrib = thk * e;                        // alpha dpi
-            a = contrib * (ldg(d.rdB + k) * rdps);
         }
         // inclusive suffix sum within the chunk
         double v = contrib;
@@ -595,7 +601,7 @@ __global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const doubl
             const size_t x = (size_t)i * d.ld + k;
             p[x] = emu<EMU>(pk, d.emu, GRIST_ROW_EOS);
             al[x] = emu<EMU>(a, d.emu, GRIST_ROW_EOS);
-            const double ph = carry + fma(-0.5, contrib, v);
+            const double ph = SHORT ? carry + fma(-0.5, contrib, v) : carry + (v - contrib) + 0.5 * contrib;
             phl[x] = DF ? pack_split(ph) : emu<EMU>(ph, d.emu, GRIST_ROW_EOS);
         }
         carry += __shfl_sync(0xffffffffu, v, 0);
@@ -1295,12 +1301,13 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const size_t o_p = take(nCL * 8), o_al = take(nCL * 8), o_phl = take(nCL * 8), o_dpp = take(nCL * 8);
     const size_t o_qv = take(nVL * sizeof(TA)), o_K = take(nCL * 8);
     size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0, o_dph = 0;
-    const size_t o_ex = take(NH ? 0 : (size_t)kExnerBins * L * sizeof(double2));
+    constexpr bool kTable = !NH && short_forms<P>();
+    const size_t o_ex = take(kTable ? (size_t)kExnerBins * L * sizeof(double2) : 0);
     if (NH) {
         o_wA = take(nCI * 8); o_wB = take(nCI * 8); o_phA = take(nCI * 8); o_phB = take(nCI * 8);
         o_wst = take(nCI * 8); o_phst = take(nCI * 8); o_pn = take(nCL * 8); o_fw = take(nCI * 8);
         o_rth = take(nCL * 8);
-        o_dph = take(solve_short<P>() ? 0 : nCL * 8);
+        o_dph = take(short_forms<P>() ? 0 : nCL * 8);
     }
     char *s = (char *)scratch(h, 1, off);
     if (!s) return GRIST_ENOMEM;
@@ -1384,7 +1391,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     }
     const Binom bpos = binomial(d.gamma), bneg = binomial(-d.gamma), bkap = binomial(d.kappa - 1.0);
     Exner ex{(double2 *)(s + o_ex), 0};
-    if (!NH) {
+    if (kTable) {
         // two octaves up to twice the power of two at or below p0 - pi_top;
         // bins that no column can fall in where the series' exponent would be
         // out of its range (kappa - 1 outside (-1, 0)).  Made in every step
@@ -1424,12 +1431,12 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                 GRIST_LAUNCH(h, PN("k_nh_explicit"), st, k_nh_explicit<P, false><<<gI, kBlock, 0, st>>>(
                     m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
             cudaError_t se = cudaSuccess;
-            GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, solve_short<P>()>(
+            GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, short_forms<P>()>(
                 m, d, DL, wst, phst, th_outs[s3], rthn, dphn, p_n, ps_outs[s3], h3, w_outs[s3], phi_outs[s3], p_outs[s3],
                 alp, phl, dpp, bpos, bneg, st)));
             if (se != cudaSuccess) return GRIST_ECUDA;
         } else {
-            GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF><<<gW, kBlock, 0, st>>>(
+            GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF, short_forms<P>()><<<gW, kBlock, 0, st>>>(
                 m, d, ex, bkap, ps_outs[s3], th_outs[s3], p, alp, phl));
         }
         GRIST_LAUNCH(h, PN("k_vertex_mass"), st, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, st>>>(m, d, ps_in, rdpv));
