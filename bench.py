@@ -70,6 +70,7 @@ def algorithmic_bytes(name, nC, nE, nV, L, T, prec):
         # u_s, u_n, F, vertex PV (edge PV formed in the kernel), K, M, 1/sum,
         # p, alpha, layer phi, dp/dpi, u_out
         "k_momentum": 2 * EL * sU + EL * sM + VL * sA + CL * 8 + CI * 8 + nC * 8 + 4 * CL * 8 + EL * sU,
+        "k_pv_edge": (EL * sM if prec == "fp64" else 0) + VL * sA + EL * sA,
         "k_eos": CL * 8 + CI * 8 + CL * 8,
         "k_nh_explicit": EL * sU + 2 * nC * 8 + CI * 8 + 4 * CI * 8 + CL * 8 + 2 * CI * 8,
         "k_nh_solve": 2 * CI * 8 + CL * 8 + nC * 8 + 2 * CI * 8 + 4 * CL * 8,

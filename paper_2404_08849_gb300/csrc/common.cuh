@@ -332,6 +332,34 @@ __device__ __forceinline__ void split_trunc(double x, float &h, float &l) {
 // result is the difference to about 2^-24 of itself.
 __device__ __forceinline__ float diff_df(float ah, float al, float bh, float bl) { return (ah - bh) + (al - bl); }
 
+// a - b, equal to the FP64 subtraction bit for bit, without the FP64 pipe where
+// the two are close: same sign and exponents at most one apart make the
+// difference of the aligned significands an exact integer, whose conversion
+// back is exact too when it is below 2^53.  About 30 integer instructions
+// against the 64 scheduler cycles that an FP64 instruction of a warp takes;
+// lanes outside the fast case (or with a difference that would leave the
+// normal range) subtract in FP64.
+__device__ __forceinline__ double sub_near(double a, double b) {
+    const uint32_t ha = (uint32_t)__double2hiint(a), hb = (uint32_t)__double2hiint(b);
+    const int sa = (int)(ha >> 20), sb = (int)(hb >> 20);   // sign and exponent
+    const int ds = sa - sb, smin = min(sa, sb);
+    unsigned long long A = ((unsigned long long)((ha & 0xfffffu) | 0x100000u) << 32) | (uint32_t)__double2loint(a);
+    unsigned long long B = ((unsigned long long)((hb & 0xfffffu) | 0x100000u) << 32) | (uint32_t)__double2loint(b);
+    if (ds > 0) A += A;
+    if (ds < 0) B += B;
+    const long long D = (long long)(A - B);
+    const unsigned long long mag = (unsigned long long)(D < 0 ? -D : D);
+    const int up = __clzll((long long)(mag | 1ull)) - 11;   // leading one to bit 52
+    const int ex = (smin & 0x7ff) - up;
+    if ((unsigned)(ds + 1) <= 2u && up >= 0 && ex > 0 && (smin & 0x7ff) < 0x7fe) {
+        const unsigned long long n = mag << up;
+        const uint32_t sgn = ((uint32_t)((unsigned long long)D >> 32) ^ ((uint32_t)smin << 20)) & 0x80000000u;
+        const uint32_t hi = mag == 0 ? 0u : ((uint32_t)(n >> 32) + ((uint32_t)(ex - 1) << 20)) | sgn;
+        return __hiloint2double((int)hi, (int)(uint32_t)n);
+    }
+    return a - b;
+}
+
 // cv<T>(x): x in type T, through the integer conversions above.
 template <typename T> struct Cvt;
 template <> struct Cvt<double> {
@@ -343,6 +371,42 @@ template <> struct Cvt<float> {
     static __device__ __forceinline__ float from(float x) { return x; }
 };
 template <typename T, typename S> __device__ __forceinline__ T cv(S x) { return Cvt<T>::from(x); }
+
+// V consecutive values of a row as 8- or 16-byte read-only loads / stores (p
+// aligned to the access).
+template <int V, typename T> __device__ __forceinline__ void ldgv(const T *p, T (&o)[V]) {
+    if constexpr (V == 1) {
+        o[0] = __ldg(p);
+    } else if constexpr (sizeof(T) * V == 8) {
+        const float2 a = __ldg((const float2 *)p);
+        o[0] = a.x; o[1] = a.y;
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4) {
+            const float4 a = __ldg((const float4 *)(p + j));
+            o[j] = a.x; o[j + 1] = a.y; o[j + 2] = a.z; o[j + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) {
+            const double2 a = __ldg((const double2 *)(p + j));
+            o[j] = a.x; o[j + 1] = a.y;
+        }
+    }
+}
+template <int V, typename T> __device__ __forceinline__ void stgv(T *p, const T (&o)[V]) {
+    if constexpr (V == 1) {
+        *p = o[0];
+    } else if constexpr (sizeof(T) * V == 8) {
+        *(float2 *)p = make_float2(o[0], o[1]);
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < V; j += 4) *(float4 *)(p + j) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) *(double2 *)(p + j) = make_double2(o[j], o[j + 1]);
+    }
+}
 
 inline unsigned grid_for(long long n, int block) {
     long long g = (n + block - 1) / block;

@@ -55,8 +55,9 @@ struct DyPar {
 // the FP64 policy only.  In the mixed policies these fields feed binary32
 // values (u, the mass flux, the advection of w and phi) by differences, and
 // an ulp of phi moves some of those by a whole binary32 rounding; there the
-// kernels keep every bit.
-template <class P> constexpr bool short_forms() { return sizeof(typename P::TA) == 8 && !P::EMU; }
+// kernels keep every bit.  (The emulating FP64 variant equals the FP64 policy
+// bit for bit where no emulated row is involved, so it takes them too.)
+template <class P> constexpr bool short_forms() { return sizeof(typename P::TA) == 8; }
 
 // Storage-rounding emulation of a single-precision row (precision search,
 // Sec. 2.2 Eqs. 1-2): in the emulating FP64 policy (E) a double value of a
@@ -677,14 +678,54 @@ __global__ void k_ke(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__re
     K[(size_t)i * d.ld + k] = P::DF ? pack_split(s) : emu<P::EMU>(s, d.emu, GRIST_ROW_KE_GRAD);
 }
 
-// PV at edge-level (e, k): the mean of the PV at the edge's two vertices.
-template <class P>
-__device__ __forceinline__ typename P::TA pv_at_edge(const DevMesh &m, const DyPar &d,
-                                                     const typename P::TA *__restrict__ qv, int e, int k) {
+// Twice the PV at an edge from the sum of its vertices' (the mean is the value
+// that the precision search rounds).
+template <class P> __device__ __forceinline__ typename P::TA twice_pv(typename P::TA sum, const DyPar &d) {
     using TA = typename P::TA;
+    if constexpr (P::EMU) return (TA)2 * emu<true>((TA)0.5 * sum, d.emu, GRIST_ROW_PV_FLUX);
+    return sum;
+}
+
+// What the momentum equation needs of the PV at edges, q_e the mean of the
+// edge's two vertices: q_e itself, so that a neighbour is one load instead of two
+// and an index; in the FP64 policy 2 F q_e, with which the PV flux
+// sum_e' w F' (q_e + q_e')/2 is (q_e sum w F' + sum w F' q_e')/2, two FP64
+// instructions a neighbour instead of six (short_forms).  V consecutive levels
+// a thread, 16 bytes: the vertex rows are gathers, and with single levels the
+// pass took 492 us, with vectors 170 (level 8, 60 levels, mixed).
+template <class P, int V>
+__global__ void __launch_bounds__(kBlock) k_pv_edge(DevMesh m, DyPar d, LevelDiv Dg, const typename P::TM *__restrict__ F,
+                                                    const typename P::TA *__restrict__ qv, typename P::TA *__restrict__ G) {
+    using TA = typename P::TA;
+    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= (uint32_t)m.nE * Dg.d) return;
+    int e, kg;
+    split_index(n, Dg, e, kg);
     const int2 v = ldg(m.voe + e);
-    return emu<P::EMU>((TA)0.5 * (ldg(qv + (size_t)v.x * d.ld + k) + ldg(qv + (size_t)v.y * d.ld + k)), d.emu,
-                       GRIST_ROW_PV_FLUX);
+    const size_t x = (size_t)e * d.ld + kg * V;
+    TA a[V], b[V];
+    ldgv<V>(qv + (size_t)v.x * d.ld + kg * V, a);
+    ldgv<V>(qv + (size_t)v.y * d.ld + kg * V, b);
+    if constexpr (short_forms<P>()) {
+        TA f[V];
+        ldgv<V>(F + x, f);
+#pragma unroll
+        for (int t = 0; t < V; t++) a[t] = f[t] * twice_pv<P>(a[t] + b[t], d);
+    } else {
+#pragma unroll
+        for (int t = 0; t < V; t++) a[t] = (TA)0.5 * (a[t] + b[t]);
+    }
+    stgv<V>(G + x, a);
+}
+
+// (double)a - (double)b of two binary32 numbers, bit for bit: where the binary32
+// difference is exact (its TwoSum error is zero) it is that number.
+__device__ __forceinline__ double wind_diff(double a, double b) { return a - b; }
+__device__ __forceinline__ double wind_diff(float a, float b) {
+    const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
+    const float err = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+    if (err == 0.f) return f2d(s);
+    return f2d(a) - f2d(b);
 }
 
 // Eq. 5 momentum tendency and stage update:
@@ -695,10 +736,18 @@ __device__ __forceinline__ typename P::TA pv_at_edge(const DevMesh &m, const DyP
 // computed in double, their tendency saved in single).  The edge layer mass
 // in the vertical advection is dB_k (ps1 + ps2 - 2 pi_top)/2, entered as
 // the product of the per-level and per-edge reciprocals.
+// Bound by the FP64 pipe: the differences of p, phi and K between the edge's
+// cells and of u between levels are taken off it without changing a bit
+// (sub_near, wind_diff), 16 -> 11 FP64 instructions an edge-level in the mixed
+// policies; 40 registers, for six blocks an SM, since the loads' latency is
+// what is left.  Level 8, 60 levels, us a launch with k_pv_edge's: mixed
+// 3457 -> 2843; FP64, level 7, 3886 -> 2070.  Two or four levels a thread
+// (shared indices and M sums) measured slower: 2752 and 3370 against 2673.
 template <class P, bool NH>
-__global__ void k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
+__global__ void __launch_bounds__(kBlock, 6) k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
                            const typename P::TU *u_n, typename P::TU *u_out, const typename P::TM *__restrict__ F,
-                           const typename P::TA *__restrict__ qv, const double *__restrict__ K,
+                           const typename P::TA *__restrict__ qv, const typename P::TA *__restrict__ G,
+                           const double *__restrict__ K,
                            const double *__restrict__ Mv, const double *__restrict__ rsum_e,
                            const double *__restrict__ p, const double *__restrict__ al,
                            const double *__restrict__ phl, const double *__restrict__ dpp, double dts,
@@ -711,16 +760,26 @@ __global__ void k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU
     split_index(n, Dv, e, k);
     const size_t x = (size_t)e * d.ld + k;
     const int2 c = ldg(m.coe + e);
-    // the edge PV values come from the vertex PV (the mean of the two
-    // vertices, formed here: this kernel is bound by the FP64 pipe and has
-    // load slots to spare, so no separate edge-PV pass is needed)
-    const TA qee = pv_at_edge<P>(m, d, qv, e, k);
     TA pv = 0;
+    if constexpr (short_forms<P>()) {
+        const int2 ve = ldg(m.voe + e);
+        const TA q2 = twice_pv<P>(ldg(qv + (size_t)ve.x * d.ld + k) + ldg(qv + (size_t)ve.y * d.ld + k), d);
+        TA s = 0;
 #pragma unroll
-    for (int j = 0; j < GRIST_MAXEOE; j++) {
-        const int e2 = ldg(m.eoe + e * 10 + j);
-        const size_t y = (size_t)e2 * d.ld + k;
-        pv += ldg(Coef<TA>::wpv(m) + e * 10 + j) * cv<TA>(ldg(F + y)) * ((TA)0.5 * (qee + pv_at_edge<P>(m, d, qv, e2, k)));
+        for (int j = 0; j < GRIST_MAXEOE; j++) {
+            const size_t y = (size_t)ldg(m.eoe + e * 10 + j) * d.ld + k;
+            const TA w = ldg(Coef<TA>::wpv(m) + e * 10 + j);
+            s += w * ldg(F + y);
+            pv += w * ldg(G + y);
+        }
+        pv = 0.25 * fma(q2, s, pv);   // (2 q_e sum w F' + sum w F' 2 q_e')/4
+    } else {
+        const TA qee = ldg(G + x);
+#pragma unroll
+        for (int j = 0; j < GRIST_MAXEOE; j++) {
+            const size_t y = (size_t)ldg(m.eoe + e * 10 + j) * d.ld + k;
+            pv += ldg(Coef<TA>::wpv(m) + e * 10 + j) * cv<TA>(ldg(F + y)) * ((TA)0.5 * (qee + ldg(G + y)));
+        }
     }
     const size_t a1 = (size_t)c.x * d.ld + k, a2 = (size_t)c.y * d.ld + k;
     if (P::DF) {
@@ -755,14 +814,14 @@ __global__ void k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU
         u_out[x] = (TU)v;
         return;
     }
-    const double uk = cv<double>(ldg(u_s + x));
+    const TU uk = ldg(u_s + x);
     double va = 0.0;
     if (k < d.L - 1)
         va = (ldg(Mv + (size_t)c.x * d.ldi + k + 1) + ldg(Mv + (size_t)c.y * d.ldi + k + 1)) *
-             (cv<double>(ldg(u_s + x + 1)) - uk);
+             wind_diff(ldg(u_s + x + 1), uk);
     if (k > 0)
         va = fma(ldg(Mv + (size_t)c.x * d.ldi + k) + ldg(Mv + (size_t)c.y * d.ldi + k),
-                 uk - cv<double>(ldg(u_s + x - 1)), va);
+                 wind_diff(uk, ldg(u_s + x - 1)), va);
     // [M sums](du) / (2 dpi_e) with dpi_e = dB (sum)/2, M_e = (M1 + M2)/2;
     // rsum_e holds 1/(2 sum)
     va *= ldg(d.rdB + k) * ldg(rsum_e + e);
@@ -772,8 +831,8 @@ __global__ void k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU
     double grad;
     if (!P::EMU || !(d.emu & GRIST_ROW_PGF)) {
         const double de = NH ? ldg(dpp + a1) + ldg(dpp + a2) : 2.0;
-        grad = fma(ldg(al + a1) + ldg(al + a2), ldg(p + a2) - ldg(p + a1),
-                   fma(de, ldg(phl + a2) - ldg(phl + a1), ldg(K + a2) - ldg(K + a1)));
+        grad = fma(ldg(al + a1) + ldg(al + a2), sub_near(ldg(p + a2), ldg(p + a1)),
+                   fma(de, sub_near(ldg(phl + a2), ldg(phl + a1)), sub_near(ldg(K + a2), ldg(K + a1))));
     } else {
         // pressure gradient and gravity from binary32 inputs, summed and
         // rounded to binary32 (precision search)
@@ -1300,6 +1359,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const size_t o_theta = take(nCL * sizeof(TA)), o_Fth = take(nEL * sizeof(TA));
     const size_t o_p = take(nCL * 8), o_al = take(nCL * 8), o_phl = take(nCL * 8), o_dpp = take(nCL * 8);
     const size_t o_qv = take(nVL * sizeof(TA)), o_K = take(nCL * 8);
+    const size_t o_Gq = take(nEL * sizeof(TA));
     size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0, o_dph = 0;
     constexpr bool kTable = !NH && short_forms<P>();
     const size_t o_ex = take(kTable ? (size_t)kExnerBins * L * sizeof(double2) : 0);
@@ -1358,7 +1418,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     TA *theta = (TA *)(s + o_theta), *Fth = (TA *)(s + o_Fth);
     double *p = (double *)(s + o_p), *alp = (double *)(s + o_al), *phl = (double *)(s + o_phl),
            *dpp = (double *)(s + o_dpp);
-    TA *qv = (TA *)(s + o_qv);
+    TA *qv = (TA *)(s + o_qv), *Gq = (TA *)(s + o_Gq);
     double *K = (double *)(s + o_K);
     double *wA = (double *)(s + o_wA), *wB = (double *)(s + o_wB), *phA = (double *)(s + o_phA),
            *phB = (double *)(s + o_phB), *wst = (double *)(s + o_wst), *phst = (double *)(s + o_phst),
@@ -1368,12 +1428,17 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     TU *u = (TU *)S->u;
     uint32_t *status = status_word(h);
     const LevelDiv DL = make_div((uint32_t)L), DI = make_div((uint32_t)(L + 1)), DH = make_div((uint32_t)(L + 1) / 2);
-    const unsigned gC = grid_for((long long)m.nC * L, kBlock), gE = grid_for((long long)m.nE * L, kBlock),
+    const unsigned gC = grid_for((long long)m.nC * L, kBlock),
                    gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for((long long)m.nC * 32, kBlock),
                    gI = grid_for((long long)m.nC * (L + 1), kBlock),
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
                    gCH = grid_for((long long)m.nC * DH.d, kBlock), gVH = grid_for((long long)m.nV * DH.d, kBlock);
+    // edge PV on 16-byte vectors of levels, or 8-byte ones, where rows are whole vectors
+    constexpr int kPvV = 16 / sizeof(TA), kPvH = sizeof(TA) == 4 ? 2 : 1;
+    const int pvv = L % kPvV == 0 && ld % kPvV == 0 ? kPvV : (L % kPvH == 0 && ld % kPvH == 0 ? kPvH : 1);
+    const LevelDiv DP = make_div((uint32_t)(L / pvv));
+    const unsigned gE = grid_for((long long)m.nE * L, kBlock), gP = grid_for((long long)m.nE * DP.d, kBlock);
     const double dts[3] = {dt / 3.0, dt / 2.0, dt};
     const double ascale = S->accum_scale != 0.0 ? S->accum_scale : 1.0;
 
@@ -1442,8 +1507,11 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
         GRIST_LAUNCH(h, PN("k_vertex_mass"), st, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, st>>>(m, d, ps_in, rdpv));
         GRIST_LAUNCH(h, PN("k_vort"), st, k_vort<P><<<gVH, kBlock, 0, st>>>(m, d, DH, u_in, rdpv, qv));
         GRIST_LAUNCH(h, PN("k_ke"), st, k_ke<P><<<gC, kBlock, 0, st>>>(m, d, DL, u_in, K));
+        GRIST_LAUNCH(h, PN("k_pv_edge"), st, (pvv == kPvV   ? k_pv_edge<P, kPvV>
+                                              : pvv == kPvH ? k_pv_edge<P, kPvH>
+                                                            : k_pv_edge<P, 1>)<<<gP, kBlock, 0, st>>>(m, d, DP, F, qv, Gq));
         GRIST_LAUNCH(h, PN("k_momentum"), st, k_momentum<P, NH><<<gE, kBlock, 0, st>>>(
-            m, d, DL, u_in, u, u_outs[s3], F, qv, K, Mv, rsum, p_outs[s3], alp, phl, dpp, h3, status));
+            m, d, DL, u_in, u, u_outs[s3], F, qv, Gq, K, Mv, rsum, p_outs[s3], alp, phl, dpp, h3, status));
         u_in = u_outs[s3];
         ps_in = ps_outs[s3];
         th_in = th_outs[s3];
