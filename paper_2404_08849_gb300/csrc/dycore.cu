@@ -662,20 +662,55 @@ __global__ void k_vort(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TU *__
 }
 
 // Cell kinetic energy, stored doubled: 2K = sum (dc dv / 2A) u^2 (FP64:
-// boxed term of Eq. 5).
-template <class P>
-__global__ void k_ke(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u, double *__restrict__ K) {
-    uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (uint32_t)m.nC * (uint32_t)d.L) return;
-    int i, k;
-    split_index(n, Dv, i, k);
-    double s = 0.0;
+// boxed term of Eq. 5), V consecutive levels a thread.  Bound by the FP64 pipe
+// (89 %): with a binary32 wind the product of the weight and u, half of the
+// FP64 instructions, is formed in integers bit for bit (MulF32; the weight is
+// unpacked once for the V levels).  Level 8, 60 levels, mixed: 846 -> 534 us a
+// launch.
+template <class P, int V>
+__global__ void __launch_bounds__(kBlock) k_ke(DevMesh m, DyPar d, LevelDiv Dg, const typename P::TU *__restrict__ u,
+                                               double *__restrict__ K) {
+    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= (uint32_t)m.nC * Dg.d) return;
+    int i, kg;
+    split_index(n, Dg, i, kg);
+    const int k = kg * V;
+    int e[GRIST_MAXE];
+    load_row6(m.eoc8, i, e);
+    double s[V];
+    bool ok[V];
+#pragma unroll
+    for (int t = 0; t < V; t++) {
+        s[t] = 0.0;
+        ok[t] = true;
+    }
 #pragma unroll
     for (int j = 0; j < GRIST_MAXE; j++) {
-        const double ue = cv<double>(ldg(u + (size_t)ldg(m.eoc + i * 6 + j) * d.ld + k));
-        s += ldg(m.kec2 + i * 6 + j) * ue * ue;
+        const double w = ldg(m.kec2 + i * 6 + j);
+        typename P::TU ue[V];
+        ldgv<V>(u + (size_t)e[j] * d.ld + k, ue);
+        if constexpr (sizeof(typename P::TU) == 4) {
+            const MulF32 wm(w);
+            if ((__double_as_longlong(w) << 1) == 0) continue;   // padding of a pentagon
+#pragma unroll
+            for (int t = 0; t < V; t++) s[t] = fma(wm.times(ue[t], ok[t]), f2d_normal(ue[t]), s[t]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; t++) s[t] += w * ue[t] * ue[t];
+        }
     }
-    K[(size_t)i * d.ld + k] = P::DF ? pack_split(s) : emu<P::EMU>(s, d.emu, GRIST_ROW_KE_GRAD);
+#pragma unroll
+    for (int t = 0; t < V; t++) {
+        if (!ok[t]) {   // a subnormal or non-finite wind
+            s[t] = 0.0;
+            for (int j = 0; j < GRIST_MAXE; j++) {
+                const double ue = cv<double>(u[(size_t)e[j] * d.ld + k + t]);
+                s[t] += ldg(m.kec2 + i * 6 + j) * ue * ue;
+            }
+        }
+        s[t] = P::DF ? pack_split(s[t]) : emu<P::EMU>(s[t], d.emu, GRIST_ROW_KE_GRAD);
+    }
+    stgv<V>(K + (size_t)i * d.ld + k, s);
 }
 
 // Twice the PV at an edge from the sum of its vertices' (the mean is the value
@@ -952,12 +987,14 @@ __global__ void k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P:
 // (32 bytes, one sector) of 32 / kSolveKC columns, so every global sector
 // is used whole; the 33-wide rows keep the shared-memory side free of bank
 // conflicts.  Four-level chunks keep a block's shared memory at 6.6 KB so
-// that 24 one-warp blocks fit on an SM.
+// that 20 one-warp blocks fit on an SM (level 8, 60 levels, us a launch by blocks
+// the registers must allow: 16 3539, 18 3368, 20 3346, 22 3451, 24 3475; chunks of
+// 2 or 8 levels 3983, 4177).
 #ifndef GRIST_SOLVE_KC
 #define GRIST_SOLVE_KC 4          // levels per staged chunk (1, 2, 4 or 8)
 #endif
 #ifndef GRIST_SOLVE_MIN_BLOCKS
-#define GRIST_SOLVE_MIN_BLOCKS 24 // resident one-warp blocks per SM the registers must allow
+#define GRIST_SOLVE_MIN_BLOCKS 20 // resident one-warp blocks per SM the registers must allow
 #endif
 constexpr int kSolveCols = 32;
 constexpr int kSolveKC = GRIST_SOLVE_KC;
@@ -1434,6 +1471,13 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
                    gCH = grid_for((long long)m.nC * DH.d, kBlock), gVH = grid_for((long long)m.nV * DH.d, kBlock);
+    // kinetic energy on 2 (binary32 wind: up to 4) levels where rows are whole,
+    // aligned vectors
+    constexpr int kKeV = sizeof(TU) == 4 ? 4 : 2;
+    auto ke_fits = [&](int v) { return L % v == 0 && ld % v == 0 && (uintptr_t)u % (v * sizeof(TU)) == 0; };
+    const int kev = kKeV == 4 && ke_fits(4) ? 4 : (ke_fits(2) ? 2 : 1);
+    const LevelDiv DK = make_div((uint32_t)(L / kev));
+    const unsigned gK = grid_for((long long)m.nC * DK.d, kBlock);
     // edge PV on 16-byte vectors of levels, or 8-byte ones, where rows are whole vectors
     constexpr int kPvV = 16 / sizeof(TA), kPvH = sizeof(TA) == 4 ? 2 : 1;
     const int pvv = L % kPvV == 0 && ld % kPvV == 0 ? kPvV : (L % kPvH == 0 && ld % kPvH == 0 ? kPvH : 1);
@@ -1506,7 +1550,9 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
         }
         GRIST_LAUNCH(h, PN("k_vertex_mass"), st, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, st>>>(m, d, ps_in, rdpv));
         GRIST_LAUNCH(h, PN("k_vort"), st, k_vort<P><<<gVH, kBlock, 0, st>>>(m, d, DH, u_in, rdpv, qv));
-        GRIST_LAUNCH(h, PN("k_ke"), st, k_ke<P><<<gC, kBlock, 0, st>>>(m, d, DL, u_in, K));
+        GRIST_LAUNCH(h, PN("k_ke"), st, (kev == 4   ? k_ke<P, kKeV>
+                                         : kev == 2 ? k_ke<P, 2>
+                                                    : k_ke<P, 1>)<<<gK, kBlock, 0, st>>>(m, d, DK, u_in, K));
         GRIST_LAUNCH(h, PN("k_pv_edge"), st, (pvv == kPvV   ? k_pv_edge<P, kPvV>
                                               : pvv == kPvH ? k_pv_edge<P, kPvH>
                                                             : k_pv_edge<P, 1>)<<<gP, kBlock, 0, st>>>(m, d, DP, F, qv, Gq));
