@@ -440,11 +440,15 @@ __global__ void __launch_bounds__(kBlock) k_mass_col(DevMesh m, DyPar d, const t
 }
 
 // Eq. 4 horizontal flux: third-order upwind (beta = 1) edge value of theta
-// times the mass flux.  A thread takes levels kg and kg + Lh (Lh = ceil(L/2))
-// of one edge, so the upwind stencil row (4 vector loads) serves both
-// levels unless their fluxes run opposite ways.
-template <class P>
-__global__ void k_theta_flux(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TM *__restrict__ F,
+// times the mass flux.  V = 4 (binary32): a thread takes four consecutive levels
+// of one edge as vectors, with one read of the upwind stencil row (4 vector
+// loads) where their fluxes run the same way, else level by level; V = 1:
+// levels kg and kg + Lh (Lh = ceil(L/2)).  Gathers of 4-byte values are
+// latency-bound: level 8, 60 levels, mixed 648 -> 435 us a launch (162 at the
+// DRAM rate).  Pairs were not faster: binary32, 30 levels, level 6 25 -> 27;
+// FP64 (bound by its pipe), level 7 501 -> 520.
+template <class P, int V>
+__global__ void __launch_bounds__(kBlock) k_theta_flux(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TM *__restrict__ F,
                              const typename P::TA *__restrict__ th, typename P::TA *__restrict__ Fth) {
     using TA = typename P::TA;
     const int Lh = (int)Dh.d;
@@ -455,10 +459,7 @@ __global__ void k_theta_flux(DevMesh m, DyPar d, LevelDiv Dh, const typename P::
     int c[GRIST_D2P];
     TA w[GRIST_D2P];
     int loaded = -1;
-#pragma unroll
-    for (int u = 0; u < 2; u++) {
-        const int k = kg + u * Lh;
-        if (k >= d.L) break;
+    auto level = [&](int k) {
         const size_t x = (size_t)e * d.ld + k;
         const TA f = cv<TA>(F[x]);
         const int side = f >= (TA)0 ? 0 : 1;
@@ -484,12 +485,47 @@ __global__ void k_theta_flux(DevMesh m, DyPar d, LevelDiv Dh, const typename P::
                  (TA)2 * ldg(Coef<TA>::dc2(m) + e) * sm;
         }
         Fth[x] = emu<P::EMU>(f * te, d.emu, GRIST_ROW_THETA);
+    };
+    if constexpr (V > 1) {
+        const size_t x = (size_t)e * d.ld + kg * V;
+        typename P::TM fm[V];
+        ldgv<V>(F + x, fm);
+        TA f[V], q[V], te[V];
+        unsigned back = 0;   // bit t: level t's flux runs from c2
+#pragma unroll
+        for (int t = 0; t < V; t++) {
+            f[t] = cv<TA>(fm[t]);
+            if (!(f[t] >= (TA)0)) back |= 1u << t;
+            te[t] = 0;
+        }
+        if (m.d2w_ok && (back == 0u || back == (1u << V) - 1u)) {
+            load_d2w(m, e, back ? 1 : 0, c, w);
+#pragma unroll
+            for (int j = 0; j < GRIST_D2P; j++) {
+                ldgv<V>(th + (size_t)c[j] * d.ld + kg * V, q);
+#pragma unroll
+                for (int t = 0; t < V; t++) te[t] += w[j] * q[t];
+            }
+#pragma unroll
+            for (int t = 0; t < V; t++) te[t] *= f[t];
+            stgv<V>(Fth + x, te);
+        } else {
+#pragma unroll 1
+            for (int t = 0; t < V; t++) level(kg * V + t);
+        }
+    } else {
+        level(kg);
+        if (kg + Lh < d.L) level(kg + Lh);
     }
 }
 
-// Eq. 4 update: dpi theta^(s) = dpi theta^n + dt_s (-div F_theta - delta(M theta)).
-template <class P>
-__global__ void k_theta_update(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TA *__restrict__ Fth,
+// Eq. 4 update: dpi theta^(s) = dpi theta^n + dt_s (-div F_theta - delta(M theta)),
+// V consecutive levels a thread (V > 1), or levels kg and kg + Lh.  th_n and
+// th_out may be the caller's rows, moved level by level where those are not
+// aligned.  Level 8, 60 levels, mixed: 420 -> 264 us a launch (233 at the DRAM
+// rate); level 6, 30 levels (pairs) 17 -> 13; FP64, level 7, 276 -> 248.
+template <class P, int V>
+__global__ void __launch_bounds__(kBlock) k_theta_update(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TA *__restrict__ Fth,
                                const typename P::TA *__restrict__ th, const double *__restrict__ Mv,
                                const double *__restrict__ th_n, double *__restrict__ th_out, double dts) {
     using TA = typename P::TA;
@@ -498,25 +534,54 @@ __global__ void k_theta_update(DevMesh m, DyPar d, LevelDiv Dh, const typename P
     if (n >= (uint32_t)m.nC * (uint32_t)Lh) return;
     int i, kg;
     split_index(n, Dh, i, kg);
-    // the cell's row once for its two levels kg and kg + Lh
+    // the cell's row once for the thread's levels
     int eidx[GRIST_MAXE];
     TA cw[GRIST_MAXE];
     load_row6(m.eoc8, i, eidx);
     load_row6(Coef<TA>::cdiv8(m), i, cw);
+    if constexpr (V > 1) {
+        const int k = kg * V;
+        const size_t x = (size_t)i * d.ld + k, y = (size_t)i * d.ldi + k;
+        TA div[V], a[V], tk[V], fl[V + 1];
+        double o[V];
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-        const int k = kg + u * Lh;
-        if (k >= d.L) break;
-        TA div = 0;
+        for (int t = 0; t < V; t++) div[t] = 0;
 #pragma unroll
-        for (int j = 0; j < GRIST_MAXE; j++) div += cw[j] * ldg(Fth + (size_t)eidx[j] * d.ld + k);
-        const size_t x = (size_t)i * d.ld + k;
-        const TA tk = th[x];
-        TA top = 0, bot = 0;
-        if (k > 0) top = cv<TA>(Mv[(size_t)i * d.ldi + k]) * ((TA)0.5 * (th[x - 1] + tk));
-        if (k < d.L - 1) bot = cv<TA>(Mv[(size_t)i * d.ldi + k + 1]) * ((TA)0.5 * (tk + th[x + 1]));
-        const TA tend = -div - (bot - top);
-        th_out[x] = th_n[x] + dts * cv<double>(tend);
+        for (int j = 0; j < GRIST_MAXE; j++) {
+            ldgv<V>(Fth + (size_t)eidx[j] * d.ld + k, a);
+#pragma unroll
+            for (int t = 0; t < V; t++) div[t] += cw[j] * a[t];
+        }
+        ldgv<V>(th + x, tk);
+        ldgv<V>(th_n + x, o);
+        const TA above = k > 0 ? ldg(th + x - 1) : (TA)0, below = k + V < d.L ? ldg(th + x + V) : (TA)0;
+#pragma unroll
+        for (int t = 0; t <= V; t++) {
+            const TA q0 = t > 0 ? tk[t > 0 ? t - 1 : 0] : above, q1 = t < V ? tk[t < V ? t : 0] : below;
+            fl[t] = (k + t > 0 && k + t < d.L) ? cv<TA>(ldg(Mv + y + t)) * ((TA)0.5 * (q0 + q1)) : (TA)0;
+        }
+#pragma unroll
+        for (int t = 0; t < V; t++) {
+            const TA tend = -div[t] - (fl[t + 1] - fl[t]);
+            o[t] = o[t] + dts * cv<double>(tend);
+        }
+        stgv<V>(th_out + x, o);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = kg + u * Lh;
+            if (k >= d.L) break;
+            TA div = 0;
+#pragma unroll
+            for (int j = 0; j < GRIST_MAXE; j++) div += cw[j] * ldg(Fth + (size_t)eidx[j] * d.ld + k);
+            const size_t x = (size_t)i * d.ld + k;
+            const TA tk = th[x];
+            TA top = 0, bot = 0;
+            if (k > 0) top = cv<TA>(Mv[(size_t)i * d.ldi + k]) * ((TA)0.5 * (th[x - 1] + tk));
+            if (k < d.L - 1) bot = cv<TA>(Mv[(size_t)i * d.ldi + k + 1]) * ((TA)0.5 * (tk + th[x + 1]));
+            const TA tend = -div - (bot - top);
+            th_out[x] = th_n[x] + dts * cv<double>(tend);
+        }
     }
 }
 
@@ -1469,8 +1534,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                    gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for((long long)m.nC * 32, kBlock),
                    gI = grid_for((long long)m.nC * (L + 1), kBlock),
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
-                   gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock), gEH = grid_for((long long)m.nE * DH.d, kBlock),
-                   gCH = grid_for((long long)m.nC * DH.d, kBlock), gVH = grid_for((long long)m.nV * DH.d, kBlock);
+                   gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock),
+                   gVH = grid_for((long long)m.nV * DH.d, kBlock);
     // kinetic energy on 2 (binary32 wind: up to 4) levels where rows are whole,
     // aligned vectors
     constexpr int kKeV = sizeof(TU) == 4 ? 4 : 2;
@@ -1482,6 +1547,12 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     constexpr int kPvV = 16 / sizeof(TA), kPvH = sizeof(TA) == 4 ? 2 : 1;
     const int pvv = L % kPvV == 0 && ld % kPvV == 0 ? kPvV : (L % kPvH == 0 && ld % kPvH == 0 ? kPvH : 1);
     const LevelDiv DP = make_div((uint32_t)(L / pvv));
+    // theta update on the same vectors, the flux on binary32 quads, or two levels
+    // half a column apart
+    const bool quad = pvv == 4;
+    const int thv = ((uintptr_t)S->dpi_theta % 16) == 0 ? pvv : 1;
+    const LevelDiv DT = quad ? DP : DH, DTU = thv > 1 ? DP : DH;
+    const unsigned gEH = grid_for((long long)m.nE * DT.d, kBlock), gCT = grid_for((long long)m.nC * DTU.d, kBlock);
     const unsigned gE = grid_for((long long)m.nE * L, kBlock), gP = grid_for((long long)m.nE * DP.d, kBlock);
     const double dts[3] = {dt / 3.0, dt / 2.0, dt};
     const double ascale = S->accum_scale != 0.0 ? S->accum_scale : 1.0;
@@ -1529,9 +1600,11 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
         GRIST_LAUNCH(h, PN("k_mass_col"), st, k_mass_col<P><<<gCG, kBlock, 0, st>>>(
             m, d, F, fcol, ps_in, psN, ps_outs[s3], th_in, theta, Mv, h3, s3 == 0 ? S->dpi_start : nullptr, rdps,
             (NH && s3 == 0) ? rthn : nullptr, dphn, S->phi, s3 == 2 ? S->vmass_flux_accum : nullptr, ascale));
-        GRIST_LAUNCH(h, PN("k_theta_flux"), st, k_theta_flux<P><<<gEH, kBlock, 0, st>>>(m, d, DH, F, theta, Fth));
-        GRIST_LAUNCH(h, PN("k_theta_update"), st, k_theta_update<P><<<gCH, kBlock, 0, st>>>(
-            m, d, DH, Fth, theta, Mv, S->dpi_theta, th_outs[s3], h3));
+        GRIST_LAUNCH(h, PN("k_theta_flux"), st, (quad ? k_theta_flux<P, sizeof(TA) == 4 ? 4 : 1> : k_theta_flux<P, 1>)<<<gEH, kBlock, 0, st>>>(m, d, DT, F, theta, Fth));
+        GRIST_LAUNCH(h, PN("k_theta_update"), st, (thv == kPvV   ? k_theta_update<P, kPvV>
+                                                   : thv == kPvH ? k_theta_update<P, kPvH>
+                                                                 : k_theta_update<P, 1>)<<<gCT, kBlock, 0, st>>>(
+            m, d, DTU, Fth, theta, Mv, S->dpi_theta, th_outs[s3], h3));
         if (NH) {
             if (s3 == 0)
                 GRIST_LAUNCH(h, PN("k_nh_explicit"), st, k_nh_explicit<P, true><<<gI, kBlock, 0, st>>>(
