@@ -511,7 +511,8 @@ __global__ void __launch_bounds__(kBlock) k_theta_flux(DevMesh m, DyPar d, Level
             stgv<V>(Fth + x, te);
         } else {
 #pragma unroll 1
-            for (int t = 0; t < V; t++) level(kg * V + t);
+            for (int t = 0; t < V; t++)
+                if (kg * V + t < d.L) level(kg * V + t);
         }
     } else {
         level(kg);
@@ -552,8 +553,14 @@ __global__ void __launch_bounds__(kBlock) k_theta_update(DevMesh m, DyPar d, Lev
 #pragma unroll
             for (int t = 0; t < V; t++) div[t] += cw[j] * a[t];
         }
+        const bool whole = k + V <= d.L;
         ldgv<V>(th + x, tk);
-        ldgv<V>(th_n + x, o);
+        if (whole) {
+            ldgv<V>(th_n + x, o);
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; t++) o[t] = k + t < d.L ? ldg(th_n + x + t) : 0.0;
+        }
         const TA above = k > 0 ? ldg(th + x - 1) : (TA)0, below = k + V < d.L ? ldg(th + x + V) : (TA)0;
 #pragma unroll
         for (int t = 0; t <= V; t++) {
@@ -565,7 +572,13 @@ __global__ void __launch_bounds__(kBlock) k_theta_update(DevMesh m, DyPar d, Lev
             const TA tend = -div[t] - (fl[t + 1] - fl[t]);
             o[t] = o[t] + dts * cv<double>(tend);
         }
-        stgv<V>(th_out + x, o);
+        if (whole) {
+            stgv<V>(th_out + x, o);
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; t++)
+                if (k + t < d.L) th_out[x + t] = o[t];
+        }
     } else {
 #pragma unroll
         for (int u = 0; u < 2; u++) {
@@ -753,7 +766,13 @@ __global__ void __launch_bounds__(kBlock) k_ke(DevMesh m, DyPar d, LevelDiv Dg, 
     for (int j = 0; j < GRIST_MAXE; j++) {
         const double w = ldg(m.kec2 + i * 6 + j);
         typename P::TU ue[V];
-        ldgv<V>(u + (size_t)e[j] * d.ld + k, ue);
+        const typename P::TU *uj = u + (size_t)e[j] * d.ld + k;
+        if (V == 1 || k + V <= d.L) {
+            ldgv<V>(uj, ue);
+        } else {
+#pragma unroll
+            for (int t = 0; t < V; t++) ue[t] = k + t < d.L ? ldg(uj + t) : (typename P::TU)0;
+        }
         if constexpr (sizeof(typename P::TU) == 4) {
             const MulF32 wm(w);
             if ((__double_as_longlong(w) << 1) == 0) continue;   // padding of a pentagon
@@ -1536,17 +1555,20 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gVH = grid_for((long long)m.nV * DH.d, kBlock);
-    // kinetic energy on 2 (binary32 wind: up to 4) levels where rows are whole,
-    // aligned vectors
+    // Vectors of levels where a row is whole, aligned vectors.  The last one may
+    // reach past the levels into the row's padding: of the scratch arrays, which
+    // have the caller's row length, it is read and written, of the caller's
+    // arrays it is not.
+    // Kinetic energy on 2 (binary32 wind: up to 4) levels
     constexpr int kKeV = sizeof(TU) == 4 ? 4 : 2;
-    auto ke_fits = [&](int v) { return L % v == 0 && ld % v == 0 && (uintptr_t)u % (v * sizeof(TU)) == 0; };
+    auto ke_fits = [&](int v) { return ld % v == 0 && (uintptr_t)u % (v * sizeof(TU)) == 0; };
     const int kev = kKeV == 4 && ke_fits(4) ? 4 : (ke_fits(2) ? 2 : 1);
-    const LevelDiv DK = make_div((uint32_t)(L / kev));
+    const LevelDiv DK = make_div((uint32_t)((L + kev - 1) / kev));
     const unsigned gK = grid_for((long long)m.nC * DK.d, kBlock);
-    // edge PV on 16-byte vectors of levels, or 8-byte ones, where rows are whole vectors
+    // edge PV on 16-byte vectors of levels, or 8-byte ones
     constexpr int kPvV = 16 / sizeof(TA), kPvH = sizeof(TA) == 4 ? 2 : 1;
-    const int pvv = L % kPvV == 0 && ld % kPvV == 0 ? kPvV : (L % kPvH == 0 && ld % kPvH == 0 ? kPvH : 1);
-    const LevelDiv DP = make_div((uint32_t)(L / pvv));
+    const int pvv = ld % kPvV == 0 ? kPvV : (ld % kPvH == 0 ? kPvH : 1);
+    const LevelDiv DP = make_div((uint32_t)((L + pvv - 1) / pvv));
     // theta update on the same vectors, the flux on binary32 quads, or two levels
     // half a column apart
     const bool quad = pvv == 4;
