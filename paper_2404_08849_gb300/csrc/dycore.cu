@@ -39,6 +39,7 @@ constexpr int kMassGroup = 8;
 struct DyPar {
     int L, ld, ldi;
     double pi_top, p0, rd, cp, g, beta, kappa, gamma;
+    double obeta, obetag;  // 1 - beta, (1 - beta) g
     const double *B;      // [L+1] interface coordinate
     const double *dB;     // [L]   layer thickness in B
     const double *rdB;    // [L]   1/dB
@@ -858,12 +859,14 @@ __device__ __forceinline__ double wind_diff(float a, float b) {
 // Bound by the FP64 pipe: the differences of p, phi and K between the edge's
 // cells and of u between levels are taken off it without changing a bit
 // (sub_near, wind_diff), 16 -> 11 FP64 instructions an edge-level in the mixed
-// policies; 40 registers, for six blocks an SM, since the loads' latency is
-// what is left.  Level 8, 60 levels, us a launch with k_pv_edge's: mixed
-// 3457 -> 2843; FP64, level 7, 3886 -> 2070.  Two or four levels a thread
-// (shared indices and M sums) measured slower: 2752 and 3370 against 2673.
+// policies; then the loads' latency is what is left, so every load is issued
+// before the first use, none behind a branch (2897 -> 2580 us below), with
+// six blocks of 256 an SM (4: 3079, 5: 2606, 7: 2784; GRIST_MIX_DF, without
+// FP64, eight: 110 -> 97 at level 6, 41 levels).  Level 8, 60 levels, us a launch
+// with k_pv_edge's: mixed 3457 -> 2750; FP64, level 7, 3886 -> 2070.  Two or
+// four levels a thread (shared indices and M sums) were slower: 2752 and 3370.
 template <class P, bool NH>
-__global__ void __launch_bounds__(kBlock, 6) k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
+__global__ void __launch_bounds__(kBlock, P::DF ? 8 : 6) k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
                            const typename P::TU *u_n, typename P::TU *u_out, const typename P::TM *__restrict__ F,
                            const typename P::TA *__restrict__ qv, const typename P::TA *__restrict__ G,
                            const double *__restrict__ K,
@@ -933,14 +936,17 @@ __global__ void __launch_bounds__(kBlock, 6) k_momentum(DevMesh m, DyPar d, Leve
         u_out[x] = (TU)v;
         return;
     }
-    const TU uk = ldg(u_s + x);
+    // every load before the first use, none behind a branch
+    const bool low = k < d.L - 1, high = k > 0;
+    const TU uk = ldg(u_s + x), ub = ldg(u_s + x + (low ? 1 : 0)), ut = ldg(u_s + x - (high ? 1 : 0)), un = u_n[x];
+    const double *M1 = Mv + (size_t)c.x * d.ldi + k, *M2 = Mv + (size_t)c.y * d.ldi + k;
+    const double mb1 = ldg(M1 + 1), mb2 = ldg(M2 + 1), mt1 = ldg(M1), mt2 = ldg(M2);
+    const double p1 = ldg(p + a1), p2 = ldg(p + a2), f1 = ldg(phl + a1), f2 = ldg(phl + a2), k1 = ldg(K + a1),
+                 k2 = ldg(K + a2), al1 = ldg(al + a1), al2 = ldg(al + a2);
+    const double d1 = NH ? ldg(dpp + a1) : 1.0, d2 = NH ? ldg(dpp + a2) : 1.0;
     double va = 0.0;
-    if (k < d.L - 1)
-        va = (ldg(Mv + (size_t)c.x * d.ldi + k + 1) + ldg(Mv + (size_t)c.y * d.ldi + k + 1)) *
-             wind_diff(ldg(u_s + x + 1), uk);
-    if (k > 0)
-        va = fma(ldg(Mv + (size_t)c.x * d.ldi + k) + ldg(Mv + (size_t)c.y * d.ldi + k),
-                 wind_diff(uk, ldg(u_s + x - 1)), va);
+    if (low) va = (mb1 + mb2) * wind_diff(ub, uk);
+    if (high) va = fma(mt1 + mt2, wind_diff(uk, ut), va);
     // [M sums](du) / (2 dpi_e) with dpi_e = dB (sum)/2, M_e = (M1 + M2)/2;
     // rsum_e holds 1/(2 sum)
     va *= ldg(d.rdB + k) * ldg(rsum_e + e);
@@ -949,23 +955,22 @@ __global__ void __launch_bounds__(kBlock, 6) k_momentum(DevMesh m, DyPar d, Leve
     // into -1/(2 dc) (hrdc) and K stored doubled
     double grad;
     if (!P::EMU || !(d.emu & GRIST_ROW_PGF)) {
-        const double de = NH ? ldg(dpp + a1) + ldg(dpp + a2) : 2.0;
-        grad = fma(ldg(al + a1) + ldg(al + a2), sub_near(ldg(p + a2), ldg(p + a1)),
-                   fma(de, sub_near(ldg(phl + a2), ldg(phl + a1)), sub_near(ldg(K + a2), ldg(K + a1))));
+        const double de = NH ? d1 + d2 : 2.0;
+        grad = fma(al1 + al2, sub_near(p2, p1), fma(de, sub_near(f2, f1), sub_near(k2, k1)));
     } else {
         // pressure gradient and gravity from binary32 inputs, summed and
         // rounded to binary32 (precision search)
         const uint32_t r = GRIST_ROW_PGF;
-        const double de = NH ? emu<P::EMU>(ldg(dpp + a1), d.emu, r) + emu<P::EMU>(ldg(dpp + a2), d.emu, r) : 2.0;
-        const double pgf = emu<P::EMU>(fma(emu<P::EMU>(ldg(al + a1), d.emu, r) + emu<P::EMU>(ldg(al + a2), d.emu, r),
-                                   emu<P::EMU>(ldg(p + a2), d.emu, r) - emu<P::EMU>(ldg(p + a1), d.emu, r),
-                                   de * (emu<P::EMU>(ldg(phl + a2), d.emu, r) - emu<P::EMU>(ldg(phl + a1), d.emu, r))),
-                               d.emu, r);
-        grad = pgf + (ldg(K + a2) - ldg(K + a1));
+        const double de = NH ? emu<P::EMU>(d1, d.emu, r) + emu<P::EMU>(d2, d.emu, r) : 2.0;
+        const double pgf = emu<P::EMU>(fma(emu<P::EMU>(al1, d.emu, r) + emu<P::EMU>(al2, d.emu, r),
+                                           emu<P::EMU>(p2, d.emu, r) - emu<P::EMU>(p1, d.emu, r),
+                                           de * (emu<P::EMU>(f2, d.emu, r) - emu<P::EMU>(f1, d.emu, r))),
+                                       d.emu, r);
+        grad = pgf + (k2 - k1);
     }
     const double slow = fma(ldg(m.hrdc + e), grad, -va);
     const TA tend = emu<P::EMU>(pv, d.emu, GRIST_ROW_PV_FLUX) + cv<TA>(slow);
-    const TU v = emu<P::EMU>(cv<TU>(cv<TA>(u_n[x]) + cv<TA>(dts) * tend), d.emu, GRIST_ROW_WIND);
+    const TU v = emu<P::EMU>(cv<TU>(cv<TA>(un) + cv<TA>(dts) * tend), d.emu, GRIST_ROW_WIND);
     if (!isfinite(v)) atomicOr(status, GRIST_FLAG_NONFINITE);
     u_out[x] = v;
 }
@@ -1011,9 +1016,13 @@ __device__ __forceinline__ float adv_diff(const AdvVal<float> &a, const AdvVal<f
 // input (advective type; the differences of the FP64 fields are formed to
 // about 2^-24 of themselves before the rounding to that type), plus the (1 - beta) share of g (dp/dpi - 1) and g w at t^n.  The
 // t^n forcing g (dp/dpi - 1) is formed in the first stage (FIRST) from the
-// t^n pressure and kept for the later stages.
+// t^n pressure and kept for the later stages.  The binary32 form is bound by
+// the integer pipe (the splits), the FP64 form by the FP64 pipe; the cell's row
+// is read as vectors and the factors 1/2 of u and of the difference are taken
+// out of the sums.  Level 8, 60 levels, mixed 1107 -> 1042 us a launch (five
+// blocks of 256 an SM; 4: 1176, 6: 1218); FP64, level 7, 1184 -> 913.
 template <class P, bool FIRST>
-__global__ void k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
+__global__ void __launch_bounds__(kBlock, 5) k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
                               const double *__restrict__ rdps_s, const double *__restrict__ Mv,
                               const double *__restrict__ w_s, const double *__restrict__ phi_s,
                               const double *__restrict__ w_n, const double *__restrict__ phi_n,
@@ -1032,17 +1041,19 @@ __global__ void k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P:
         return;
     }
     const AdvVal<TA> wi(w_s[xi]), pi(phi_s[xi]);
+    // sums of cdiv (u_{j-1} + u_j) dx: four times the advection (exact scalings
+    // of its terms, taken out of the loop)
     TA hw = 0, hp = 0;
+    int e[GRIST_MAXE], nb[GRIST_MAXE];
+    TA cw[GRIST_MAXE];
+    load_row6(m.eoc8, i, e);
+    load_row6(m.coc8, i, nb);
+    load_row6(Coef<TA>::cdiv8(m), i, cw);
 #pragma unroll
     for (int s = 0; s < GRIST_MAXE; s++) {
-        const int e = ldg(m.eoc + i * 6 + s);
-        const int nb = ldg(m.coc + i * 6 + s);
-        TA ui;
-        const size_t ue = (size_t)e * d.ld;
-        if (j == 0) ui = cv<TA>(ldg(u_s + ue));
-        else ui = (TA)0.5 * (cv<TA>(ldg(u_s + ue + j - 1)) + cv<TA>(ldg(u_s + ue + j)));
-        const TA cu = ldg(Coef<TA>::cdiv(m) + i * 6 + s) * ui * (TA)0.5;
-        const size_t y = (size_t)nb * d.ldi + j;
+        const size_t ue = (size_t)e[s] * d.ld + j, y = (size_t)nb[s] * d.ldi + j;
+        const TA ub = cv<TA>(ldg(u_s + ue)), ut = j == 0 ? ub : cv<TA>(ldg(u_s + ue - 1));
+        const TA cu = cw[s] * (ut + ub);
         hw += cu * adv_diff(AdvVal<TA>(ldg(w_s + y)), wi);
         hp += cu * adv_diff(AdvVal<TA>(ldg(phi_s + y)), pi);
     }
@@ -1061,8 +1072,9 @@ __global__ void k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P:
             fw = fw_n[xi];
         }
     }
-    wst[xi] = w_n[xi] + dts * (cv<double>(emu<P::EMU>(-hw - vw, d.emu, GRIST_ROW_NH_ADV)) + (1.0 - d.beta) * fw);
-    phst[xi] = phi_n[xi] + dts * (cv<double>(emu<P::EMU>(-hp - vp, d.emu, GRIST_ROW_NH_ADV)) + (1.0 - d.beta) * d.g * w_n[xi]);
+    const TA q = (TA)0.25;
+    wst[xi] = w_n[xi] + dts * (cv<double>(emu<P::EMU>(-q * hw - vw, d.emu, GRIST_ROW_NH_ADV)) + d.obeta * fw);
+    phst[xi] = phi_n[xi] + dts * (cv<double>(emu<P::EMU>(-q * hp - vp, d.emu, GRIST_ROW_NH_ADV)) + d.obetag * w_n[xi]);
 }
 
 // Staging of a [32 columns][kSolveKC levels] tile between global memory
@@ -1522,7 +1534,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     DyPar d;
     d.L = L; d.ld = ld; d.ldi = ldi;
     d.pi_top = prm->pi_top; d.p0 = prm->p0; d.rd = prm->rd; d.cp = prm->cp; d.g = prm->g;
-    d.beta = prm->offcentre_beta; d.kappa = prm->rd / prm->cp; d.gamma = prm->cp / (prm->cp - prm->rd);
+    d.beta = prm->offcentre_beta; d.obeta = 1.0 - d.beta; d.obetag = d.obeta * d.g; d.kappa = prm->rd / prm->cp; d.gamma = prm->cp / (prm->cp - prm->rd);
     d.B = dvg; d.dB = dvg + L + 1; d.rdB = dvg + 2 * L + 1; d.hrdBi = dvg + 3 * L + 1; d.dBi = dvg + 4 * L + 2;
     d.phis = prm->phi_surface;
     d.Bm = dvg + 5 * L + 3;
