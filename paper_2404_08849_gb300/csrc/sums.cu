@@ -23,10 +23,16 @@ struct DD {
     double s, c;  // value = s + c (c carries the accumulated rounding error)
 };
 
+// Neumaier's step: the smaller of the two by magnitude goes through the
+// rounding error.  The magnitudes are compared as integers and selected, so
+// the FP64 pipe, which bounds the sums, carries four additions (a branch on an
+// FP64 comparison issues both of its sides in a warp of mixed lanes).
 __device__ __forceinline__ void neumaier(DD &a, double v) {
     const double t = a.s + v;
-    if (fabs(a.s) >= fabs(v)) a.c += (a.s - t) + v;
-    else a.c += (v - t) + a.s;
+    const unsigned long long ms = (unsigned long long)__double_as_longlong(a.s) << 1,
+                             mv = (unsigned long long)__double_as_longlong(v) << 1;
+    const double big = ms >= mv ? a.s : v, small = ms >= mv ? v : a.s;
+    a.c += (big - t) + small;
     a.s = t;
 }
 
@@ -64,13 +70,13 @@ __global__ void k_sum_partial(DevMesh m, int kind, const T *__restrict__ x, cons
     for (long long r = (long long)blockIdx.x * kSumThreads + threadIdx.x; r < n; r += stride) {
         double v;
         if (kind == 0) {
-            v = ldg(m.area + r) * ((double)x[r] - offset);
+            v = ldg(m.area + r) * (cv<double>(x[r]) - offset);
         } else {
             int i, k;
             split_index((uint32_t)r, Dv, i, k);
             const size_t y = (size_t)i * ld + k;
             const double w = kind == 1 ? ldg(m.area + i) * dpi[y] : ldg(m.area + i);
-            v = w * (double)x[y];
+            v = w * cv<double>(x[y]);
         }
         neumaier(acc, v);
     }

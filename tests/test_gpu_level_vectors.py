@@ -52,3 +52,26 @@ def test_same_bits_at_every_width(mesh_cache, prec, nh, L):
             assert torch.equal(ref[k], got[k]), (k, pad, shift)
     assert mesh.last_status() == 0
     mesh.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mix"])
+@pytest.mark.parametrize("L,pad", [(1, 0), (4, 0), (6, 0), (7, 1), (8, 1), (60, 0)])
+def test_vorticity_at_every_width(mesh_cache, prec, L, pad):
+    """Against numpy: 3 products and 2 sums of FP64, so a few ulp of the terms."""
+    import torch
+    import paper_2404_08849_gb300 as G
+    m = mesh_cache(3)
+    mesh = G.Mesh(m)
+    rng = np.random.default_rng(L)
+    u = rng.standard_normal((m["n_edges"], L)) * 10.0
+    u = u if prec == "fp64" else u.astype(np.float32)
+    rows = np.full((m["n_edges"], L + pad), np.nan, u.dtype)
+    rows[:, :L] = mesh.to_internal(u, "edge", 0)
+    vor = mesh.vorticity(torch.from_numpy(rows).cuda(), L)
+    torch.cuda.synchronize()
+    got = mesh.from_internal(vor.cpu().numpy()[:, :L], "vertex", 0)
+    ev = m["edges_on_vertex"]
+    w = m["edge_sign_on_vertex"] * m["edge_dc"][ev] / m["vertex_area"][:, None]
+    terms = w[:, :, None] * u[ev].astype(np.float64)
+    assert np.all(np.abs(got - terms.sum(1)) <= 8 * np.finfo(float).eps * np.abs(terms).sum(1))
+    mesh.close()
