@@ -483,6 +483,12 @@ const HostTables &host_tables(grist_mesh_s *m);
 std::vector<double> &vg_cache(grist_mesh_s *m);
 const void *&vg_ptr(grist_mesh_s *m);
 
+// The dycore's side streams, each with its fork and join event, made on first
+// use; false if they could not be.  They belong to the handle: two dycore
+// steps of one handle never overlap.
+constexpr int kSides = 2;
+bool side_stream(grist_mesh_s *m, int which, cudaStream_t *s, cudaEvent_t **ev);
+
 // Tracer-step context (tuning, device tables, graph cache) kept in the
 // handle; defined in tracer.cu.
 struct TracerCtx;

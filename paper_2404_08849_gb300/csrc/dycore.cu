@@ -1481,6 +1481,44 @@ __global__ void k_add_scalar(double *x, double v) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *x += v;
 }
 
+// Where the wind's diagnostics go in the NH core: beside the mass kernels from
+// the start of the stage, or beside the column solve.  Small meshes leave SMs
+// idle all along and gain from the early start (10,242 cells: 464 against 484
+// us a step); on large ones every kernel fills the GPU and the solve, with a
+// third of the warps and waiting for its chains, is what can take them
+// (163,842 cells, FP64: 16953 against 17128; 655,362, mixed: 28667, 28775;
+// 40,962 equal).
+inline bool wind_beside_solve(int nC) { return nC > 100000; }
+
+// One side stream of a dycore step: work on s after fork(k) follows what st has
+// so far; join(k) makes st wait for all of s so far.  Every fork is joined
+// before the step returns, also on an error, so that the caller's buffers are
+// used on st's order only and a capture of st takes the side stream in and
+// gives it back.  While kernels are timed one by one, or without the stream,
+// s is st itself.
+struct Side {
+    cudaStream_t st, s;
+    cudaEvent_t *ev;
+    bool on, open = false;
+    Side(grist_mesh_s *h, int which, cudaStream_t st_) : st(st_), s(st_), ev(nullptr), on(false) {
+        if (!profiling(h)) on = side_stream(h, which, &s, &ev);
+        if (!on) s = st;
+    }
+    ~Side() { if (open) join(); }
+    void fork() {
+        if (!on) return;
+        cudaEventRecord(ev[0], st);
+        cudaStreamWaitEvent(s, ev[0], 0);
+        open = true;
+    }
+    void join() {
+        if (!open) return;
+        cudaEventRecord(ev[1], s);
+        cudaStreamWaitEvent(st, ev[1], 0);
+        open = false;
+    }
+};
+
 template <class P, bool NH>
 int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_params *prm, double dt, cudaStream_t st) {
     using TU = typename P::TU;
@@ -1631,6 +1669,11 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             d, ex.base, (double2 *)(s + o_ex)));
     }
 
+    auto edge_pv = [&](cudaStream_t sw) {
+        GRIST_LAUNCH(h, PN("k_pv_edge"), sw, (pvv == kPvV   ? k_pv_edge<P, kPvV>
+                                              : pvv == kPvH ? k_pv_edge<P, kPvH>
+                                                            : k_pv_edge<P, 1>)<<<gP, kBlock, 0, sw>>>(m, d, DP, F, qv, Gq));
+    };
     double *p_outs[3] = {p, p, (NH && S->p_nh) ? S->p_nh : p};
 
     const TU *u_in = u;
@@ -1640,25 +1683,59 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     double *th_outs[3] = {thA, thB, S->dpi_theta};
     double *w_outs[3] = {wA, wB, S->w};
     double *phi_outs[3] = {phA, phB, S->phi};
+    // Two chains of a stage do not depend on each other until the column solve
+    // or the momentum equation: mass -> theta (-> column), and the wind's
+    // diagnostics (vertex PV, edge PV, kinetic energy) of the stage input; in
+    // the NH core the advection of w and phi needs the mass kernels only.
+    // They run on side streams of the handle, forked and joined by events.  us a
+    // step in one chain / with them: level 5 coupled, 30 levels, recorded 506 /
+    // 464; level 6 hydrostatic, 30 levels, mixed 1686 / 1589, FP64 1880 / 1802;
+    // level 6 NH, 41 levels 1606 / 1446; level 7 FP64 NH 17277 / 16953; level 8
+    // mixed NH 28962 / 28667.
+    Side sw_(h, 0, st), sx_(h, 1, st);   // the wind's diagnostics, the advection
+    const bool late = NH && wind_beside_solve(m.nC);
     for (int s3 = 0; s3 < 3; s3++) {
         const double h3 = dts[s3];
+        auto wind = [&](cudaStream_t sw) {
+            GRIST_LAUNCH(h, PN("k_vertex_mass"), sw, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, sw>>>(m, d, ps_in, rdpv));
+            GRIST_LAUNCH(h, PN("k_vort"), sw, k_vort<P><<<gVH, kBlock, 0, sw>>>(m, d, DH, u_in, rdpv, qv));
+            GRIST_LAUNCH(h, PN("k_ke"), sw, (kev == 4   ? k_ke<P, kKeV>
+                                             : kev == 2 ? k_ke<P, 2>
+                                                        : k_ke<P, 1>)<<<gK, kBlock, 0, sw>>>(m, d, DK, u_in, K));
+            if (!short_forms<P>()) edge_pv(sw);
+        };
+        auto explicit_part = [&](cudaStream_t sw) {
+            if (s3 == 0)
+                GRIST_LAUNCH(h, PN("k_nh_explicit"), sw, k_nh_explicit<P, true><<<gI, kBlock, 0, sw>>>(
+                    m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
+            else
+                GRIST_LAUNCH(h, PN("k_nh_explicit"), sw, k_nh_explicit<P, false><<<gI, kBlock, 0, sw>>>(
+                    m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
+        };
+        if (!late || !NH) {
+            sw_.fork();
+            wind(sw_.s);
+        }
         GRIST_LAUNCH(h, PN("k_mass_edge"), st, k_mass_edge<P><<<gEG, kBlock, 0, st>>>(
             m, d, ps_in, u_in, F, s3 == 2 ? S->mass_flux_accum : nullptr, ascale, rsum, fcol));
         GRIST_LAUNCH(h, PN("k_mass_col"), st, k_mass_col<P><<<gCG, kBlock, 0, st>>>(
             m, d, F, fcol, ps_in, psN, ps_outs[s3], th_in, theta, Mv, h3, s3 == 0 ? S->dpi_start : nullptr, rdps,
             (NH && s3 == 0) ? rthn : nullptr, dphn, S->phi, s3 == 2 ? S->vmass_flux_accum : nullptr, ascale));
+        if (NH) {
+            sx_.fork();
+            explicit_part(sx_.s);
+        }
         GRIST_LAUNCH(h, PN("k_theta_flux"), st, (quad ? k_theta_flux<P, sizeof(TA) == 4 ? 4 : 1> : k_theta_flux<P, 1>)<<<gEH, kBlock, 0, st>>>(m, d, DT, F, theta, Fth));
         GRIST_LAUNCH(h, PN("k_theta_update"), st, (thv == kPvV   ? k_theta_update<P, kPvV>
                                                    : thv == kPvH ? k_theta_update<P, kPvH>
                                                                  : k_theta_update<P, 1>)<<<gCT, kBlock, 0, st>>>(
             m, d, DTU, Fth, theta, Mv, S->dpi_theta, th_outs[s3], h3));
         if (NH) {
-            if (s3 == 0)
-                GRIST_LAUNCH(h, PN("k_nh_explicit"), st, k_nh_explicit<P, true><<<gI, kBlock, 0, st>>>(
-                    m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
-            else
-                GRIST_LAUNCH(h, PN("k_nh_explicit"), st, k_nh_explicit<P, false><<<gI, kBlock, 0, st>>>(
-                    m, d, DI, u_in, rdps, Mv, w_in, phi_in, S->w, S->phi, p_n, fwn, wst, phst, h3));
+            sx_.join();
+            if (late) {
+                sw_.fork();
+                wind(sw_.s);
+            }
             cudaError_t se = cudaSuccess;
             GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, short_forms<P>()>(
                 m, d, DL, wst, phst, th_outs[s3], rthn, dphn, p_n, ps_outs[s3], h3, w_outs[s3], phi_outs[s3], p_outs[s3],
@@ -1668,14 +1745,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF, short_forms<P>()><<<gW, kBlock, 0, st>>>(
                 m, d, ex, bkap, ps_outs[s3], th_outs[s3], p, alp, phl));
         }
-        GRIST_LAUNCH(h, PN("k_vertex_mass"), st, k_vertex_mass<P::EMU><<<gVx, kBlock, 0, st>>>(m, d, ps_in, rdpv));
-        GRIST_LAUNCH(h, PN("k_vort"), st, k_vort<P><<<gVH, kBlock, 0, st>>>(m, d, DH, u_in, rdpv, qv));
-        GRIST_LAUNCH(h, PN("k_ke"), st, (kev == 4   ? k_ke<P, kKeV>
-                                         : kev == 2 ? k_ke<P, 2>
-                                                    : k_ke<P, 1>)<<<gK, kBlock, 0, st>>>(m, d, DK, u_in, K));
-        GRIST_LAUNCH(h, PN("k_pv_edge"), st, (pvv == kPvV   ? k_pv_edge<P, kPvV>
-                                              : pvv == kPvH ? k_pv_edge<P, kPvH>
-                                                            : k_pv_edge<P, 1>)<<<gP, kBlock, 0, st>>>(m, d, DP, F, qv, Gq));
+        sw_.join();
+        if (short_forms<P>()) edge_pv(st);   // 2 F q_e: after the mass flux
         GRIST_LAUNCH(h, PN("k_momentum"), st, k_momentum<P, NH><<<gE, kBlock, 0, st>>>(
             m, d, DL, u_in, u, u_outs[s3], F, qv, Gq, K, Mv, rsum, p_outs[s3], alp, phl, dpp, h3, status));
         u_in = u_outs[s3];

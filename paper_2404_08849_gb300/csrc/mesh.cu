@@ -28,6 +28,10 @@ struct grist_mesh_s {
     // the dycore's vertical-grid table as last uploaded, and where
     std::vector<double> vg_cache;
     const void *vg_ptr = nullptr;
+    // the dycore's side streams (0 not made, 1 made, -1 could not be)
+    int side_state = 0;
+    cudaStream_t side[kSides] = {nullptr};
+    cudaEvent_t side_ev[kSides][2] = {{nullptr}};
     // profiling
     bool prof_on = false;
     std::vector<cudaEvent_t> ev;            // pool, pairs (2j, 2j+1)
@@ -46,6 +50,21 @@ TracerCtx *&tracer_ctx(grist_mesh_s *m) { return m->tctx; }
 const HostTables &host_tables(grist_mesh_s *m) { return m->ht; }
 std::vector<double> &vg_cache(grist_mesh_s *m) { return m->vg_cache; }
 const void *&vg_ptr(grist_mesh_s *m) { return m->vg_ptr; }
+
+bool side_stream(grist_mesh_s *m, int which, cudaStream_t *s, cudaEvent_t **ev) {
+    if (m->side_state == 0) {
+        bool ok = true;
+        for (int i = 0; i < kSides; i++) {
+            ok = ok && cudaStreamCreateWithFlags(&m->side[i], cudaStreamNonBlocking) == cudaSuccess;
+            for (auto &e : m->side_ev[i]) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+        }
+        m->side_state = ok ? 1 : -1;
+        if (!ok) cudaGetLastError();
+    }
+    *s = m->side[which];
+    *ev = m->side_ev[which];
+    return m->side_state == 1;
+}
 
 static const int kEventPairs = 4096;
 
@@ -520,6 +539,11 @@ extern "C" int grist_mesh_destroy(grist_mesh m) {
     cudaSetDevice(m->device);
     cudaDeviceSynchronize();
     for (auto &e : m->ev) cudaEventDestroy(e);
+    for (int i = 0; i < kSides; i++) {
+        for (auto &e : m->side_ev[i])
+            if (e) cudaEventDestroy(e);
+        if (m->side[i]) cudaStreamDestroy(m->side[i]);
+    }
     tracer_ctx_free(m->tctx);
     for (int s = 0; s < 8; s++)
         if (m->scr[s]) cudaFree(m->scr[s]);
