@@ -40,6 +40,7 @@ struct DyPar {
     int L, ld, ldi;
     double pi_top, p0, rd, cp, g, beta, kappa, gamma;
     double obeta, obetag;  // 1 - beta, (1 - beta) g
+    double rp0;            // 1/p0, or 0 where p/p0 has to be divided
     const double *B;      // [L+1] interface coordinate
     const double *dB;     // [L]   layer thickness in B
     const double *rdB;    // [L]   1/dB
@@ -637,54 +638,81 @@ __global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
 // Bound by the FP64 pipe: about 24 instructions a cell-level with the table
 // above (SHORT, see short_forms) against about 130 with pow(); level-6 mesh,
 // 30 levels: 323 -> 76 us a launch, plus 10 us a step for the table.
+// With pow() a warp takes two columns, so that the correctly rounded
+// 1/dps runs one column per lane, p/p0 is the product with 1/p0 corrected by its
+// remainder (the correctly rounded quotient: rp0 is correctly rounded and p0's
+// significand not all ones, which the host checks) and the pressure below is the
+// next lane's above: the same bits.  Level 6, 30 levels, us a mixed step by
+// columns: 1 1556, 2 1526, 4 1564, 8 1660 (1590 before).
+template <bool SHORT> constexpr int diag_cols() { return SHORT ? 1 : 2; }
 template <bool EMU, bool DF, bool SHORT>
-__global__ void k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const double *__restrict__ ps,
+__global__ void __launch_bounds__(kBlock) k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const double *__restrict__ ps,
                              const double *__restrict__ th, double *__restrict__ p, double *__restrict__ al,
                              double *__restrict__ phl) {
-    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    constexpr int C = diag_cols<SHORT>();
+    const int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * C;
     const int lane = threadIdx.x & 31;
-    if (i >= m.nC) return;
-    const double dps = ps[i] - d.pi_top;
-    const double rdps = SHORT ? rcp_nr(dps) : rcp(dps);
-    const int nch = (d.L + 31) >> 5;
-    const int bin = SHORT ? (__double2hiint(dps) >> 13) - ex.base : -1;
-    const bool tabled = bin >= 0 && bin < kExnerBins;   // the same for the whole warp
-    const double off = SHORT ? dps - exner_centre(ex.base, bin) : 0.0;
-    const double2 *row = ex.tab + (size_t)(tabled ? bin : 0) * d.L;
-    double carry = ldg(d.phis + i);
-    for (int ch = nch - 1; ch >= 0; ch--) {
-        const int k = ch * 32 + lane;
-        double contrib = 0.0, a = 0.0, pk = 0.0;
-        if (k < d.L) {
-            const double thk = th[(size_t)i * d.ld + k];
+    if (i0 >= m.nC) return;
+    double dps_l = 0.0, rdps_l = 0.0;
+    if (!SHORT && i0 + lane < m.nC && lane < C) {
+        dps_l = ps[i0 + lane] - d.pi_top;
+        rdps_l = rcp(dps_l);
+    }
+    const int nch = (d.L + 31) >> 5, ncol = min(C, m.nC - i0);
+#pragma unroll 1
+    for (int c = 0; c < ncol; c++) {
+        const int i = i0 + c;
+        const double dps = SHORT ? ps[i] - d.pi_top : __shfl_sync(0xffffffffu, dps_l, c);
+        const double rdps = SHORT ? rcp_nr(dps) : __shfl_sync(0xffffffffu, rdps_l, c);
+        const int bin = SHORT ? (__double2hiint(dps) >> 13) - ex.base : -1;
+        const bool tabled = bin >= 0 && bin < kExnerBins;   // the same for the whole warp
+        const double off = SHORT ? dps - exner_centre(ex.base, bin) : 0.0;
+        const double2 *row = ex.tab + (size_t)(tabled ? bin : 0) * d.L;
+        double carry = ldg(d.phis + i);
+        for (int ch = nch - 1; ch >= 0; ch--) {
+            const int k = ch * 32 + lane;
+            double contrib = 0.0, a = 0.0, pk = 0.0;
             if (tabled) {
-                const double2 r = ldg(row + k);
-                pk = fma(ldg(d.Bm + k), dps, d.pi_top);
-                contrib = thk * (r.x * horner_tail<4, 8>(r.y * off, bk));   // alpha dpi
-                a = contrib * (ldg(d.rdB + k) * rdps);
+                if (k < d.L) {
+                    const double2 r = ldg(row + k);
+                    pk = fma(ldg(d.Bm + k), dps, d.pi_top);
+                    contrib = th[(size_t)i * d.ld + k] * (r.x * horner_tail<4, 8>(r.y * off, bk));   // alpha dpi
+                    a = contrib * (ldg(d.rdB + k) * rdps);
+                }
             } else {
-                const double pt = d.pi_top + ldg(d.B + k) * dps, pb = d.pi_top + ldg(d.B + k + 1) * dps;
-                const double dp = pb - pt;
-                pk = 0.5 * (pt + pb);
-                a = d.rd * (thk * ldg(d.rdB + k) * rdps) * pow(pk / d.p0, d.kappa) / pk;
-                contrib = a * dp;
+                const double pt = d.pi_top + ldg(d.B + min(k, d.L)) * dps;
+                double pb = __shfl_down_sync(0xffffffffu, pt, 1);
+                if (lane == 31 && k < d.L) pb = d.pi_top + ldg(d.B + k + 1) * dps;
+                if (k < d.L) {
+                    const double dp = sub_near(pb, pt);
+                    pk = 0.5 * (pt + pb);
+                    double q;
+                    if (d.rp0 != 0.0) {
+                        q = pk * d.rp0;
+                        q = fma(fma(-q, d.p0, pk), d.rp0, q);
+                    } else {
+                        q = pk / d.p0;
+                    }
+                    a = d.rd * (th[(size_t)i * d.ld + k] * ldg(d.rdB + k) * rdps) * pow(q, d.kappa) / pk;
+                    contrib = a * dp;
+                }
             }
-        }
-        // inclusive suffix sum within the chunk
-        double v = contrib;
+            // inclusive suffix sum within the chunk
+            double v = contrib;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            double t = __shfl_down_sync(0xffffffffu, v, o);
-            if (lane + o < 32) v += t;
+            for (int o = 1; o < 32; o <<= 1) {
+                double t = __shfl_down_sync(0xffffffffu, v, o);
+                if (lane + o < 32) v += t;
+            }
+            if (k < d.L) {
+                const size_t x = (size_t)i * d.ld + k;
+                p[x] = emu<EMU>(pk, d.emu, GRIST_ROW_EOS);
+                al[x] = emu<EMU>(a, d.emu, GRIST_ROW_EOS);
+                const double ph = SHORT ? carry + fma(-0.5, contrib, v) : carry + (v - contrib) + 0.5 * contrib;
+                phl[x] = DF ? pack_split(ph) : emu<EMU>(ph, d.emu, GRIST_ROW_EOS);
+            }
+            carry += __shfl_sync(0xffffffffu, v, 0);
         }
-        if (k < d.L) {
-            const size_t x = (size_t)i * d.ld + k;
-            p[x] = emu<EMU>(pk, d.emu, GRIST_ROW_EOS);
-            al[x] = emu<EMU>(a, d.emu, GRIST_ROW_EOS);
-            const double ph = SHORT ? carry + fma(-0.5, contrib, v) : carry + (v - contrib) + 0.5 * contrib;
-            phl[x] = DF ? pack_split(ph) : emu<EMU>(ph, d.emu, GRIST_ROW_EOS);
-        }
-        carry += __shfl_sync(0xffffffffu, v, 0);
     }
 }
 
@@ -1585,6 +1613,13 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     DyPar d;
     d.L = L; d.ld = ld; d.ldi = ldi;
     d.pi_top = prm->pi_top; d.p0 = prm->p0; d.rd = prm->rd; d.cp = prm->cp; d.g = prm->g;
+    {
+        // p/p0 by the corrected product needs p0 and the quotient away from the
+        // ends of the range, and a significand other than all ones
+        int e2 = 0;
+        const double f = std::isfinite(prm->p0) ? std::frexp(prm->p0, &e2) : 0.0;
+        d.rp0 = std::isfinite(prm->p0) && std::abs(e2) < 200 && f != 1.0 - 0x1p-53 ? 1.0 / prm->p0 : 0.0;
+    }
     d.beta = prm->offcentre_beta; d.obeta = 1.0 - d.beta; d.obetag = d.obeta * d.g; d.kappa = prm->rd / prm->cp; d.gamma = prm->cp / (prm->cp - prm->rd);
     d.B = dvg; d.dB = dvg + L + 1; d.rdB = dvg + 2 * L + 1; d.hrdBi = dvg + 3 * L + 1; d.dBi = dvg + 4 * L + 2;
     d.phis = prm->phi_surface;
@@ -1613,7 +1648,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     uint32_t *status = status_word(h);
     const LevelDiv DL = make_div((uint32_t)L), DI = make_div((uint32_t)(L + 1)), DH = make_div((uint32_t)(L + 1) / 2);
     const unsigned gC = grid_for((long long)m.nC * L, kBlock),
-                   gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for((long long)m.nC * 32, kBlock),
+                   gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for(((long long)m.nC + diag_cols<short_forms<P>()>() - 1) / diag_cols<short_forms<P>()>() * 32, kBlock),
                    gI = grid_for((long long)m.nC * (L + 1), kBlock),
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock),
