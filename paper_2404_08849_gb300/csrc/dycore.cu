@@ -7,15 +7,17 @@
 // layer mass in FP64.
 //
 // Layer fields [entity][ld], interface fields [cell][ld_int]; one thread per
-// (entity, level) for the horizontal stencils, one warp per column for the
-// vertical scans (continuity prefix, hydrostatic integral) and one thread
-// per column for the tridiagonal solve.
+// (entity, level) or vector of levels for the horizontal stencils, a warp's
+// lanes over the levels of a column for the vertical scans (continuity prefix,
+// hydrostatic integral) and one thread per column for the tridiagonal solve.
 //
 // FP64 arithmetic is the scarce resource on this GPU (about 1/60 of the FP32
-// rate), so divisions by layer masses are replaced by products with
+// rate: an FP64 instruction of a warp holds its scheduler's pipe for 64
+// cycles), so divisions by layer masses are replaced by products with
 // reciprocals formed once per column / edge / vertex (1/(ps - pi_top)) and
-// once per level (1/dB), and the equation of state inside a stage is
-// evaluated relative to the stage-input state (see pow1p_near0).
+// once per level (1/dB), the equation of state inside a stage is evaluated
+// relative to the stage-input state (see pow1p_near0), and exact differences
+// and products are taken in integers (sub_near, MulF32).
 #include <cmath>
 #include <type_traits>
 #include <vector>
@@ -441,6 +443,14 @@ __global__ void __launch_bounds__(kBlock) k_mass_col(DevMesh m, DyPar d, const t
     }
 }
 
+// f >= 0, for binary64 from the bits (an FP64 comparison holds the FP64 pipe
+// like an addition); -0 counts as 0, NaN by its sign.
+__device__ __forceinline__ bool runs_to_c2(float f) { return f >= 0.f; }
+__device__ __forceinline__ bool runs_to_c2(double f) {
+    const long long b = __double_as_longlong(f);
+    return b >= 0 || (b << 1) == 0;
+}
+
 // Eq. 4 horizontal flux: third-order upwind (beta = 1) edge value of theta
 // times the mass flux.  V = 4 (binary32): a thread takes four consecutive levels
 // of one edge as vectors, with one read of the upwind stencil row (4 vector
@@ -464,7 +474,7 @@ __global__ void __launch_bounds__(kBlock) k_theta_flux(DevMesh m, DyPar d, Level
     auto level = [&](int k) {
         const size_t x = (size_t)e * d.ld + k;
         const TA f = cv<TA>(F[x]);
-        const int side = f >= (TA)0 ? 0 : 1;
+        const int side = runs_to_c2(f) ? 0 : 1;
         TA te;
         if (m.d2w_ok) {
             // one weighted sum over the upwind side's stencil (the mean of
@@ -868,7 +878,7 @@ __global__ void __launch_bounds__(kBlock) k_pv_edge(DevMesh m, DyPar d, LevelDiv
 
 // (double)a - (double)b of two binary32 numbers, bit for bit: where the binary32
 // difference is exact (its TwoSum error is zero) it is that number.
-__device__ __forceinline__ double wind_diff(double a, double b) { return a - b; }
+__device__ __forceinline__ double wind_diff(double a, double b) { return sub_near(a, b); }
 __device__ __forceinline__ double wind_diff(float a, float b) {
     const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
     const float err = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
@@ -891,7 +901,7 @@ __device__ __forceinline__ double wind_diff(float a, float b) {
 // before the first use, none behind a branch (2897 -> 2580 us below), with
 // six blocks of 256 an SM (4: 3079, 5: 2606, 7: 2784; GRIST_MIX_DF, without
 // FP64, eight: 110 -> 97 at level 6, 41 levels).  Level 8, 60 levels, us a launch
-// with k_pv_edge's: mixed 3457 -> 2750; FP64, level 7, 3886 -> 2070.  Two or
+// with k_pv_edge's: mixed 3457 -> 2750; FP64, level 7, 3886 -> 1990.  Two or
 // four levels a thread (shared indices and M sums) were slower: 2752 and 3370.
 template <class P, bool NH>
 __global__ void __launch_bounds__(kBlock, P::DF ? 8 : 6) k_momentum(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
@@ -922,7 +932,7 @@ __global__ void __launch_bounds__(kBlock, P::DF ? 8 : 6) k_momentum(DevMesh m, D
             s += w * ldg(F + y);
             pv += w * ldg(G + y);
         }
-        pv = 0.25 * fma(q2, s, pv);   // (2 q_e sum w F' + sum w F' 2 q_e')/4
+        pv = fma(q2, s, pv);   // 2 q_e sum w F' + sum w F' 2 q_e': four times the flux
     } else {
         const TA qee = ldg(G + x);
 #pragma unroll
@@ -997,7 +1007,9 @@ __global__ void __launch_bounds__(kBlock, P::DF ? 8 : 6) k_momentum(DevMesh m, D
         grad = pgf + (k2 - k1);
     }
     const double slow = fma(ldg(m.hrdc + e), grad, -va);
-    const TA tend = emu<P::EMU>(pv, d.emu, GRIST_ROW_PV_FLUX) + cv<TA>(slow);
+    const TA tend = P::EMU             ? emu<P::EMU>((TA)0.25 * pv, d.emu, GRIST_ROW_PV_FLUX) + cv<TA>(slow)
+                    : short_forms<P>() ? fma((TA)0.25, pv, cv<TA>(slow))
+                                       : pv + cv<TA>(slow);
     const TU v = emu<P::EMU>(cv<TU>(cv<TA>(un) + cv<TA>(dts) * tend), d.emu, GRIST_ROW_WIND);
     if (!isfinite(v)) atomicOr(status, GRIST_FLAG_NONFINITE);
     u_out[x] = v;
@@ -1034,9 +1046,12 @@ template <> struct AdvVal<float> {
     __device__ __forceinline__ explicit AdvVal(double x) { split_trunc(x, h, l); }
 };
 __device__ __forceinline__ double adv_diff(const AdvVal<double> &a, const AdvVal<double> &b) { return a.v - b.v; }
+// of phi, whose neighbours are close: the same bits off the FP64 pipe
+__device__ __forceinline__ double adv_diff_near(const AdvVal<double> &a, const AdvVal<double> &b) { return sub_near(a.v, b.v); }
 __device__ __forceinline__ float adv_diff(const AdvVal<float> &a, const AdvVal<float> &b) {
     return diff_df(a.h, a.l, b.h, b.l);
 }
+__device__ __forceinline__ float adv_diff_near(const AdvVal<float> &a, const AdvVal<float> &b) { return adv_diff(a, b); }
 
 // Explicit parts of Eqs. 6-7 at every interface: horizontal advection
 // V.grad(x) = (1/A) sum s dv u^int (x_nb - x)/2 and vertical advection
@@ -1048,7 +1063,7 @@ __device__ __forceinline__ float adv_diff(const AdvVal<float> &a, const AdvVal<f
 // the integer pipe (the splits), the FP64 form by the FP64 pipe; the cell's row
 // is read as vectors and the factors 1/2 of u and of the difference are taken
 // out of the sums.  Level 8, 60 levels, mixed 1107 -> 1042 us a launch (five
-// blocks of 256 an SM; 4: 1176, 6: 1218); FP64, level 7, 1184 -> 913.
+// blocks of 256 an SM; 4: 1176, 6: 1218); FP64, level 7, 1184 -> 888.
 template <class P, bool FIRST>
 __global__ void __launch_bounds__(kBlock, 5) k_nh_explicit(DevMesh m, DyPar d, LevelDiv Dv, const typename P::TU *__restrict__ u_s,
                               const double *__restrict__ rdps_s, const double *__restrict__ Mv,
@@ -1083,7 +1098,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_nh_explicit(DevMesh m, DyPar d, L
         const TA ub = cv<TA>(ldg(u_s + ue)), ut = j == 0 ? ub : cv<TA>(ldg(u_s + ue - 1));
         const TA cu = cw[s] * (ut + ub);
         hw += cu * adv_diff(AdvVal<TA>(ldg(w_s + y)), wi);
-        hp += cu * adv_diff(AdvVal<TA>(ldg(phi_s + y)), pi);
+        hp += cu * adv_diff_near(AdvVal<TA>(ldg(phi_s + y)), pi);
     }
     TA vw = 0, vp = 0;
     double fw = 0.0;
@@ -1091,7 +1106,7 @@ __global__ void __launch_bounds__(kBlock, 5) k_nh_explicit(DevMesh m, DyPar d, L
         const double rd2 = ldg(d.hrdBi + j) * ldg(rdps_s + i);   // 1/(dpi_{j-1} + dpi_j)
         const TA r = cv<TA>(Mv[(size_t)i * d.ldi + j] * rd2);
         vw = r * adv_diff(AdvVal<TA>(w_s[xi + 1]), AdvVal<TA>(w_s[xi - 1]));
-        vp = r * adv_diff(AdvVal<TA>(phi_s[xi + 1]), AdvVal<TA>(phi_s[xi - 1]));
+        vp = r * adv_diff_near(AdvVal<TA>(phi_s[xi + 1]), AdvVal<TA>(phi_s[xi - 1]));
         if (FIRST) {
             // first stage: the stage input is t^n, so rdps_s is 1/(ps^n - pi_top)
             fw = d.g * fma(p_n[(size_t)i * d.ld + j] - p_n[(size_t)i * d.ld + j - 1], 2.0 * rd2, -1.0);
