@@ -36,6 +36,9 @@
  *     runs on another (e.g. the tracers of step n beside the dycore of step
  *     n + 1, with their fluxes in separate buffers); two dycore steps, or
  *     two tracer steps, of one handle must not overlap.
+ *   - A dycore step runs parts of its stages on side streams of the handle,
+ *     forked from `stream` and joined to it by events before the call returns:
+ *     for the caller, stream captures included, its work is on `stream`.
  */
 #ifndef GRIST_H
 #define GRIST_H
@@ -238,9 +241,13 @@ int grist_tracer_step(grist_mesh mesh, const grist_tracer_batch *batch, double d
  *                       shared memory, never written to global memory);
  *                       ignored when persistent = 1.
  *   levels_per_thread   1 or 2: levels one thread of a per-phase launch
- *                       carries (levels g and g + ceil(L/2) for 2; the
- *                       entity's stencil tables are read once for both);
- *                       the persistent launch uses 1.
+ *                       carries, with one read of the entity's stencil tables:
+ *                       1 = a single level; 2 = a vector of consecutive levels
+ *                       (16 or 8 bytes of q: 4 or 2 binary32, 2 binary64)
+ *                       where the member's level count, row length and buffers
+ *                       are multiples of it (dpi and mass_flux on 16 bytes),
+ *                       else levels g and g + ceil(L/2); the persistent launch
+ *                       uses 1.
  *   cell_edges          1 = with beta_upwind = 1 the edge fluxes are formed
  *                       cell-centrically: the thread of a cell gathers q over
  *                       the cell and its neighbours once and writes the flux
