@@ -1338,8 +1338,8 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
 //   D   the block's threads over the flat (column, level) index, so the
 //       outputs are written as whole rows.
 // The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 40).
-// One warp for 32 columns needs about 24 blocks an SM to keep the pipe busy
-// (78 % then); with fewer columns than that the levels are the parallelism
+// One warp for 32 columns needs about 20 blocks an SM to keep the pipe busy
+// (75 % then); with fewer columns than that the levels are the parallelism
 // left (solve_by_blocks has the figures).
 // SHORT: rth_r holds dphi_r / th_r and the series' tails are binary32.
 constexpr int kSolveWarps = 8;
@@ -1464,7 +1464,7 @@ __global__ void __launch_bounds__(kSolveWarps * 32) k_nh_solve_block(
 // 10,242, 40,962, 163,842 and 655,362 columns): 30 levels 99 / 52, 155 / 151,
 // 552 / 485, 1845 / 1828; 60 levels 195 / 97, 298 / 275, 1022 / 1026, 3519 /
 // 3811; 100 levels 355 / 303, 496 / 728, 1717 / 2387.  So the block form while
-// the one-warp form has less than a wave (24 resident blocks of 32 columns on
+// the one-warp form has less than a wave (20 resident blocks of 32 columns on
 // 152 SMs) or columns are short, where three blocks' arrays fit an SM (70
 // levels; with fewer blocks an SM waits through every pass); above 70 levels
 // only for a few blocks per SM in all.

@@ -26,8 +26,9 @@
 // us per launch, one level / vectors: div 231 / 145, edge 365 / 231, update
 // 226 / 140 (then at the DRAM rate), ratios 545 / 335 (half of it the
 // division's slow path, see fct_ratio), final 440 / 307, low-order 270 / 128
-// more in the first edge phase; the step 3261 / 2110.  binary64 is bound by
-// the FP64 pipe and gains little from the width.
+// more in the first edge phase; the step 3261 / 2110 (1976 with the vertical
+// transport as it stands).  binary64 is bound by the FP64 pipe and gains little
+// from the width.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
