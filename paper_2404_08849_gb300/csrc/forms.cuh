@@ -1,0 +1,112 @@
+// Comparisons, signs and ratios of binary64 (and their binary32 counterparts)
+// in integer arithmetic, shared by the kernels.  The file needs nothing but the
+// bit-cast and rounding intrinsics, so that it also compiles on the host.
+#pragma once
+
+namespace grist {
+
+// Comparisons, maxima and minima of binary64 in integer arithmetic.  A DSETP
+// occupies the FP64 pipe, which bounds the FP64 policy, like an addition: 64
+// cycles of a scheduler for a warp; the integer form is 8 to 12 instructions of
+// the otherwise idle ALU.  The order key of a double's bits: negative
+// numbers with their magnitude bits inverted, so that keys compare like the
+// numbers (+-NaN beyond the infinities); the map is its own inverse.
+__device__ __forceinline__ long long okey(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double of_okey(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+constexpr long long kKeyInf = 0x7ff0000000000000ll;       // of +infinity
+constexpr long long kKeyNegInf = ~kKeyInf;                 // of -infinity
+
+// x >= 0, with -0 (NaN by its sign)
+__device__ __forceinline__ bool nonneg(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 || b == (long long)0x8000000000000000ull;
+}
+__device__ __forceinline__ bool nonneg(float x) { return x >= 0.f; }
+// x > 0 and x != 0 for the finite mesh weights
+__device__ __forceinline__ bool pos(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool pos(float x) { return x > 0.f; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
+__device__ __forceinline__ bool is_nan(double x) { return (__double_as_longlong(x) & 0x7fffffffffffffffll) > kKeyInf; }
+
+// Running maximum and minimum that ignore NaN as fmax and fmin do.
+template <typename TC> struct Bounds;
+template <> struct Bounds<float> {
+    float hi, lo;
+    __device__ __forceinline__ Bounds() {}
+    __device__ __forceinline__ Bounds(float a, float b) : hi(a), lo(b) {}
+    __device__ __forceinline__ void take(float a, float b) {
+        hi = fmaxf(hi, a);
+        lo = fminf(lo, b);
+    }
+    __device__ __forceinline__ float max() const { return hi; }
+    __device__ __forceinline__ float min() const { return lo; }
+};
+template <> struct Bounds<double> {
+    long long hi, lo;   // keys; NaN starts as the key that every number beats
+    __device__ __forceinline__ Bounds() {}
+    __device__ __forceinline__ Bounds(double a, double b) : hi(okey(a)), lo(okey(b)) {
+        if (hi > kKeyInf) hi = (long long)0x8000000000000000ull;
+        if (lo < kKeyNegInf) lo = 0x7fffffffffffffffll;
+    }
+    __device__ __forceinline__ void take(double a, double b) {
+        const long long ka = okey(a), kb = okey(b);
+        if (ka > hi && ka <= kKeyInf) hi = ka;
+        if (kb < lo && kb >= kKeyNegInf) lo = kb;
+    }
+    __device__ __forceinline__ double max() const { return of_okey(hi); }
+    __device__ __forceinline__ double min() const { return of_okey(lo); }
+};
+// min(a, b) of two numbers (no NaN)
+__device__ __forceinline__ float min_num(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ double min_num(double a, double b) { return okey(b) < okey(a) ? b : a; }
+
+// a <= b (false for NaN), |a|
+__device__ __forceinline__ bool le_num(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool le_num(double a, double b) {
+    const long long ka = okey(a), kb = okey(b);
+    return ka <= kb && kb <= kKeyInf && ka >= kKeyNegInf;
+}
+__device__ __forceinline__ float abs_num(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_num(double x) { return fabs(x); }
+// a == b for a value and a copy of it
+__device__ __forceinline__ bool same_num(float a, float b) { return a == b; }
+__device__ __forceinline__ bool same_num(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+
+// pm += max(0, x), pp += max(0, -x): the other sum would gain a zero, so one
+// addition serves both.  NaN adds nothing.
+__device__ __forceinline__ void add_signed(float x, float &pp, float &pm) {
+    pp += fmaxf(0.f, -x);
+    pm += fmaxf(0.f, x);
+}
+__device__ __forceinline__ void add_signed(double x, double &pp, double &pm) {
+    const bool neg = __double2hiint(x) < 0;
+    const double acc = neg ? pp : pm;
+    double sum = acc + fabs(x);
+    if (is_nan(x)) sum = acc;
+    pp = neg ? sum : pp;
+    pm = neg ? pm : sum;
+}
+
+// min(1, Q / P) for P >= TINY > 0, the bits of the division for every operand
+// (1 where that gives NaN).  The division is reached only where a cell is
+// limited: Q >= P is 1, and 0 is 0 without the division's slow path, which
+// operands near TINY take (where a tracer is constant, Q = 0 and P = TINY).
+__device__ __forceinline__ float fct_ratio(float Q, float P) {
+    if (!(Q < P)) return 1.f;
+    return Q == 0.f ? Q : fminf(1.f, Q / P);
+}
+// binary64: decided on the keys.
+__device__ __forceinline__ double fct_ratio(double Q, double P) {
+    if (okey(Q) >= okey(P) || is_nan(Q) || is_nan(P)) return 1.0;
+    if (!nonzero(Q)) return Q;
+    const double a = Q / P;
+    return is_nan(a) ? 1.0 : a;
+}
+
+}  // namespace grist

@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "forms.cuh"
 
 #define PN(n) (sizeof(TC) == 4 ? n "/mix" : n "/fp64")
 
@@ -188,94 +189,6 @@ template <bool PERS, typename T> __device__ __forceinline__ T lds(const T *p) {
 template <typename TC> __device__ __forceinline__ TC tiny_of();
 template <> __device__ __forceinline__ double tiny_of<double>() { return 2.2250738585072014e-308; }
 template <> __device__ __forceinline__ float tiny_of<float>() { return 1.17549435e-38f; }
-
-// Comparisons, maxima and minima of binary64 in integer arithmetic.  A DSETP
-// occupies the FP64 pipe, which bounds the FP64 policy, like an addition: 64
-// cycles of a scheduler for a warp; the integer form is 8 to 12 instructions of
-// the otherwise idle ALU.  The order key of a double's bits: negative
-// numbers with their magnitude bits inverted, so that keys compare like the
-// numbers (+-NaN beyond the infinities); the map is its own inverse.
-__device__ __forceinline__ long long okey(double x) {
-    const long long b = __double_as_longlong(x);
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
-__device__ __forceinline__ double of_okey(long long k) {
-    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
-}
-constexpr long long kKeyInf = 0x7ff0000000000000ll;       // of +infinity
-constexpr long long kKeyNegInf = ~kKeyInf;                 // of -infinity
-
-// x >= 0, with -0 (NaN by its sign)
-__device__ __forceinline__ bool nonneg(double x) {
-    const long long b = __double_as_longlong(x);
-    return b >= 0 || b == (long long)0x8000000000000000ull;
-}
-__device__ __forceinline__ bool nonneg(float x) { return x >= 0.f; }
-// x > 0 and x != 0 for the finite mesh weights
-__device__ __forceinline__ bool pos(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool pos(float x) { return x > 0.f; }
-__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
-__device__ __forceinline__ bool is_nan(double x) { return (__double_as_longlong(x) & 0x7fffffffffffffffll) > kKeyInf; }
-
-// Running maximum and minimum that ignore NaN as fmax and fmin do.
-template <typename TC> struct Bounds;
-template <> struct Bounds<float> {
-    float hi, lo;
-    __device__ __forceinline__ Bounds() {}
-    __device__ __forceinline__ Bounds(float a, float b) : hi(a), lo(b) {}
-    __device__ __forceinline__ void take(float a, float b) {
-        hi = fmaxf(hi, a);
-        lo = fminf(lo, b);
-    }
-    __device__ __forceinline__ float max() const { return hi; }
-    __device__ __forceinline__ float min() const { return lo; }
-};
-template <> struct Bounds<double> {
-    long long hi, lo;   // keys; NaN starts as the key that every number beats
-    __device__ __forceinline__ Bounds() {}
-    __device__ __forceinline__ Bounds(double a, double b) : hi(okey(a)), lo(okey(b)) {
-        if (hi > kKeyInf) hi = (long long)0x8000000000000000ull;
-        if (lo < kKeyNegInf) lo = 0x7fffffffffffffffll;
-    }
-    __device__ __forceinline__ void take(double a, double b) {
-        const long long ka = okey(a), kb = okey(b);
-        if (ka > hi && ka <= kKeyInf) hi = ka;
-        if (kb < lo && kb >= kKeyNegInf) lo = kb;
-    }
-    __device__ __forceinline__ double max() const { return of_okey(hi); }
-    __device__ __forceinline__ double min() const { return of_okey(lo); }
-};
-// min(a, b) of two numbers (no NaN)
-__device__ __forceinline__ float min_num(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double min_num(double a, double b) { return okey(b) < okey(a) ? b : a; }
-
-// a <= b (false for NaN), |a|
-__device__ __forceinline__ bool le_num(float a, float b) { return a <= b; }
-__device__ __forceinline__ bool le_num(double a, double b) {
-    const long long ka = okey(a), kb = okey(b);
-    return ka <= kb && kb <= kKeyInf && ka >= kKeyNegInf;
-}
-__device__ __forceinline__ float abs_num(float x) { return fabsf(x); }
-__device__ __forceinline__ double abs_num(double x) { return fabs(x); }
-// a == b for a value and a copy of it
-__device__ __forceinline__ bool same_num(float a, float b) { return a == b; }
-__device__ __forceinline__ bool same_num(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
-
-// pm += max(0, x), pp += max(0, -x): the other sum would gain a zero, so one
-// addition serves both.  NaN adds nothing.
-__device__ __forceinline__ void add_signed(float x, float &pp, float &pm) {
-    pp += fmaxf(0.f, -x);
-    pm += fmaxf(0.f, x);
-}
-__device__ __forceinline__ void add_signed(double x, double &pp, double &pm) {
-    const bool neg = __double2hiint(x) < 0;
-    const double acc = neg ? pp : pm;
-    double sum = acc + fabs(x);
-    if (is_nan(x)) sum = acc;
-    pp = neg ? sum : pp;
-    pm = neg ? pm : sum;
-}
 
 // ---------------------------------------------------------------------------
 // phase bodies (one work item each)
@@ -832,33 +745,6 @@ __device__ __forceinline__ void item_lowres(const CellRow<TC> &r, const MemberDe
         }
         store_lowres<TC, V>(mb, (size_t)t * mb.qs + x, r1, r2, qi, divl);
     }
-}
-
-// min(1, Q / P) for P >= TINY > 0.  binary32: the approximate reciprocal and
-// one correction of the quotient by its remainder, about half an ulp, instead
-// of the division, which takes its slow path (a call) where P is near TINY,
-// that is wherever a tracer is constant.  A quotient that overflows ends as
-// NaN, and fminf then returns 1.
-__device__ __forceinline__ float fct_ratio(float Q, float P) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(P));
-    const float a = Q * r;
-    return fminf(1.f, fmaf(fmaf(-a, P, Q), r, a));
-}
-// binary64: 1 where Q >= P, decided on the keys, so that a warp none of whose
-// cells is limited issues no division; else Q/P from the FMA reciprocal and
-// the same correction (P above 2^1020: the division).  NaN gives 1.
-__device__ __forceinline__ double fct_ratio(double Q, double P) {
-    if (okey(Q) >= okey(P)) return 1.0;
-    double a;
-    if (__double2hiint(P) < 0x7fb00000) {
-        const double r = rcp_nr(P);
-        a = Q * r;
-        a = fma(fma(-a, P, Q), r, a);
-    } else {
-        a = Q / P;
-    }
-    return is_nan(a) ? 1.0 : a;
 }
 
 // FCT 2: bounds over the cell and its neighbours of {q^n, q^td} (from the
