@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "series.cuh"
 
 #define PN(n) (P::DF ? n "/mixdf" : (sizeof(TA) == 4 ? (sizeof(TM) == 8 ? n "/mixdbl" : n "/mix") : n "/fp64"))
 
@@ -55,8 +56,8 @@ struct DyPar {
 };
 
 // Whether the pressure, geopotential and column kernels take forms that round
-// differently from the first ones (short series, tabled reference states):
-// the FP64 policy only.  In the mixed policies these fields feed binary32
+// differently from the first ones (tabled reference columns, dphi/th as one
+// field, the PV flux in two sums): the FP64 policy only.  In the mixed policies these fields feed binary32
 // values (u, the mass flux, the advection of w and phi) by differences, and
 // an ulp of phi moves some of those by a whole binary32 rounding; there the
 // kernels keep every bit.  (The emulating FP64 variant equals the FP64 policy
@@ -157,81 +158,6 @@ __device__ __forceinline__ auto entity_sums(Leaf &leaf, int j, int lane) {
         const bool up = (lane & O) != 0;
         return lane_add(lane_pick(up, b, a), lane_xor(lane_pick(up, a, b), O));
     }
-}
-
-// r^g for a ratio r close to 1 by the binomial series
-// (1 + x)^g = sum_n C(g, n) x^n, Horner in FP64, with the binomial
-// coefficients C(g, n) = C(g, n-1) (g - n + 1)/n formed on the host.  For
-// |g| < 2 the coefficients stay below 4 in magnitude up to n = 16, so after N
-// terms the omitted tail is below 4 |x|^N / (1 - |x|): the warp takes the
-// shortest series with 4 |x|^N <= 2^-58 for the largest |x| among its lanes
-// (N = 4, 5, 6, 8, 10 for |x| < 2^-15, 2^-12, 2^-10, 2^-8, 2^-6) - a
-// warp-uniform branch, so no FP64 issue slot is spent on terms no lane
-// needs.  A lane with |x| > 2^-6 uses the library pow().  mask: the lanes
-// executing the call.
-struct Binom {
-    double c[10];
-    float f[10];   // the same coefficients in binary32
-};
-
-template <int N> __device__ __forceinline__ double horner(double x, const Binom &B) {
-    double s = B.c[N - 1];
-#pragma unroll
-    for (int n = N - 2; n >= 0; n--) s = fma(s, x, B.c[n]);
-    return s;
-}
-
-// (1 + x)^g for a small x given directly.
-__device__ __forceinline__ double pow1p_near0(double x, double g, const Binom &B, unsigned mask) {
-    // high word of |x|: exponent and leading fraction bits, monotone in |x|
-    const unsigned hx = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    const unsigned hm = __reduce_max_sync(mask, hx);
-    if (hm < 0x3f000000u) return horner<4>(x, B);    // |x| < 2^-15
-    if (hm < 0x3f300000u) return horner<5>(x, B);    // 2^-12
-    if (hm < 0x3f500000u) return horner<6>(x, B);    // 2^-10
-    if (hm < 0x3f700000u) return horner<8>(x, B);    // 2^-8
-    if (hx > 0x3f900000u || (hx == 0x3f900000u && __double2loint(x) != 0)) return pow(1.0 + x, g);
-    return horner<10>(x, B);
-}
-
-// The same with the last terms, from the M-th on, where |x|^M <= 2^-30, summed
-// by Horner's rule in binary32: their rounding, 2^-24 of them, is below 2^-53
-// of the result, and 2, 3, 4 or 6 FP64 instructions do for |x| < 2^-15,
-// 2^-11, 2^-8, 2^-6 where all terms in FP64 take 3, 5, 7 or 9.  For the FP64
-// policy and the hydrostatic core; in the mixed policies the NH column state
-// keeps the bits of the form above (an ulp of phi moves the binary32
-// advection of the next stage by whole roundings).
-__device__ __forceinline__ double f2d_normal(float f) {   // a normal number or zero
-    const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
-    const uint32_t hi = a < 0x00800000u ? 0u : (a >> 3) + 0x38000000u;
-    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(a << 29));
-}
-template <int M, int N> __device__ __forceinline__ double horner_tail(double x, const Binom &B) {
-    const float xf = d2f_trunc(x);
-    float t = B.f[N - 1];
-#pragma unroll
-    for (int n = N - 2; n >= M; n--) t = fmaf(t, xf, B.f[n]);
-    double s = f2d_normal(t);
-#pragma unroll
-    for (int n = M - 1; n >= 0; n--) s = fma(s, x, B.c[n]);
-    return s;
-}
-__device__ __forceinline__ double pow1p_tail(double x, double g, const Binom &B, unsigned mask) {
-    const unsigned hx = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    const unsigned hm = __reduce_max_sync(mask, hx);
-    if (hm < 0x3f000000u) return horner_tail<2, 4>(x, B);    // |x| < 2^-15
-    if (hm < 0x3f400000u) return horner_tail<3, 6>(x, B);    // 2^-11
-    if (hm < 0x3f700000u) return horner_tail<4, 8>(x, B);    // 2^-8
-    if (hx > 0x3f900000u || (hx == 0x3f900000u && __double2loint(x) != 0)) return pow(1.0 + x, g);
-    return horner_tail<6, 10>(x, B);
-}
-
-Binom binomial(double g) {
-    Binom b;
-    b.c[0] = 1.0;
-    for (int n = 1; n < 10; n++) b.c[n] = b.c[n - 1] * (g - (n - 1)) / n;
-    for (int n = 0; n < 10; n++) b.f[n] = (float)b.c[n];
-    return b;
 }
 
 // GRIST_MIX_DF form of p (1 + x)^g for |x| <= 2^-6: the increment
@@ -618,7 +544,7 @@ __global__ void __launch_bounds__(kBlock) k_theta_update(DevMesh m, DyPar d, Lev
 // dps_c of the bin that dps falls in,
 //   Rd (p/p0)^kappa / p = [Rd (p_c/p0)^kappa / p_c] (1 + x)^(kappa - 1),
 //   x = Bm_k (dps - dps_c) / p_c,   |x| <= 2^-8 since Bm_k dps_c <= p_c,
-// summed by the 8-term series of pow1p_near0 (tail below 2^-58).  A bin is one
+// summed by the 8-term series of pow1p_near0 (tail below 2^-60).  A bin is one
 // value of the exponent and the first 7 fraction bits of dps; the table
 // covers the two octaves that end at twice the one of p0 - pi_top (32.8 to
 // 131 kPa for p0 = 1e5), other columns call pow().  Entry [bin][k] = {the
@@ -645,26 +571,26 @@ __global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
 // Eq. 8 (hydrostatic diagnostics), one warp per column: mid-layer pressure,
 // alpha = Rd theta (p/p0)^kappa / p, geopotential integrated upward from
 // phi_s by a suffix scan, layer geopotential = mean of its interfaces.
-// Bound by the FP64 pipe: about 24 instructions a cell-level with the table
+// Bound by the FP64 pipe: about 27 instructions a cell-level with the table
 // above (SHORT, see short_forms) against about 130 with pow(); level-6 mesh,
-// 30 levels: 323 -> 76 us a launch, plus 10 us a step for the table.
-// With pow() a warp takes two columns, so that the correctly rounded
-// 1/dps runs one column per lane, p/p0 is the product with 1/p0 corrected by its
-// remainder (the correctly rounded quotient: rp0 is correctly rounded and p0's
-// significand not all ones, which the host checks) and the pressure below is the
-// next lane's above: the same bits.  Level 6, 30 levels, us a mixed step by
-// columns: 1 1556, 2 1526, 4 1564, 8 1660 (1590 before).
-template <bool SHORT> constexpr int diag_cols() { return SHORT ? 1 : 2; }
+// 30 levels: 323 -> 77 us a launch, plus 10 us a step for the table.
+// A warp takes two columns, so that the correctly rounded 1/dps runs one column
+// per lane.  Level 6, 30 levels, us a step by columns, 1, 2, 4: FP64 1833, 1807,
+// 1805; mixed 1551, 1518, 1557.  With pow(), p/p0 is the product with 1/p0
+// corrected by its remainder (the correctly rounded quotient: rp0 is correctly
+// rounded and p0's significand not all ones, which the host checks) and the
+// pressure below is the next lane's above: the bits of the division.
+constexpr int kDiagCols = 2;
 template <bool EMU, bool DF, bool SHORT>
 __global__ void __launch_bounds__(kBlock) k_hydro_diag(DevMesh m, DyPar d, Exner ex, Binom bk, const double *__restrict__ ps,
                              const double *__restrict__ th, double *__restrict__ p, double *__restrict__ al,
                              double *__restrict__ phl) {
-    constexpr int C = diag_cols<SHORT>();
+    constexpr int C = kDiagCols;
     const int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * C;
     const int lane = threadIdx.x & 31;
     if (i0 >= m.nC) return;
     double dps_l = 0.0, rdps_l = 0.0;
-    if (!SHORT && i0 + lane < m.nC && lane < C) {
+    if (i0 + lane < m.nC && lane < C) {
         dps_l = ps[i0 + lane] - d.pi_top;
         rdps_l = rcp(dps_l);
     }
@@ -672,8 +598,7 @@ __global__ void __launch_bounds__(kBlock) k_hydro_diag(DevMesh m, DyPar d, Exner
 #pragma unroll 1
     for (int c = 0; c < ncol; c++) {
         const int i = i0 + c;
-        const double dps = SHORT ? ps[i] - d.pi_top : __shfl_sync(0xffffffffu, dps_l, c);
-        const double rdps = SHORT ? rcp_nr(dps) : __shfl_sync(0xffffffffu, rdps_l, c);
+        const double dps = __shfl_sync(0xffffffffu, dps_l, c), rdps = __shfl_sync(0xffffffffu, rdps_l, c);
         const int bin = SHORT ? (__double2hiint(dps) >> 13) - ex.base : -1;
         const bool tabled = bin >= 0 && bin < kExnerBins;   // the same for the whole warp
         const double off = SHORT ? dps - exner_centre(ex.base, bin) : 0.0;
@@ -686,7 +611,7 @@ __global__ void __launch_bounds__(kBlock) k_hydro_diag(DevMesh m, DyPar d, Exner
                 if (k < d.L) {
                     const double2 r = ldg(row + k);
                     pk = fma(ldg(d.Bm + k), dps, d.pi_top);
-                    contrib = th[(size_t)i * d.ld + k] * (r.x * horner_tail<4, 8>(r.y * off, bk));   // alpha dpi
+                    contrib = th[(size_t)i * d.ld + k] * (r.x * horner<8>(r.y * off, bk));   // alpha dpi
                     a = contrib * (ldg(d.rdB + k) * rdps);
                 }
             } else {
@@ -776,6 +701,12 @@ __global__ void k_vort(DevMesh m, DyPar d, LevelDiv Dh, const typename P::TU *__
                                                    d.emu, GRIST_ROW_PV_FLUX);
         }
     }
+}
+
+__device__ __forceinline__ double f2d_normal(float f) {   // a normal number or zero
+    const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+    const uint32_t hi = a < 0x00800000u ? 0u : (a >> 3) + 0x38000000u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(a << 29));
 }
 
 // Cell kinetic energy, stored doubled: 2K = sum (dc dv / 2A) u^2 (FP64:
@@ -1229,9 +1160,8 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
                 // x = th dphi_r / (th_r dphi**) - 1, the ratio's offset from 1
                 const double tr = sA[2 * kStage + o] * sA[3 * kStage + o];
                 const double x = SHORT ? fma(tr, rdfj, -1.0) : fma(tr, sA[1 * kStage + o] * rdfj, -1.0);
-                const double pstj = DF      ? scale_near1_df(sA[4 * kStage + o], x, d.gamma, bg_pos)
-                                    : SHORT ? sA[4 * kStage + o] * pow1p_tail(x, d.gamma, bg_pos, amask)
-                                            : sA[4 * kStage + o] * pow1p_near0(x, d.gamma, bg_pos, amask);
+                const double pstj = DF ? scale_near1_df(sA[4 * kStage + o], x, d.gamma, bg_pos)
+                                       : sA[4 * kStage + o] * pow1p_near0(x, d.gamma, bg_pos, amask);
                 pst[j] = pstj;
                 rdf[j] = rdfj;
                 const double C = gbg * pstj * rdfj;
@@ -1298,9 +1228,8 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
                 const double w_bot = (kk + 1 < nk) ? sA[1 * kStage + o + kRow] : sA[6 * kStage + lane];
                 const double phi_bot = (k + 1 < L) ? fma(bg, w_bot, sA[o]) : ldg(d.phis + i);
                 const double xk = bg * (w_top - w_bot) * rdf[k];
-                const double pk = DF      ? scale_near1_df(pst[k], xk, -d.gamma, bg_neg)
-                                  : SHORT ? pst[k] * pow1p_tail(xk, -d.gamma, bg_neg, amask)
-                                          : pst[k] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
+                const double pk = DF ? scale_near1_df(pst[k], xk, -d.gamma, bg_neg)
+                                     : pst[k] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
                 double hcur = 0.5;
                 if (k > 0) {
                     hcur = (pk - pprev) * (ldg(d.hrdBi + k) * rdps);
@@ -1337,11 +1266,11 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
 //   C   lanes = columns, a warp per level: the new pressure;
 //   D   the block's threads over the flat (column, level) index, so the
 //       outputs are written as whole rows.
-// The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 40).
+// The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 43).
 // One warp for 32 columns needs about 20 blocks an SM to keep the pipe busy
 // (75 % then); with fewer columns than that the levels are the parallelism
 // left (solve_by_blocks has the figures).
-// SHORT: rth_r holds dphi_r / th_r and the series' tails are binary32.
+// SHORT: rth_r holds dphi_r / th_r.
 constexpr int kSolveWarps = 8;
 
 template <bool EMU, bool DF, bool SHORT>
@@ -1374,9 +1303,8 @@ __global__ void __launch_bounds__(kSolveWarps * 32) k_nh_solve_block(
             const double pr = p_r[x0 + k], tr = ldg(th + x0 + k) * ldg(rth_r + x0 + k);
             // th dphi_r / (th_r dphi**) - 1
             const double x = SHORT ? fma(tr, rdf, -1.0) : fma(tr, ldg(dphi_r + x0 + k) * rdf, -1.0);
-            const double pst = DF      ? scale_near1_df(pr, x, d.gamma, bg_pos)
-                               : SHORT ? pr * pow1p_tail(x, d.gamma, bg_pos, amask)
-                                       : pr * pow1p_near0(x, d.gamma, bg_pos, amask);
+            const double pst = DF ? scale_near1_df(pr, x, d.gamma, bg_pos)
+                                  : pr * pow1p_near0(x, d.gamma, bg_pos, amask);
             const int o = k * kRow + lane;
             sP[o] = pst;
             sD[o] = rdf;
@@ -1419,9 +1347,8 @@ __global__ void __launch_bounds__(kSolveWarps * 32) k_nh_solve_block(
             const int o = k * kRow + lane;
             const double w_bot = k + 1 < L ? sW[o + kRow] : 0.0;
             const double xk = bg * (sW[o] - w_bot) * sD[o];
-            sP[o] = DF      ? scale_near1_df(sP[o], xk, -d.gamma, bg_neg)
-                    : SHORT ? sP[o] * pow1p_tail(xk, -d.gamma, bg_neg, amask)
-                            : sP[o] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
+            sP[o] = DF ? scale_near1_df(sP[o], xk, -d.gamma, bg_neg)
+                       : sP[o] * pow1p_near0(xk, -d.gamma, bg_neg, amask);
         }
     }
     __syncthreads();
@@ -1663,7 +1590,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     uint32_t *status = status_word(h);
     const LevelDiv DL = make_div((uint32_t)L), DI = make_div((uint32_t)(L + 1)), DH = make_div((uint32_t)(L + 1) / 2);
     const unsigned gC = grid_for((long long)m.nC * L, kBlock),
-                   gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for(((long long)m.nC + diag_cols<short_forms<P>()>() - 1) / diag_cols<short_forms<P>()>() * 32, kBlock),
+                   gV = grid_for((long long)m.nV * L, kBlock), gW = grid_for(((long long)m.nC + kDiagCols - 1) / kDiagCols * 32, kBlock),
                    gI = grid_for((long long)m.nC * (L + 1), kBlock),
                    gVx = grid_for(m.nV, kBlock), gEG = grid_for(((long long)m.nE + kMassGroup - 1) / kMassGroup * 32, kBlock),
                    gCG = grid_for(((long long)m.nC + kMassGroup - 1) / kMassGroup * 32, kBlock),

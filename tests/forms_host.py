@@ -31,12 +31,12 @@ static bool same(float a, float b) { return bits(a) == bits(b) || (std::isnan(a)
 """
 
 
-def run(tmp_path, header, main):
+def run(tmp_path, header, main, shim=""):
     """Numbers that `main` prints, as floats."""
     if shutil.which("g++") is None:
         pytest.skip("g++ not found")
     src = tmp_path / "test.cpp"
-    src.write_text(SHIM + '#include "%s"\nusing namespace grist;\n' % os.path.join(CSRC, header) + main)
+    src.write_text(SHIM + shim + '#include "%s"\nusing namespace grist;\n' % os.path.join(CSRC, header) + main)
     exe = tmp_path / "test"
     subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-o", str(exe), str(src)], check=True)
     return [float(x) for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()]
