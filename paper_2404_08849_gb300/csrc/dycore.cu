@@ -49,7 +49,8 @@ struct DyPar {
     const double *rdB;    // [L]   1/dB
     const double *hrdBi;  // [L+1] 1/(dB[j-1] + dB[j]) at interior interfaces j (half the reciprocal mean)
     const double *dBi;    // [L+1] (dB[j-1] + dB[j])/2 at interior interfaces j
-    const double *Bm;     // [L]   (B[k] + B[k+1])/2, mid-layer coordinate
+    const double *Bm;     // [L]   (B[k] + B[k+1])/2, mid-layer coordinate, rounded,
+    const double *Bml;    // [L]   and the rest of it
     const float *dBf;     // [L]   dB rounded to single precision
     const double *phis;   // [nC]  surface geopotential
     uint32_t emu;         // GRIST_ROW_* rows rounded to binary32 (precision search)
@@ -536,36 +537,20 @@ __global__ void __launch_bounds__(kBlock) k_theta_update(DevMesh m, DyPar d, Lev
     }
 }
 
-// Reference states of the hydrostatic equation of state.  pow() costs about
-// 100 FP64 instructions, which bounded k_hydro_diag (pipe 90 % active); but
-// Rd (p/p0)^kappa / p at level k depends on the column's mass
-// dps = ps - pi_top alone, p = pi_top + Bm_k dps, so a table of reference
-// columns turns it into a short series: with the reference at the middle
-// dps_c of the bin that dps falls in,
-//   Rd (p/p0)^kappa / p = [Rd (p_c/p0)^kappa / p_c] (1 + x)^(kappa - 1),
-//   x = Bm_k (dps - dps_c) / p_c,   |x| <= 2^-8 since Bm_k dps_c <= p_c,
-// summed by the 8-term series of pow1p_near0 (tail below 2^-60).  A bin is one
-// value of the exponent and the first 7 fraction bits of dps; the table
-// covers the two octaves that end at twice the one of p0 - pi_top (32.8 to
-// 131 kPa for p0 = 1e5), other columns call pow().  Entry [bin][k] = {the
-// bracket, Bm_k / p_c}: 256 x L x 16 bytes, of which a run touches the bins
-// its surface pressures span (a few tens of kB).
+// The table of the hydrostatic equation of state (exner_entry, series.cuh):
+// 256 bins x L entries of 16 bytes, of which a run touches the bins its surface
+// pressures span (a few tens of kB).
 constexpr int kExnerBins = 256;
 struct Exner {
     const double2 *tab;
     int base;   // (high word of dps) >> 13 of bin 0
 };
-__device__ __forceinline__ double exner_centre(int base, int bin) {
-    return __hiloint2double(((base + bin) << 13) | (1 << 12), 0);
-}
 
 __global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= kExnerBins * d.L) return;
     const int bin = n / d.L, k = n - bin * d.L;
-    const double bm = d.Bm[k];
-    const double pc = d.pi_top + bm * exner_centre(base, bin);
-    tab[n] = make_double2(d.rd * pow(pc / d.p0, d.kappa) / pc, bm / pc);
+    tab[n] = exner_entry(d.pi_top, d.Bm[k], d.Bml[k], exner_centre(base, bin), d.p0, d.rd, d.kappa);
 }
 
 // Eq. 8 (hydrostatic diagnostics), one warp per column: mid-layer pressure,
@@ -610,8 +595,8 @@ __global__ void __launch_bounds__(kBlock) k_hydro_diag(DevMesh m, DyPar d, Exner
             if (tabled) {
                 if (k < d.L) {
                     const double2 r = ldg(row + k);
-                    pk = fma(ldg(d.Bm + k), dps, d.pi_top);
-                    contrib = th[(size_t)i * d.ld + k] * (r.x * horner<8>(r.y * off, bk));   // alpha dpi
+                    pk = fma(ldg(d.Bm + k), dps, fma(ldg(d.Bml + k), dps, d.pi_top));
+                    contrib = th[(size_t)i * d.ld + k] * exner_at(r, off, bk);   // alpha dpi
                     a = contrib * (ldg(d.rdB + k) * rdps);
                 }
             } else {
@@ -1502,7 +1487,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += al(bytes); return o; };
-    const size_t nvg = 6 * (size_t)L + 3 + ((size_t)L + 1) / 2;   // doubles, then L floats
+    const size_t nvg = 7 * (size_t)L + 3 + ((size_t)L + 1) / 2;   // doubles, then L floats
     const size_t o_vg = take(sizeof(double) * nvg);
     const size_t o_uA = take(nEL * sizeof(TU)), o_uB = take(nEL * sizeof(TU));
     const size_t o_psA = take(m.nC * 8), o_psB = take(m.nC * 8), o_psN = take(m.nC * 8);
@@ -1527,7 +1512,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     if (!s) return GRIST_ENOMEM;
 
     // vertical grid: B (L+1) | dB (L) | 1/dB (L) | 1/(dB[j-1]+dB[j]) (L+1) | (dB[j-1]+dB[j])/2 (L+1) |
-    // (B[k]+B[k+1])/2 (L) | dB in binary32 (L floats)
+    // (B[k]+B[k+1])/2 (L) | its rest (L) | dB in binary32 (L floats)
     std::vector<double> vg(nvg, 0.0);
     double *hB = vg.data(), *hdB = hB + L + 1, *hrdB = hdB + L, *hhrdBi = hrdB + L, *hdBi = hhrdBi + L + 1;
     for (int k = 0; k <= L; k++) hB[k] = prm->b_interface[k];
@@ -1540,8 +1525,14 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
         hdBi[j] = 0.5 * (hdB[j - 1] + hdB[j]);
     }
     double *hBm = hdBi + L + 1;
-    for (int k = 0; k < L; k++) hBm[k] = 0.5 * (hB[k] + hB[k + 1]);
-    float *hdBf = reinterpret_cast<float *>(hBm + L);
+    double *hBml = hBm + L;
+    for (int k = 0; k < L; k++) {
+        // the sum's rounding error by the larger summand (B increases)
+        const double sum = hB[k] + hB[k + 1];
+        hBm[k] = 0.5 * sum;
+        hBml[k] = 0.5 * (hB[k] - (sum - hB[k + 1]));
+    }
+    float *hdBf = reinterpret_cast<float *>(hBml + L);
     for (int k = 0; k < L; k++) hdBf[k] = (float)hdB[k];
     double *dvg = (double *)(s + o_vg);
     if (vg_ptr(h) != dvg || vg_cache(h) != vg) {
@@ -1566,7 +1557,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     d.B = dvg; d.dB = dvg + L + 1; d.rdB = dvg + 2 * L + 1; d.hrdBi = dvg + 3 * L + 1; d.dBi = dvg + 4 * L + 2;
     d.phis = prm->phi_surface;
     d.Bm = dvg + 5 * L + 3;
-    d.dBf = reinterpret_cast<const float *>(dvg + 6 * L + 3);
+    d.Bml = dvg + 6 * L + 3;
+    d.dBf = reinterpret_cast<const float *>(dvg + 7 * L + 3);
     d.emu = prm->emulate_fp32_rows;
 
     TU *uA = (TU *)(s + o_uA), *uB = (TU *)(s + o_uB);

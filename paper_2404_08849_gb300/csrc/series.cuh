@@ -52,4 +52,47 @@ inline Binom binomial(double g) {
     return b;
 }
 
+// Reference columns of the hydrostatic equation of state.  pow() costs about
+// 100 FP64 instructions, which bounded the hydrostatic diagnostics (pipe 90 %
+// active); but Rd (p/p0)^kappa / p at level k depends on the column's mass
+// dps = ps - pi_top alone, p = pi_top + B_k dps with the mid-layer coordinate
+// B_k, so a table of reference columns turns it into a short series: with the
+// reference at the middle dps_c of the bin that dps falls in,
+//   Rd (p/p0)^kappa / p = [Rd (p_c/p0)^kappa / p_c] (1 + x)^(kappa - 1),
+//   x = B_k (dps - dps_c) / p_c,   |x| <= 2^-8 since B_k dps_c <= p_c,
+// summed by the 8-term series of pow1p_near0 (tail below 2^-60).  A bin is one
+// value of the exponent and the first 7 fraction bits of dps; the table
+// covers the two octaves that end at twice the one of p0 - pi_top (32.8 to
+// 131 kPa for p0 = 1e5), other columns call pow().
+__device__ __forceinline__ double exner_centre(int base, int bin) {
+    return __hiloint2double(((base + bin) << 13) | (1 << 12), 0);
+}
+
+// Entry {the bracket, B_k / p_c} for B_k = bm + bl.  The bracket carries the
+// error of pow() and half an ulp: the roundings of p_c, of p_c/p0 and of the
+// product are collected and added at the end.  With a plain bracket and the
+// series rounded before the product, the largest error of alpha was 6.7 to 7.4
+// units of 2^-53 and its rms 1.45, where pow() of the pressure itself gives 6.2
+// and 1.30; as it is, 5.6 and 1.23.
+__device__ __forceinline__ double2 exner_entry(double pi_top, double bm, double bl, double c, double p0, double rd,
+                                               double kappa) {
+    const double h = __dmul_rn(bm, c), s = __dadd_rn(pi_top, h), b = __dadd_rn(s, -pi_top);
+    const double e = __dadd_rn(__dadd_rn(pi_top, -__dadd_rn(s, -b)), __dadd_rn(h, -b)) + fma(bl, c, fma(bm, c, -h));
+    const double pc = __dadd_rn(s, e), dpc = __dadd_rn(e, -__dadd_rn(pc, -s));   // p_c = pc + dpc
+    const double q = pc / p0, dq = fma(-q, p0, pc) + dpc;                       // p_c/p0 = q (1 + dq/pc)
+    const double y = pow(q, kappa), t = __dmul_rn(rd, y), z = t / pc;
+    const double dt = fma(rd, y, -t) + t * ((kappa * dq - dpc) / pc);
+    return make_double2(z + (fma(-z, pc, t) + dt) / pc, bm / pc);
+}
+
+// The bracket times (1 + x)^(kappa - 1), x = r.y off: the series less its one is
+// added in the product, which rounds once.
+__device__ __forceinline__ double exner_at(double2 r, double off, const Binom &B) {
+    const double x = r.y * off;
+    double s = B.c[7];
+#pragma unroll
+    for (int n = 6; n >= 1; n--) s = fma(s, x, B.c[n]);
+    return fma(r.x, x * s, r.x);
+}
+
 }  // namespace grist
