@@ -375,6 +375,18 @@ int grist_dycore_step_hydro(grist_mesh mesh, grist_dycore_state *state, const gr
 int grist_dycore_step_nh(grist_mesh mesh, grist_dycore_state *state, const grist_dycore_params *params,
                          grist_precision prec, double dt, void *stream);
 
+/* Which of equivalent forms the dycore steps of a mesh take (no counterpart
+ * in the paper); every choice gives the same bits.
+ *   column_solve        the NH core's column solve: 0 = by the numbers of
+ *                       columns and levels; 1 = one warp per 32 columns, one
+ *                       thread per column; 2 = a block of 8 warps per 32 columns.
+ * Default 0.  GRIST_EINVAL for other values. */
+typedef struct {
+    int32_t column_solve;
+} grist_dycore_tuning;
+int grist_dycore_set_tuning(grist_mesh mesh, const grist_dycore_tuning *tuning);
+int grist_dycore_get_tuning(grist_mesh mesh, grist_dycore_tuning *tuning);
+
 /* Diagnostic: relative vorticity at the vertices, zeta_v = (1/A_v) sum over
  * the vertex's edges of t(e,v) dc_e u_e, on every level (the velocity
  * diagnostic of Eq. 1).

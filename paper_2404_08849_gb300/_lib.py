@@ -56,6 +56,10 @@ class DycoreParams(ctypes.Structure):
                 ("emulate_fp32_rows", ctypes.c_uint32)]
 
 
+class DycoreTuning(ctypes.Structure):
+    _fields_ = [("column_solve", _I)]
+
+
 class DycoreState(ctypes.Structure):
     _fields_ = [("u", _V), ("ps", _V), ("dpi_theta", _V), ("w", _V), ("phi", _V), ("mass_flux_accum", _V),
                 ("accum_weight", _V), ("dpi_start", _V), ("p_nh", _V), ("p_nh_valid", _I), ("accum_scale", _D),
@@ -71,6 +75,8 @@ EXPORTS = {
     "grist_tracer_step": ([_V, _P(TracerBatch), _D, _V], ctypes.c_int),
     "grist_dycore_step_hydro": ([_V, _P(DycoreState), _P(DycoreParams), ctypes.c_int, _D, _V], ctypes.c_int),
     "grist_dycore_step_nh": ([_V, _P(DycoreState), _P(DycoreParams), ctypes.c_int, _D, _V], ctypes.c_int),
+    "grist_dycore_set_tuning": ([_V, _P(DycoreTuning)], ctypes.c_int),
+    "grist_dycore_get_tuning": ([_V, _P(DycoreTuning)], ctypes.c_int),
     "grist_global_sums": ([_V, ctypes.c_int, _V, _V, _I, _I, ctypes.c_int, _D, _P(_D), _V], ctypes.c_int),
     "grist_last_step_status": ([_V, _P(ctypes.c_uint32)], ctypes.c_int),
     "grist_status_string": ([ctypes.c_int], ctypes.c_char_p),

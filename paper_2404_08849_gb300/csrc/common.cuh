@@ -482,6 +482,7 @@ const HostTables &host_tables(grist_mesh_s *m);
 // waits for the copy) only when either changed.
 std::vector<double> &vg_cache(grist_mesh_s *m);
 const void *&vg_ptr(grist_mesh_s *m);
+grist_dycore_tuning &dycore_tuning(grist_mesh_s *m);
 
 // The dycore's side streams, each with its fork and join event, made on first
 // use; false if they could not be.  They belong to the handle: two dycore

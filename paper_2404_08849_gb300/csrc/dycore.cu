@@ -1372,14 +1372,19 @@ __global__ void __launch_bounds__(kSolveWarps * 32) k_nh_solve_block(
     }
 }
 
-// Which form, by columns and levels.  Measured (us a launch, one warp / block,
-// 10,242, 40,962, 163,842 and 655,362 columns): 30 levels 99 / 52, 155 / 151,
-// 552 / 485, 1845 / 1828; 60 levels 195 / 97, 298 / 275, 1022 / 1026, 3519 /
-// 3811; 100 levels 355 / 303, 496 / 728, 1717 / 2387.  So the block form while
-// the one-warp form has less than a wave (20 resident blocks of 32 columns on
-// 152 SMs) or columns are short, where three blocks' arrays fit an SM (70
-// levels; with fewer blocks an SM waits through every pass); above 70 levels
-// only for a few blocks per SM in all.
+// Which form, by columns and levels; both give the same bits
+// (tests/test_gpu_solve_bits.py).  Mixed, us a launch, one warp / block:
+//   levels            20         30         41         50         60         71
+//   10,242 cells   57 /  35   91 /  49  128 /  65  156 /  95  184 /  91  216 / 138
+//   40,962         93 / 100  142 / 138  201 / 185  237 / 279  274 / 260  342 / 373
+//   163,842       326 / 317  518 / 458  754 / 620  878 / 864  938 / 975 1297 /1260
+//   655,362                 1845 /1828                       3519 /3811
+// 80 levels: 244 / 179, 364 / 455, 1246 / 1541; FP64 within 4 % of these.  So the
+// block form while the one-warp form has less than a wave (20 resident blocks of
+// 32 columns on 152 SMs) or columns are short, where three blocks' arrays fit an
+// SM (70 levels; with fewer blocks an SM waits through every pass); above 70
+// levels only for a few blocks per SM in all.  The line at 40 levels is on the safe
+// side: at 163,842 cells the block form is the faster one up to 50.
 inline bool solve_by_blocks(int nC, int L) {
     if (L > 70) return nC <= 152 * kSolveCols * 3;
     return nC < 152 * kSolveCols * kSolveMinBlocks || L <= 40;
@@ -1389,9 +1394,9 @@ template <bool EMU, bool DF, bool SHORT>
 cudaError_t launch_solve(const DevMesh &m, const DyPar &d, LevelDiv Dv, const double *wst, const double *phst,
                          const double *th, const double *rth, const double *dphi, const double *p_r, const double *ps,
                          double dts, double *w_out, double *phi_out, double *p, double *al, double *phl, double *dpp,
-                         const Binom &bp, const Binom &bn, cudaStream_t st) {
+                         const Binom &bp, const Binom &bn, int form, cudaStream_t st) {
     const unsigned grid = grid_for(m.nC, kSolveCols);
-    if (solve_by_blocks(m.nC, d.L)) {
+    if (form == 2 || (form == 0 && solve_by_blocks(m.nC, d.L))) {
         const int bytes = 4 * d.L * kRow * 8;
         const cudaError_t e = cudaFuncSetAttribute(k_nh_solve_block<EMU, DF, SHORT>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1708,7 +1713,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             cudaError_t se = cudaSuccess;
             GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, short_forms<P>()>(
                 m, d, DL, wst, phst, th_outs[s3], rthn, dphn, p_n, ps_outs[s3], h3, w_outs[s3], phi_outs[s3], p_outs[s3],
-                alp, phl, dpp, bpos, bneg, st)));
+                alp, phl, dpp, bpos, bneg, dycore_tuning(h).column_solve, st)));
             if (se != cudaSuccess) return GRIST_ECUDA;
         } else {
             GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF, short_forms<P>()><<<gW, kBlock, 0, st>>>(
@@ -1791,6 +1796,18 @@ extern "C" int grist_dycore_step_nh(grist_mesh h, grist_dycore_state *S, const g
         case GRIST_MIX_DF: return dycore_step<PolMIXDF, true>(h, S, prm, dt, st);
         default: return dycore_step<PolMIXDBL, true>(h, S, prm, dt, st);
     }
+}
+
+extern "C" int grist_dycore_set_tuning(grist_mesh h, const grist_dycore_tuning *t) {
+    if (!h || !t || t->column_solve < 0 || t->column_solve > 2) return GRIST_EINVAL;
+    dycore_tuning(h) = *t;
+    return GRIST_OK;
+}
+
+extern "C" int grist_dycore_get_tuning(grist_mesh h, grist_dycore_tuning *t) {
+    if (!h || !t) return GRIST_EINVAL;
+    *t = dycore_tuning(h);
+    return GRIST_OK;
 }
 
 extern "C" int grist_diag_vorticity(grist_mesh h, const void *u, grist_precision prec, int32_t n_levels, int32_t ld,

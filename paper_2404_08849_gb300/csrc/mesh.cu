@@ -28,6 +28,7 @@ struct grist_mesh_s {
     // the dycore's vertical-grid table as last uploaded, and where
     std::vector<double> vg_cache;
     const void *vg_ptr = nullptr;
+    grist_dycore_tuning dytune{};   // forms of the dycore, all by size
     // the dycore's side streams (0 not made, 1 made, -1 could not be)
     int side_state = 0;
     cudaStream_t side[kSides] = {nullptr};
@@ -50,6 +51,7 @@ TracerCtx *&tracer_ctx(grist_mesh_s *m) { return m->tctx; }
 const HostTables &host_tables(grist_mesh_s *m) { return m->ht; }
 std::vector<double> &vg_cache(grist_mesh_s *m) { return m->vg_cache; }
 const void *&vg_ptr(grist_mesh_s *m) { return m->vg_ptr; }
+grist_dycore_tuning &dycore_tuning(grist_mesh_s *m) { return m->dytune; }
 
 bool side_stream(grist_mesh_s *m, int which, cudaStream_t *s, cudaEvent_t **ev) {
     if (m->side_state == 0) {
