@@ -380,9 +380,14 @@ int grist_dycore_step_nh(grist_mesh mesh, grist_dycore_state *state, const grist
  *   column_solve        the NH core's column solve: 0 = by the numbers of
  *                       columns and levels; 1 = one warp per 32 columns, one
  *                       thread per column; 2 = a block of 8 warps per 32 columns.
- * Default 0.  GRIST_EINVAL for other values. */
+ *   wind_placement      where the NH core runs the stage's wind diagnostics,
+ *                       which need neither the mass nor the column kernels: 0 = by
+ *                       the number of columns; 1 = on a side stream from the start
+ *                       of the stage; 2 = on a side stream beside the column solve.
+ *                       (The hydrostatic core: from the start.)
+ * Default 0, 0.  GRIST_EINVAL for other values. */
 typedef struct {
-    int32_t column_solve;
+    int32_t column_solve, wind_placement;
 } grist_dycore_tuning;
 int grist_dycore_set_tuning(grist_mesh mesh, const grist_dycore_tuning *tuning);
 int grist_dycore_get_tuning(grist_mesh mesh, grist_dycore_tuning *tuning);

@@ -321,16 +321,16 @@ class Mesh:
     def dycore_step_nh(self, state, params, dt, prec="fp64", stream=None):
         self._dycore("grist_dycore_step_nh", state, params, prec, dt, stream)
 
-    def set_dycore_tuning(self, column_solve=0):
+    def set_dycore_tuning(self, column_solve=0, wind_placement=0):
         """Which of the dycore's equivalent forms to take
         (grist_dycore_set_tuning); 0 = by size."""
-        t = _lib.DycoreTuning(int(column_solve))
+        t = _lib.DycoreTuning(int(column_solve), int(wind_placement))
         _lib.check("grist_dycore_set_tuning", _lib.load().grist_dycore_set_tuning(self.handle, ctypes.byref(t)))
 
     def dycore_tuning(self):
         t = _lib.DycoreTuning()
         _lib.check("grist_dycore_get_tuning", _lib.load().grist_dycore_get_tuning(self.handle, ctypes.byref(t)))
-        return {"column_solve": t.column_solve}
+        return {"column_solve": t.column_solve, "wind_placement": t.wind_placement}
 
     def vorticity(self, u, n_levels, out=None, stream=None):
         """Relative vorticity at the vertices, [nV][ld] float64 on the device

@@ -57,7 +57,7 @@ class DycoreParams(ctypes.Structure):
 
 
 class DycoreTuning(ctypes.Structure):
-    _fields_ = [("column_solve", _I)]
+    _fields_ = [("column_solve", _I), ("wind_placement", _I)]
 
 
 class DycoreState(ctypes.Structure):

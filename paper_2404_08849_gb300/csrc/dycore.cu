@@ -1667,7 +1667,8 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     // level 6 NH, 41 levels 1606 / 1446; level 7 FP64 NH 17277 / 16953; level 8
     // mixed NH 28962 / 28667.
     Side sw_(h, 0, st), sx_(h, 1, st);   // the wind's diagnostics, the advection
-    const bool late = NH && wind_beside_solve(m.nC);
+    const int place = dycore_tuning(h).wind_placement;
+    const bool late = NH && (place == 2 || (place == 0 && wind_beside_solve(m.nC)));
     for (int s3 = 0; s3 < 3; s3++) {
         const double h3 = dts[s3];
         auto wind = [&](cudaStream_t sw) {
@@ -1800,6 +1801,7 @@ extern "C" int grist_dycore_step_nh(grist_mesh h, grist_dycore_state *S, const g
 
 extern "C" int grist_dycore_set_tuning(grist_mesh h, const grist_dycore_tuning *t) {
     if (!h || !t || t->column_solve < 0 || t->column_solve > 2) return GRIST_EINVAL;
+    if (t->wind_placement < 0 || t->wind_placement > 2) return GRIST_EINVAL;
     dycore_tuning(h) = *t;
     return GRIST_OK;
 }
