@@ -1503,7 +1503,13 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     const size_t o_theta = take(nCL * sizeof(TA)), o_Fth = take(nEL * sizeof(TA));
     const size_t o_p = take(nCL * 8), o_al = take(nCL * 8), o_phl = take(nCL * 8), o_dpp = take(nCL * 8);
     const size_t o_qv = take(nVL * sizeof(TA)), o_K = take(nCL * 8);
-    const size_t o_Gq = take(nEL * sizeof(TA));
+    // The edge PV takes the theta flux's array where it is formed after the theta
+    // update: in the FP64 policy, which needs the mass flux for it anyway, and on
+    // large meshes, where the array counts (level 9, 60 levels: 1.9 GB in
+    // binary32).  By size alone, so that no choice of forms moves the scratch of a
+    // recorded step.
+    const bool pv_shares = short_forms<P>() || wind_beside_solve(m.nC);
+    const size_t o_Gq = pv_shares ? o_Fth : take(nEL * sizeof(TA));
     size_t o_wA = 0, o_wB = 0, o_phA = 0, o_phB = 0, o_wst = 0, o_phst = 0, o_pn = 0, o_fw = 0, o_rth = 0, o_dph = 0;
     constexpr bool kTable = !NH && short_forms<P>();
     const size_t o_ex = take(kTable ? (size_t)kExnerBins * L * sizeof(double2) : 0);
@@ -1669,6 +1675,9 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
     Side sw_(h, 0, st), sx_(h, 1, st);   // the wind's diagnostics, the advection
     const int place = dycore_tuning(h).wind_placement;
     const bool late = NH && (place == 2 || (place == 0 && wind_beside_solve(m.nC)));
+    // the edge PV with the wind's chain; else on its stream once the theta
+    // update is done, or (FP64 policy) on st after the join
+    const bool pv_with_wind = !pv_shares || (late && !short_forms<P>());
     for (int s3 = 0; s3 < 3; s3++) {
         const double h3 = dts[s3];
         auto wind = [&](cudaStream_t sw) {
@@ -1677,7 +1686,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
             GRIST_LAUNCH(h, PN("k_ke"), sw, (kev == 4   ? k_ke<P, kKeV>
                                              : kev == 2 ? k_ke<P, 2>
                                                         : k_ke<P, 1>)<<<gK, kBlock, 0, sw>>>(m, d, DK, u_in, K));
-            if (!short_forms<P>()) edge_pv(sw);
+            if (pv_with_wind) edge_pv(sw);
         };
         auto explicit_part = [&](cudaStream_t sw) {
             if (s3 == 0)
@@ -1705,6 +1714,10 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                                                    : thv == kPvH ? k_theta_update<P, kPvH>
                                                                  : k_theta_update<P, 1>)<<<gCT, kBlock, 0, st>>>(
             m, d, DTU, Fth, theta, Mv, S->dpi_theta, th_outs[s3], h3));
+        if (!pv_with_wind && !short_forms<P>()) {
+            sw_.fork();
+            edge_pv(sw_.s);
+        }
         if (NH) {
             sx_.join();
             if (late) {
@@ -1721,7 +1734,7 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                 m, d, ex, bkap, ps_outs[s3], th_outs[s3], p, alp, phl));
         }
         sw_.join();
-        if (short_forms<P>()) edge_pv(st);   // 2 F q_e: after the mass flux
+        if (short_forms<P>()) edge_pv(st);
         GRIST_LAUNCH(h, PN("k_momentum"), st, k_momentum<P, NH><<<gE, kBlock, 0, st>>>(
             m, d, DL, u_in, u, u_outs[s3], F, qv, Gq, K, Mv, rsum, p_outs[s3], alp, phl, dpp, h3, status));
         u_in = u_outs[s3];
