@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(kVertWarps * 32) k_tr_vertical(DevMesh m, Memb
     if (implicit) mib = __shfl_down_sync(kAllLanes, mi[0], 1);
     if (lane == 31) {
         meb = mib = (TC)0;
-        upb = 0;
+        upb = 1;   // no flux times its own last level: there is no next lane
     }
     TC rb[K];
 #pragma unroll
