@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "forms.cuh"
 #include "series.cuh"
 
 #define PN(n) (P::DF ? n "/mixdf" : (sizeof(TA) == 4 ? (sizeof(TM) == 8 ? n "/mixdbl" : n "/mix") : n "/fp64"))
@@ -370,14 +371,6 @@ __global__ void __launch_bounds__(kBlock) k_mass_col(DevMesh m, DyPar d, const t
     }
 }
 
-// f >= 0, for binary64 from the bits (an FP64 comparison holds the FP64 pipe
-// like an addition); -0 counts as 0, NaN by its sign.
-__device__ __forceinline__ bool runs_to_c2(float f) { return f >= 0.f; }
-__device__ __forceinline__ bool runs_to_c2(double f) {
-    const long long b = __double_as_longlong(f);
-    return b >= 0 || (b << 1) == 0;
-}
-
 // Eq. 4 horizontal flux: third-order upwind (beta = 1) edge value of theta
 // times the mass flux.  V = 4 (binary32): a thread takes four consecutive levels
 // of one edge as vectors, with one read of the upwind stencil row (4 vector
@@ -401,7 +394,7 @@ __global__ void __launch_bounds__(kBlock) k_theta_flux(DevMesh m, DyPar d, Level
     auto level = [&](int k) {
         const size_t x = (size_t)e * d.ld + k;
         const TA f = cv<TA>(F[x]);
-        const int side = runs_to_c2(f) ? 0 : 1;
+        const int side = nonneg(f) ? 0 : 1;
         TA te;
         if (m.d2w_ok) {
             // one weighted sum over the upwind side's stencil (the mean of
@@ -790,16 +783,6 @@ __global__ void __launch_bounds__(kBlock) k_pv_edge(DevMesh m, DyPar d, LevelDiv
         for (int t = 0; t < V; t++) a[t] = (TA)0.5 * (a[t] + b[t]);
     }
     stgv<V>(G + x, a);
-}
-
-// (double)a - (double)b of two binary32 numbers, bit for bit: where the binary32
-// difference is exact (its TwoSum error is zero) it is that number.
-__device__ __forceinline__ double wind_diff(double a, double b) { return sub_near(a, b); }
-__device__ __forceinline__ double wind_diff(float a, float b) {
-    const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
-    const float err = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
-    if (err == 0.f) return f2d(s);
-    return f2d(a) - f2d(b);
 }
 
 // Eq. 5 momentum tendency and stage update:

@@ -1,6 +1,7 @@
-// Comparisons, signs and ratios of binary64 (and their binary32 counterparts)
-// in integer arithmetic, shared by the kernels.  The file needs nothing but the
-// bit-cast and rounding intrinsics, so that it also compiles on the host.
+// Comparisons, signs, differences and ratios of binary64 (and their binary32
+// counterparts) kept off the FP64 pipe, shared by the kernels.  The file needs
+// f2d and sub_near (common.cuh) and the bit-cast and rounding intrinsics only, so
+// that it also compiles on the host.
 #pragma once
 
 namespace grist {
@@ -69,7 +70,7 @@ __device__ __forceinline__ double min_num(double a, double b) { return okey(b) <
 // a <= b (false for NaN), |a|
 __device__ __forceinline__ bool le_num(float a, float b) { return a <= b; }
 __device__ __forceinline__ bool le_num(double a, double b) {
-    const long long ka = okey(a), kb = okey(b);
+    const long long ka = okey(a), k = okey(b), kb = k == -1 ? 0 : k;   // -0 as 0
     return ka <= kb && kb <= kKeyInf && ka >= kKeyNegInf;
 }
 __device__ __forceinline__ float abs_num(float x) { return fabsf(x); }
@@ -107,6 +108,16 @@ __device__ __forceinline__ double fct_ratio(double Q, double P) {
     if (!nonzero(Q)) return Q;
     const double a = Q / P;
     return is_nan(a) ? 1.0 : a;
+}
+
+// (double)a - (double)b of two binary32 numbers, bit for bit: where the binary32
+// difference is exact (its TwoSum error is zero) it is that number.
+__device__ __forceinline__ double wind_diff(double a, double b) { return sub_near(a, b); }
+__device__ __forceinline__ double wind_diff(float a, float b) {
+    const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
+    const float err = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+    if (err == 0.f) return f2d(s);
+    return f2d(a) - f2d(b);
 }
 
 }  // namespace grist

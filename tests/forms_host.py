@@ -25,9 +25,16 @@ static int __double2loint(double x) { return (int)bits(x); }
 static double __hiloint2double(int h, int l) { return real(((uint64_t)(uint32_t)h << 32) | (uint32_t)l); }
 static long long __double_as_longlong(double x) { return (long long)bits(x); }
 static double __longlong_as_double(long long x) { return real((uint64_t)x); }
+static float __fsub_rn(float a, float b) { return a - b; }
+static float __fadd_rn(float a, float b) { return a + b; }
 // the same number, or both NaN
 static bool same(double a, double b) { return bits(a) == bits(b) || (std::isnan(a) && std::isnan(b)); }
 static bool same(float a, float b) { return bits(a) == bits(b) || (std::isnan(a) && std::isnan(b)); }
+"""
+# what forms.cuh takes from common.cuh, as plain operations
+PLAIN = """
+static double f2d(float f) { return (double)f; }
+static double sub_near(double a, double b) { return a - b; }
 """
 
 

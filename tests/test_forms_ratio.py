@@ -1,6 +1,6 @@
 """The limiter's ratio min(1, Q / P) (csrc/forms.cuh: fct_ratio) has the bits of
 the division for every operand, overflowing and subnormal ones included."""
-from forms_host import run
+from forms_host import PLAIN, run
 
 MAIN = r"""
 template <class T> T pick(std::mt19937_64 &r, int how) {
@@ -40,6 +40,6 @@ int main() {
 
 
 def test_ratio_has_the_bits_of_the_division(tmp_path):
-    bad32, bad64, n32, n64 = run(tmp_path, "forms.cuh", MAIN)
+    bad32, bad64, n32, n64 = run(tmp_path, "forms.cuh", MAIN, PLAIN)
     assert bad32 == 0 and bad64 == 0
     assert n32 > 1e6 and n64 > 1e6
