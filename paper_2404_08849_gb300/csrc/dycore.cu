@@ -1377,9 +1377,9 @@ template <bool EMU, bool DF, bool SHORT>
 cudaError_t launch_solve(const DevMesh &m, const DyPar &d, LevelDiv Dv, const double *wst, const double *phst,
                          const double *th, const double *rth, const double *dphi, const double *p_r, const double *ps,
                          double dts, double *w_out, double *phi_out, double *p, double *al, double *phl, double *dpp,
-                         const Binom &bp, const Binom &bn, int form, cudaStream_t st) {
+                         const Binom &bp, const Binom &bn, bool blocks, cudaStream_t st) {
     const unsigned grid = grid_for(m.nC, kSolveCols);
-    if (form == 2 || (form == 0 && solve_by_blocks(m.nC, d.L))) {
+    if (blocks) {
         const int bytes = 4 * d.L * kRow * 8;
         const cudaError_t e = cudaFuncSetAttribute(k_nh_solve_block<EMU, DF, SHORT>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1708,9 +1708,11 @@ int dycore_step(grist_mesh_s *h, grist_dycore_state *S, const grist_dycore_param
                 wind(sw_.s);
             }
             cudaError_t se = cudaSuccess;
-            GRIST_LAUNCH(h, PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, short_forms<P>()>(
+            const int form = dycore_tuning(h).column_solve;
+            const bool blocks = form == 2 || (form == 0 && solve_by_blocks(m.nC, L));
+            GRIST_LAUNCH(h, blocks ? PN("k_nh_solve_block") : PN("k_nh_solve"), st, se = (launch_solve<P::EMU, P::DF, short_forms<P>()>(
                 m, d, DL, wst, phst, th_outs[s3], rthn, dphn, p_n, ps_outs[s3], h3, w_outs[s3], phi_outs[s3], p_outs[s3],
-                alp, phl, dpp, bpos, bneg, dycore_tuning(h).column_solve, st)));
+                alp, phl, dpp, bpos, bneg, blocks, st)));
             if (se != cudaSuccess) return GRIST_ECUDA;
         } else {
             GRIST_LAUNCH(h, PN("k_hydro_diag"), st, k_hydro_diag<P::EMU, P::DF, short_forms<P>()><<<gW, kBlock, 0, st>>>(
