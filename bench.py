@@ -101,13 +101,15 @@ def algorithmic_bytes(name, nC, nE, nV, L, T, prec):
 # level-7 mesh (163,842 cells, 60 levels) of the same workload and step.
 # Units: cell-levels "c", edge-levels "e", vertex-levels "v", cell-interfaces
 # (L + 1 per column) "i".  Per-launch figures scale with the units processed.
-# Only kernels whose arithmetic is that of their capture are listed (the
-# column solve has since lost one subtraction a level, taken off here; the
-# momentum, kinetic-energy and explicit w/phi kernels moved FP64 work to the
-# integer units, and the tracer limiter passes issue none).
+# Only kernels whose arithmetic is that of their capture are listed
+# (profiles/vector_integer_forms_L7.md; k_nh_explicit: the mean of the three
+# stages; the tracer limiter passes issue none).
 FP64_WORK_MIX = {
     # kernel: (unit, FP64 flop per unit, DRAM bytes per unit)
-    "k_nh_solve": ("c", 62.70, 283.4),     # the one-warp form (large meshes)
+    "k_nh_solve": ("c", 62.70, 236.0),     # the one-warp form (large meshes)
+    "k_momentum": ("e", 14.93, 38.1),
+    "k_ke": ("c", 12.00, 18.3),
+    "k_nh_explicit": ("i", 11.41, 73.5),
     "k_eos": ("c", 93.0, 21.1),
     "k_tr_div": ("c", 12.00, 31.5),
 }

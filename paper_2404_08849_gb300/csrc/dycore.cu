@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kBlock) k_mass_edge(DevMesh m, DyPar d, const 
 // warp scan, theta = (dpi theta)/dpi of the stage input for Eq. 4.  In the
 // first stage of the NH core also the t^n state that the column solve's
 // equation of state is taken relative to: 1/(dpi theta) and dphi, or their
-// product (solve_short).
+// product (short_forms).
 //
 // The two 32-level chunks of a pair are loaded and scanned together (the scans
 // are independent until the carry is added), which hides half the shuffles'
@@ -549,9 +549,9 @@ __global__ void k_exner_table(DyPar d, int base, double2 *__restrict__ tab) {
 // Eq. 8 (hydrostatic diagnostics), one warp per column: mid-layer pressure,
 // alpha = Rd theta (p/p0)^kappa / p, geopotential integrated upward from
 // phi_s by a suffix scan, layer geopotential = mean of its interfaces.
-// Bound by the FP64 pipe: about 27 instructions a cell-level with the table
+// Bound by the FP64 pipe: 29 instructions a cell-level with the table
 // above (SHORT, see short_forms) against about 130 with pow(); level-6 mesh,
-// 30 levels: 323 -> 77 us a launch, plus 10 us a step for the table.
+// 30 levels: 323 -> 73 us a launch, plus 11 us a step for the table.
 // A warp takes two columns, so that the correctly rounded 1/dps runs one column
 // per lane.  Level 6, 30 levels, us a step by columns, 1, 2, 4: FP64 1833, 1807,
 // 1805; mixed 1551, 1518, 1557.  With pow(), p/p0 is the product with 1/p0
@@ -1234,7 +1234,8 @@ __global__ void __launch_bounds__(32, kSolveMinBlocks) k_nh_solve(DevMesh m, DyP
 //   C   lanes = columns, a warp per level: the new pressure;
 //   D   the block's threads over the flat (column, level) index, so the
 //       outputs are written as whole rows.
-// The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 43).
+// The FP64 pipe bounds both kernels, 44 instructions a cell-level (SHORT: 43; the
+// block form 46).
 // One warp for 32 columns needs about 20 blocks an SM to keep the pipe busy
 // (75 % then); with fewer columns than that the levels are the parallelism
 // left (solve_by_blocks has the figures).

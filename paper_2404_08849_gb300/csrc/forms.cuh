@@ -98,6 +98,9 @@ __device__ __forceinline__ void add_signed(double x, double &pp, double &pm) {
 // (1 where that gives NaN).  The division is reached only where a cell is
 // limited: Q >= P is 1, and 0 is 0 without the division's slow path, which
 // operands near TINY take (where a tracer is constant, Q = 0 and P = TINY).
+// k_tr_ratios, level 7, 4 tracers, 60 levels, us a launch: binary32 545 with the
+// division everywhere, 359 (335 with an approximate reciprocal and one
+// correction, which lost the results at overflow); binary64 2102.
 __device__ __forceinline__ float fct_ratio(float Q, float P) {
     if (!(Q < P)) return 1.f;
     return Q == 0.f ? Q : fminf(1.f, Q / P);

@@ -11,9 +11,9 @@
 // iterations.  The phases run either as one launch each or inside one
 // persistent cooperative kernel separated by bounded grid barriers.
 //
-// These kernels are bound by instruction issue and latency, not by the FP64
-// pipe, so they keep the hardware binary32/binary64 conversions (one issue
-// slot each) rather than the integer ones the FP64-bound dycore kernels use.
+// In binary32 these kernels are bound by instruction issue, the L1 data pipe and
+// latency, in binary64 by the FP64 pipe; conversions run in integers (cv), as
+// the hardware's issue on that pipe.
 //
 // Data layout: q [T][nC][ld], dpi [nC][ld], mass flux [nE][ld], edge
 // fluxes [T][nE][ld]; consecutive threads take consecutive levels of one
@@ -24,11 +24,11 @@
 // L1 data pipe (79 % of its wavefronts) and the latency of many small gathers
 // bounded the binary32 phases.  Level-7 mesh, 4 tracers, 60 levels, binary32,
 // us per launch, one level / vectors: div 231 / 145, edge 365 / 231, update
-// 226 / 140 (then at the DRAM rate), ratios 545 / 335 (half of it the
+// 226 / 148 (then at the DRAM rate), ratios 545 / 359 (half of it the
 // division's slow path, see fct_ratio), final 440 / 307, low-order 270 / 128
-// more in the first edge phase; the step 3261 / 2110 (1976 with the vertical
-// transport as it stands).  binary64 is bound by the FP64 pipe and gains little
-// from the width.
+// more in the first edge phase; the step 3261 / 1998 with the vertical transport
+// as it stands.  binary64 is bound by the FP64 pipe and gains little from the
+// width.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -504,20 +504,6 @@ __device__ __forceinline__ void item_edge_levels(const DevMesh &m, const MemberD
     }
 }
 
-// Cell-centric form of the edge flux (beta = 1, combined weights, every
-// stencil the upwind cell's ring {i, neighbours} in the order of the cell's
-// neighbour list): the thread of cell i gathers q over its ring and forms
-// the flux of each edge whose flux leaves the cell, so each edge-level is
-// written once, by its upwind cell, with the weights and the summation
-// order of the edge-centric form (bit-identical), from 7 gathers per
-// cell-level instead of 7 per edge-level.  The ring values of up to
-// ring_tracers() tracers are gathered first, so each drained edge's weights
-// are read once for them.  The drained edge-levels are kept as a mask (bit
-// 8 v + j: level v, edge j), and each thread walks its own drained edges: a
-// warp's cells drain different edges, so a walk over all six would spend 4.6
-// passes on the three that each thread has.  An edge whose V levels all
-// drain this cell is stored as one vector.  In the final stage of a limited
-// step (qn = q^n) the phase stores A = F^H - F^L, F^L = F q^n_i.
 // The low-order results of V levels at cell-level y of the tracer arrays: the
 // local bounds {max, min}(q^n, q^td) and div F^L.
 template <typename TC, int V>
@@ -539,6 +525,21 @@ __device__ __forceinline__ void store_lowres(const MemberDev &mb, size_t y, cons
 template <typename TC, int V, bool LOW> constexpr int ring_tracers() {
     return sizeof(TC) * V <= 8 || (LOW && sizeof(TC) == 4) ? 2 : 1;
 }
+// Cell-centric form of the edge flux (beta = 1, combined weights, every
+// stencil the upwind cell's ring {i, neighbours} in the order of the cell's
+// neighbour list): the thread of cell i gathers q over its ring and forms
+// the flux of each edge whose flux leaves the cell, so each edge-level is
+// written once, by its upwind cell, with the weights and the summation
+// order of the edge-centric form (bit-identical), from 7 gathers per
+// cell-level instead of 7 per edge-level.  The ring values of up to
+// ring_tracers() tracers are gathered first, so each drained edge's weights
+// are read once for them.  The drained edge-levels are kept as a mask (bit
+// 8 v + j: level v, edge j), and each thread walks its own drained edges: a
+// warp's cells drain different edges, so a walk over all six would spend 4.6
+// passes on the three that each thread has.  An edge whose V levels all
+// drain this cell is stored as one vector.  In the final stage of a limited
+// step (qn = q^n) the phase stores A = F^H - F^L, F^L = F q^n_i.
+//
 // LOW (the first stage of a limited step, q = q^n): the ring and the fluxes
 // are all that the low-order solution needs, so its phase (item_lowres, the
 // same operations) is done here, without gathering them again.
