@@ -223,6 +223,13 @@ __device__ __forceinline__ double rcp_nr(double x) {
     return fma(fma(e, e, e), y, y);
 }
 
+// PTX's binary32 reciprocal, within one ulp.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Conversions between binary32 and binary64 in integer arithmetic.  On this
 // GPU the hardware conversion instructions issue on the FP64 pipe, the
 // scarce resource of the mixed-precision kernels, so the IEEE-754 fields are

@@ -1,6 +1,6 @@
 // Comparisons, signs, differences and ratios of binary64 (and their binary32
 // counterparts) kept off the FP64 pipe, shared by the kernels.  The file needs
-// f2d and sub_near (common.cuh) and the bit-cast and rounding intrinsics only, so
+// f2d, sub_near and rcp_approx (common.cuh) and the bit-cast and rounding intrinsics only, so
 // that it also compiles on the host.
 #pragma once
 
@@ -94,18 +94,31 @@ __device__ __forceinline__ void add_signed(double x, double &pp, double &pm) {
     pm = neg ? pm : sum;
 }
 
-// min(1, Q / P) for P >= TINY > 0, the bits of the division for every operand
-// (1 where that gives NaN).  The division is reached only where a cell is
-// limited: Q >= P is 1, and 0 is 0 without the division's slow path, which
-// operands near TINY take (where a tracer is constant, Q = 0 and P = TINY).
-// k_tr_ratios, level 7, 4 tracers, 60 levels, us a launch: binary32 545 with the
-// division everywhere, 359 (335 with an approximate reciprocal and one
-// correction, which lost the results at overflow); binary64 2102.
+// min(1, Q / P) for P >= TINY > 0, the division's value (1 where that is NaN).
+// binary32: Markstein's division (IBM J. Res. Dev. 34, 1990).  From a reciprocal
+// within one ulp one Newton step gives the correctly rounded one, except where
+// all bits of P's significand are set (one in 2^23); the product with it,
+// corrected by its remainder, is the rounded quotient.  The scaling by a power of
+// two keeps every intermediate normal (left over: operands of 2^62 and more with a
+// quotient below 2^-100, to 2 ulp, or beyond -2^120, perhaps -infinity).  Where
+// that is NaN, by P = infinity (0) or a quotient beyond the range (infinite), the
+// plain product stands.  No branches, so that a
+// thread's eight ratios overlap: k_tr_ratios, level 7, 4 tracers, 60 levels, us a
+// launch 345; the division itself, which takes its slow path (a call) where P is
+// near TINY, that is wherever a tracer is constant, 545; the division behind
+// Q < P and Q != 0, 359.
 __device__ __forceinline__ float fct_ratio(float Q, float P) {
-    if (!(Q < P)) return 1.f;
-    return Q == 0.f ? Q : fminf(1.f, Q / P);
+    const float s = fmaxf(fabsf(Q), P) < 0x1p62f ? 0x1p64f : 0x1p-64f, p = P * s, q = Q * s;
+    float y = rcp_approx(p);
+    const float plain = q * y;
+    y = fmaf(fmaf(-p, y, 1.f), y, y);
+    float a = q * y;
+    a = fmaf(fmaf(-a, p, q), y, a);
+    a = a == a ? a : plain;
+    return fminf(1.f, a);
 }
-// binary64: decided on the keys.
+// binary64: the division, reached only where Q < P (decided on the keys) and not
+// for Q = 0; 2107 us there, 2813 with a refined reciprocal and one correction.
 __device__ __forceinline__ double fct_ratio(double Q, double P) {
     if (okey(Q) >= okey(P) || is_nan(Q) || is_nan(P)) return 1.0;
     if (!nonzero(Q)) return Q;

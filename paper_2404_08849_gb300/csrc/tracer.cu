@@ -24,9 +24,9 @@
 // L1 data pipe (79 % of its wavefronts) and the latency of many small gathers
 // bounded the binary32 phases.  Level-7 mesh, 4 tracers, 60 levels, binary32,
 // us per launch, one level / vectors: div 231 / 145, edge 365 / 231, update
-// 226 / 148 (then at the DRAM rate), ratios 545 / 359 (half of it the
+// 226 / 148 (then at the DRAM rate), ratios 545 / 345 (half of it the
 // division's slow path, see fct_ratio), final 440 / 307, low-order 270 / 128
-// more in the first edge phase; the step 3261 / 1998 with the vertical transport
+// more in the first edge phase; the step 3261 / 1982 with the vertical transport
 // as it stands.  binary64 is bound by the FP64 pipe and gains little from the
 // width.
 #include <algorithm>

@@ -35,6 +35,15 @@ static bool same(float a, float b) { return bits(a) == bits(b) || (std::isnan(a)
 PLAIN = """
 static double f2d(float f) { return (double)f; }
 static double sub_near(double a, double b) { return a - b; }
+// any reciprocal within one ulp
+static float rcp_approx(float x) {
+    static uint32_t n = 0;
+    const float y = 1 / x;
+    if (!std::isfinite(x) || x == 0) return y;
+    n = n * 1664525u + 1013904223u;
+    const float z = n >> 30 == 0 ? std::nextafter(y, -INFINITY) : n >> 30 == 1 ? std::nextafter(y, INFINITY) : y;
+    return std::fabs((double)z - 1.0 / x) <= std::fabs((double)std::nextafter(y, 2 * y) - y) ? z : y;
+}
 """
 
 

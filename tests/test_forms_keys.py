@@ -11,6 +11,7 @@ static int __clzll(long long x) { return x ? __builtin_clzll(x) : 64; }
 static int min(int a, int b) { return a < b ? a : b; }
 static long fell = 0, converted = 0;     // FP64 subtractions in sub_near, conversions in wind_diff
 static double f2d(float f) { converted++; return (double)f; }
+static float rcp_approx(float x) { return 1 / x; }
 """
 
 MAIN = r"""
