@@ -26,7 +26,7 @@
 // us per launch, one level / vectors: div 231 / 145, edge 365 / 231, update
 // 226 / 148 (then at the DRAM rate), ratios 545 / 345 (half of it the
 // division's slow path, see fct_ratio), final 440 / 307, low-order 270 / 128
-// more in the first edge phase; the step 3261 / 1982 with the vertical transport
+// more in the first edge phase; the step 3316 / 2001 with the vertical transport
 // as it stands.  binary64 is bound by the FP64 pipe and gains little from the
 // width.
 #include <algorithm>
